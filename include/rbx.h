@@ -45,7 +45,7 @@ typedef enum {
 } rbx_status;
 
 typedef enum {
-    RBX_FP32 = 0,      /* FP32 SIMT contractions */
+    RBX_FP32 = 0,      /* FP32-accurate contractions (three BF16 parts per operand, six products) */
     RBX_BF16 = 1,      /* BF16 tensor-core contractions, FP32 accumulation */
     RBX_BF16X3 = 2     /* split BF16 (hi + lo, three products), FP32 accumulation */
 } rbx_precision;
@@ -89,7 +89,7 @@ typedef struct {
                                RBX_K_SYNTH_FWD did it) */
 #define RBX_K_GEMM_BP 4     /* back-projection contraction with fused row-dot */
 #define RBX_K_FIELDS 5      /* smoothing + derivative fields */
-#define RBX_K_TABLES 6      /* direct Green's function (+ angular density array, FP32) */
+#define RBX_K_TABLES 6      /* direct Green's function */
 #define RBX_K_UPDATE 7      /* residual + update */
 
 /* Create a job bound to a CUDA stream (a cudaStream_t; NULL means the legacy default

@@ -1,0 +1,90 @@
+// Born weights of the forward (Eq. scattering-potential) and the reduction of its partial sums,
+// shared by every precision.
+#include "rbx_internal.cuh"
+
+namespace rbx {
+
+// Scattering potential Upsilon_m = omega c k~ (Eq. scattering-potential), with
+// k~ = omega/c + alpha0 omega^y (tan(pi y/2) + i) (Eq. szabo_dispersion_equation):
+// (omega^2 + omega c alpha tan(pi y/2), omega c alpha), alpha = alpha0 omega^y; omega^2 lossless.
+__device__ __forceinline__ double2 upsilon_m(double w, double c, double alpha, double tn)
+{
+    return make_double2(w * w + w * c * alpha * tn, w * c * alpha);
+}
+
+// v[x] = Upsilon_m dA (m - m_s) on the mask: Born weight of the rough part of the model.
+__global__ void k_born_rough(const float *__restrict__ c, const double *__restrict__ ns, const int *__restrict__ idx,
+                             int X, double w, double dA, const float *__restrict__ alpha0, double wy, double tn,
+                             float2 *__restrict__ v)
+{
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= X) return;
+    int k = idx[q];
+    double cc = c[k], n = ns[k];
+    double2 u = upsilon_m(w, cc, alpha0 ? wy * (double)alpha0[k] : 0.0, tn);
+    double d = dA * (1.0 / (cc * cc) - n * n);
+    v[q] = make_float2((float)(u.x * d), (float)(u.y * d));
+}
+
+__global__ void k_born_dm(const float *__restrict__ dm, const float *__restrict__ c, const int *__restrict__ idx, int X,
+                          double w, double dA, const float *__restrict__ alpha0, double wy, double tn,
+                          float2 *__restrict__ v)
+{
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= X) return;
+    int k = idx[q];
+    double2 u = alpha0 ? upsilon_m(w, (double)c[k], wy * (double)alpha0[k], tn) : make_double2(w * w, 0.0);
+    double d = dA * (double)dm[k];
+    v[q] = make_float2((float)(u.x * d), (float)(u.y * d));
+}
+
+static void lossy_factors(const Lossy &ab, double w, double &wy, double &tn)
+{
+    wy = tn = 0.0;
+    if (ab.alpha0) {
+        wy = pow(w, ab.y);
+        tn = tan(3.14159265358979323846 * ab.y / 2.0);
+    }
+}
+
+void launch_born_weights_rough(const float *c, const double *ns64, const int *idx, int X, double f, double dA,
+                               const Lossy &ab, float2 *v, cudaStream_t s)
+{
+    double w = 2.0 * 3.14159265358979323846 * f, wy, tn;
+    lossy_factors(ab, w, wy, tn);
+    k_born_rough<<<(X + 255) / 256, 256, 0, s>>>(c, ns64, idx, X, w, dA, ab.alpha0, wy, tn, v);
+}
+
+void launch_born_weights_dm(const float *dm, const float *c, const int *idx, int X, double f, double dA,
+                            const Lossy &ab, float2 *v, cudaStream_t s)
+{
+    double w = 2.0 * 3.14159265358979323846 * f, wy, tn;
+    lossy_factors(ab, w, wy, tn);
+    k_born_dm<<<(X + 255) / 256, 256, 0, s>>>(dm, c, idx, X, w, dA, ab.alpha0, wy, tn, v);
+}
+
+// D[e,r] = D[r,e] = sum over splits (fixed order) of the upper-triangle partials.
+__global__ void k_forward_reduce(const float2 *__restrict__ part, int N, int splits, float2 *__restrict__ D)
+{
+    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (i >= (size_t)N * N) return;
+    int e = (int)(i / N), r = (int)(i % N);
+    if (e > r) return;
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int q = 0; q < splits; q++) {
+        float2 p = part[(size_t)q * N * N + i];
+        acc.x += p.x;
+        acc.y += p.y;
+    }
+    D[(size_t)e * N + r] = acc;
+    D[(size_t)r * N + e] = acc;
+}
+
+void launch_forward_reduce(const float2 *part, int N, int splits, float2 *D, cudaStream_t s)
+{
+    size_t n = (size_t)N * N;
+    k_forward_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, N, splits, D);
+}
+
+}  // namespace rbx

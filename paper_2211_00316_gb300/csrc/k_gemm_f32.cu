@@ -1,0 +1,639 @@
+// Steps a6-a8 at FP32 accuracy on the tensor cores: Green's function synthesis and the two
+// complex contractions of an FP32 job (and the plain adjoint of every job).
+//
+//  forward (Eqs. perturb1, derivative):  D[e,r] = sum_x G_e[x] G_r[x] v[x]
+//  back-projection (Eq. sound_speed_update2), exact two-term factorisation:
+//     W_er = 2 (1 + s cos(gamma_e - gamma_r)) = 2 + s (kappa_e conj(kappa_r) + conj(kappa_e) kappa_r),
+//     kappa = e^{i gamma}, s = -1 (printed scattering angle) or +1 (isochron); since W and
+//     u_e u_r are symmetric in (e, r) the residual may be replaced by R_s = (R + R^T)/2, so
+//     grad[x] = 2 sum_e u_e P0[x,e] + 2 s sum_e kappa_e u_e P1[x,e],
+//     P0 = U^T R_s, P1 = (conj(kappa) U)^T R_s,
+//  i.e. a complex GEMM with the two stacks as rows and a fused row-dot epilogue.
+//
+// An FP32 operand is held as three BF16 parts, v = hi + mid + lo, which together carry its 24
+// bits exactly; the six products hi hi, hi mid, mid hi, mid mid, hi lo, lo hi leave out terms of
+// 2^-26 of the product. tcgen05 adds to its FP32 accumulators in tensor memory without rounding
+// to nearest, so a long sum there drifts; here a sum in tensor memory covers 32 terms of K (one
+// pipeline stage, the five small products before hi hi so that only four additions meet the
+// full-size sum) and is then added to FP32 registers, rounded to nearest, by the epilogue warps.
+// Two accumulator buffers alternate, so the MMAs do not wait for that. Sums over 16 terms gave
+// no smaller error (twice as many FP32 additions follow) and ran 7 % slower.
+#include "rbx_internal.cuh"
+#include "tc_sm100.cuh"
+
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+namespace rbx {
+using namespace tc;
+
+namespace {
+
+constexpr int BM = 128, BN = 128, BK = 32;
+constexpr int PARTS = 6;                                   // re hi, mid, lo, im hi, mid, lo
+constexpr uint32_t PLANE = BM * BK * 2;                    // 8 KB: one part of one operand tile
+constexpr uint32_t OPER = PARTS * PLANE;                   // 48 KB: an operand's tile, all parts
+constexpr int STAGES = 2;
+constexpr size_t G_SMEM = 1024 + (size_t)STAGES * 2 * OPER + 4352;
+constexpr int EPI = 256;                                   // epilogue threads (warps 2..9)
+constexpr int THREADS = 64 + EPI;
+
+__device__ __forceinline__ float phase_cycles_(float T, int K, float fhi, float flo)
+{
+    float p = fhi * T;
+    float err = fmaf(fhi, T, -p) + flo * T;
+    float r = (p - rintf(p)) + err;
+    return r + 0.125f - 0.25f * (float)K;
+}
+
+// Box of `planes` parts: with a 128-row box the K-major tile [part][row][32] (64-byte swizzle),
+// with a 32-row box the M-major half tile [part][k][64] (128-byte swizzle).
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, uint64_t *bar, int x, int y, int z)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(
+            dst),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+
+// K-major, 64-byte swizzle (rows of 32 BF16, 8-row groups 512 B apart).
+__device__ __forceinline__ uint64_t desc_k64(uint32_t saddr)
+{
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+}
+// M-major, 128-byte swizzle: 64 rows of M contiguous, the next 64 rows PARTS * 4 KB on, groups
+// of 8 K 1024 B apart.
+__device__ __forceinline__ uint64_t desc_m128(uint32_t saddr)
+{
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((OPER / 2) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// sin and cos of g in [-pi, pi] to about 1 ulp: sincospif of g / pi with the rounding of the
+// quotient carried as a first-order correction.
+__device__ __forceinline__ float2 unit_of(float g)
+{
+    const float IPI = 0.318309886183790672f, IPI_LO = 1.28412766e-8f, PI = 3.14159265358979f;
+    const float r = g * IPI, d = PI * (fmaf(g, IPI, -r) + g * IPI_LO);
+    float s, c;
+    sincospif(r, &s, &c);
+    return make_float2(fmaf(-s, d, c), fmaf(c, d, s));
+}
+
+struct GemmArgs {
+    CUtensorMap a, b;
+    int N, ntile, nk, kper;         // forward: tile rows, K chunks, chunks per split
+    float2 *part;                   // forward: [split][N][N] partial D
+    const TabEntry *tab;            // back-projection: directions of stack 1
+    const __nv_bfloat16 *planes;    // back-projection: parts of the weights, [plane][N][xld]
+    size_t pstride;
+    int xld, X, x0, nx;             // back-projection: row length, nodes in all, first node and count of the slab
+    float2 *bpart;                  // back-projection: [stack][e tile][X] partial row-dots
+    unsigned *err;
+};
+
+// BP false: the forward's upper tile pair (te, tr) over the K chunks of one split.
+// BP true: for 128 nodes, 128 emitters and one stack, P = A^T R_s over all receivers and the
+// row-dot with the weights. CONJ: the plain adjoint, A = W = conj(G).
+//
+// Bound: shared-memory bandwidth of the tensor cores. A 128 x 128 x 16 MMA reads 8 KB in the 64
+// clocks it takes at the peak rate (128 B per clock, all an SM has), the tile loads write 31 B
+// per clock besides, so 0.7-0.8 of the BF16 peak over the six products is what the form allows.
+// K chunks of 32 because a 64-term stage of both operands' parts (192 KB) leaves no second one.
+// Against FP32 multiply-adds on the CUDA cores (64 x 64 tiles, 0.5 of their peak), ncu: 256
+// transducers, 48,120 nodes: forward 437 -> 89 us, back-projection 1297 -> 321 us; 768
+// transducers, 19,760 nodes: plain adjoint 2915 -> 384 us. Error against 64 bits no larger at any
+// size from 48 transducers on (N = 1024, 20,000 nodes: forward 6.0e-7 -> 2.2e-7, plain adjoint
+// 6.1e-7 -> 1.7e-7).
+template <bool BP, bool CONJ>
+__global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant__ GemmArgs g)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t *full = reinterpret_cast<uint64_t *>(tiles + (size_t)STAGES * 2 * OPER);
+    uint64_t *empty = full + STAGES;
+    uint64_t *accf = empty + STAGES;       // [2] accumulator buffer ready to drain
+    uint64_t *acce = accf + 2;             // [2] accumulator buffer drained
+    float2 *quarter_sum = reinterpret_cast<float2 *>(acce + 2);   // [4][128]
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(quarter_sum + 4 * BM);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int N = g.N;
+
+    int ta, tb, c0 = 0, nc;                // tile of A (rows of D), tile of B (columns), K chunks
+    if (BP) {
+        tb = blockIdx.x;
+        ta = blockIdx.y;
+        nc = g.nk;
+    } else {
+        int b = blockIdx.x, te = 0;
+        while (b >= g.ntile - te) { b -= g.ntile - te; te++; }
+        ta = te;
+        tb = te + b;
+        c0 = blockIdx.y * g.kper;
+        nc = min(g.nk, c0 + g.kper) - c0;
+    }
+    const int stack = BP ? blockIdx.z : 0;
+    const int ncol = min(BN, (N - tb * BN + 15) & ~15);   // columns of the MMAs (a ragged last tile)
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; s++) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
+        for (int q = 0; q < 2; q++) { mbar_init(accf + q, 1); mbar_init(acce + q, EPI); }
+        fence_mbar_init();
+    }
+    if (warp == 1) tmem_alloc(tslot, 512);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tslot;
+
+    if (warp == 0 && lane == 0) {
+        prefetch_tmap(&g.a);
+        if (BP) prefetch_tmap(&g.b);
+        int issued = 0;
+        for (int c = 0; c < nc; c++) {
+            const int s = c % STAGES;
+            if (c >= STAGES && !mbar_wait(empty + s, ((c / STAGES) - 1) & 1)) { atomicOr(g.err, 1u); break; }
+            mbar_arrive_expect_tx(full + s, 2 * OPER);
+            const uint32_t base = smem_u32(tiles + (size_t)s * 2 * OPER);
+            const int k = (c0 + c) * BK;
+            if (BP) {
+                tma_load_3d(base, &g.a, full + s, ta * BM, k, PARTS * stack);
+                tma_load_3d(base + OPER / 2, &g.a, full + s, ta * BM + 64, k, PARTS * stack);
+                tma_load_3d(base + OPER, &g.b, full + s, k, tb * BN, 0);
+            } else {
+                tma_load_3d(base, &g.a, full + s, k, ta * BM, 0);
+                tma_load_3d(base + OPER, &g.a, full + s, k, tb * BN, PARTS);
+            }
+            issued++;
+        }
+        // no copy may still be in flight when the CTA retires
+        for (int c = (issued > STAGES ? issued - STAGES : 0); c < issued; c++)
+            if (!mbar_wait(full + (c % STAGES), (c / STAGES) & 1)) atomicOr(g.err, 4u);
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t mn = BP ? (1u << 15) : 0u;      // A is M-major
+            const uint32_t ip = idesc_bf16(BM, ncol, 0) | mn, in = idesc_bf16(BM, ncol, 1) | mn;
+            const uint32_t i_re = CONJ ? ip : in, i_im = CONJ ? in : ip;   // signs of A_im B_im and A_im B_re
+            bool ok = true;
+            for (int c = 0; c < nc && ok; c++) {
+                const int buf = c & 1, s = c % STAGES;
+                if (c >= 2 && !mbar_wait(acce + buf, ((c >> 1) - 1) & 1)) { atomicOr(g.err, 32u); ok = false; break; }
+                if (!mbar_wait(full + s, (c / STAGES) & 1)) { atomicOr(g.err, 2u); ok = false; break; }
+                fence_after();
+                const uint32_t dre = tmem + buf * 2 * BN, dim = dre + BN;
+                const uint32_t a = smem_u32(tiles + (size_t)s * 2 * OPER), b = a + OPER;
+                constexpr uint32_t APART = BP ? PLANE / 2 : PLANE, AK = BP ? 2048 : 32;
+#pragma unroll
+                for (int p = 0; p < 6; p++) {
+                    // (hi, lo), (lo, hi), (mid, mid), (hi, mid), (mid, hi), (hi, hi)
+                    constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};
+#pragma unroll
+                    for (int k = 0; k < BK / 16; k++) {
+                        const uint32_t ar = a + PA[p] * APART + k * AK, br = b + PB[p] * PLANE + k * 32;
+                        const uint64_t a0 = BP ? desc_m128(ar) : desc_k64(ar);
+                        const uint64_t a1 = BP ? desc_m128(ar + 3 * APART) : desc_k64(ar + 3 * APART);
+                        const uint64_t b0 = desc_k64(br), b1 = desc_k64(br + 3 * PLANE);
+                        const uint32_t acc = (p > 0 || k > 0) ? 1u : 0u;
+                        mma_bf16(dre, a0, b0, ip, acc);
+                        mma_bf16(dre, a1, b1, i_re, 1u);
+                        mma_bf16(dim, a0, b1, ip, acc);
+                        mma_bf16(dim, a1, b0, i_im, 1u);
+                    }
+                }
+                mma_commit(empty + s);
+                mma_commit(accf + buf);
+            }
+            // every MMA of this CTA has completed once the last buffer is signalled
+            if (ok && !mbar_wait(accf + ((nc - 1) & 1), ((nc - 1) >> 1) & 1)) atomicOr(g.err, 8u);
+        }
+        __syncwarp();
+    } else if (warp >= 2) {
+        // warp w reads TMEM lanes 32 (w mod 4) .. + 31; warps 2-5 columns 0-63, warps 6-9 the rest
+        const int sub = warp & 3, row = sub * 32 + lane, half = (warp - 2) >> 2;
+        const uint32_t at = tmem + ((uint32_t)(sub * 32) << 16) + half * 64;
+        float re[64], im[64];
+#pragma unroll
+        for (int i = 0; i < 64; i++) re[i] = im[i] = 0.f;
+        bool ok = true;
+        for (int c = 0; c < nc; c++) {
+            const int buf = c & 1;
+            ok = __all_sync(0xffffffffu, mbar_wait(accf + buf, (c >> 1) & 1));
+            if (!ok) {
+                if (lane == 0) atomicOr(g.err, 16u);
+                break;
+            }
+            fence_after();
+            if (half * 64 < ncol) {
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    float t[32];
+                    tmem_ld32(at + buf * 2 * BN + (q >> 1) * BN + (q & 1) * 32, t);
+                    float *d = (q < 2 ? re : im) + (q & 1) * 32;
+#pragma unroll
+                    for (int i = 0; i < 32; i++) d[i] += t[i];
+                }
+            }
+            fence_before();
+            mbar_arrive(acce + buf);
+        }
+        if (!BP) {
+            const int e = ta * BM + row;
+            float2 *P = g.part + ((size_t)blockIdx.y * N + e) * N;
+            if (e < N) {
+#pragma unroll
+                for (int i = 0; i < 64; i++) {
+                    const int r = tb * BN + half * 64 + i;
+                    if (r < N) P[r] = make_float2(re[i], im[i]);
+                }
+            }
+        } else {
+            // P through shared memory (the stages are free: every MMA has read them), column i of
+            // 128 rows at P[i]; then each thread takes two neighbouring nodes and 32 emitters
+            float2 *P = reinterpret_cast<float2 *>(tiles);
+#pragma unroll
+            for (int i = 0; i < 64; i++) P[(half * 64 + i) * BM + row] = make_float2(re[i], im[i]);
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // the epilogue warps
+            const int t = threadIdx.x - 64, r2 = 2 * (t & 63), quarter = t >> 6;
+            const int xl = ta * BM + r2, e0 = tb * BN + quarter * 32, ne = min(32, N - e0);
+            // eight partial sums, of every eighth emitter
+            float2 s[2][8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) s[0][k] = s[1][k] = make_float2(0.f, 0.f);
+            if (ok && xl < g.nx && ne > 0) {
+                const bool two = xl + 1 < g.nx;
+                const __nv_bfloat16 *w = g.planes + (size_t)e0 * g.xld + xl;
+                const TabEntry *tab = g.tab + (size_t)e0 * g.X + g.x0 + xl;
+                // eight rows at a time, all their loads first: the weights come from L2 or HBM,
+                // and a chain of single rows waits for each
+#pragma unroll 1
+                for (int i0 = 0; i0 < ne; i0 += 8) {
+                    __nv_bfloat162 q[8][6];
+                    float gam[8][2];
+#pragma unroll
+                    for (int k = 0; k < 8; k++) {
+                        const int i = min(i0 + k, ne - 1);
+#pragma unroll
+                        for (int m = 0; m < 6; m++)
+                            q[k][m] = *reinterpret_cast<const __nv_bfloat162 *>(w + (size_t)i * g.xld + m * g.pstride);
+                        if (!CONJ && stack == 1) {
+                            // an uncovered entry's weight is zero and its direction not a number
+                            const uint4 v0 = __ldg(reinterpret_cast<const uint4 *>(tab + (size_t)i * g.X));
+                            const uint4 v1 = __ldg(reinterpret_cast<const uint4 *>(tab + (size_t)i * g.X + (two ? 1 : 0)));
+                            gam[k][0] = v0.x == kUncovered ? 0.f : __uint_as_float(v0.w);
+                            gam[k][1] = v1.x == kUncovered ? 0.f : __uint_as_float(v1.w);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; k++) {
+                        const bool in = i0 + k < ne;
+                        const float4 p = *reinterpret_cast<const float4 *>(P + (quarter * 32 + i0 + k) * BM + r2);
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            float v[6];   // the parts add up to the FP32 weight exactly
+#pragma unroll
+                            for (int m = 0; m < 6; m++) v[m] = h ? __high2float(q[k][m]) : __low2float(q[k][m]);
+                            float wr = v[0] + v[1] + v[2], wi = v[3] + v[4] + v[5];
+                            if (CONJ) wi = -wi;
+                            if (!CONJ && stack == 1) {
+                                const float2 kap = unit_of(gam[k][h]);
+                                const float ur = wr;
+                                wr = kap.x * ur - kap.y * wi;
+                                wi = kap.x * wi + kap.y * ur;
+                            }
+                            const float pr = h ? p.z : p.x, pi = h ? p.w : p.y;
+                            if (in) {
+                                s[h][k].x = fmaf(wr, pr, s[h][k].x);
+                                s[h][k].x = fmaf(-wi, pi, s[h][k].x);
+                                s[h][k].y = fmaf(wr, pi, s[h][k].y);
+                                s[h][k].y = fmaf(wi, pr, s[h][k].y);
+                            }
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+#pragma unroll
+                for (int d = 4; d > 0; d >>= 1)
+#pragma unroll
+                    for (int k = 0; k < d; k++) {
+                        s[h][k].x += s[h][k + d].x;
+                        s[h][k].y += s[h][k + d].y;
+                    }
+                quarter_sum[quarter * BM + r2 + h] = s[h][0];
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            const int xo = ta * BM + t;
+            if (t < BM && xo < g.nx) {
+                const float2 a = quarter_sum[t], b = quarter_sum[BM + t], c = quarter_sum[2 * BM + t],
+                             d = quarter_sum[3 * BM + t];
+                g.bpart[((size_t)stack * gridDim.x + tb) * g.X + g.x0 + xo] =
+                    make_float2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
+// v = hi + mid + lo, each BF16
+__device__ __forceinline__ void split3(float v, __nv_bfloat16 *q)
+{
+    q[0] = __float2bfloat16_rn(v);
+    v -= __bfloat162float(q[0]);
+    q[1] = __float2bfloat16_rn(v);
+    v -= __bfloat162float(q[1]);
+    q[2] = __float2bfloat16_rn(v);
+}
+
+// The six parts of two neighbouring complex values to [plane][N][xld]
+__device__ __forceinline__ void put_parts(__nv_bfloat16 *planes, size_t pstride, size_t at, const float2 *z)
+{
+    __nv_bfloat16 a[6], b[6];
+    split3(z[0].x, a);
+    split3(z[0].y, a + 3);
+    split3(z[1].x, b);
+    split3(z[1].y, b + 3);
+#pragma unroll
+    for (int k = 0; k < 6; k++)
+        *reinterpret_cast<__nv_bfloat162 *>(planes + k * pstride + at) = __halves2bfloat162(a[k], b[k]);
+}
+
+// Operands of the contractions from the tables, two nodes and `walk` transducers per thread, as
+// parts in [plane][N][xld] for the slab of nx nodes from x0 on.
+//  KIND 0: planes 0-5 G_e[x] = (8 pi omega/c0)^(-1/2) a exp(i 2 pi (f T - K/4 + 1/8)) (Eq. 2D_greens)
+//  KIND 1: planes 0-5 G, planes 6-11 G v (the forward)
+//  KIND 2: planes 0-5 u_e[x] = dgamma / ((8 pi omega/c0)^(-1/2) a) exp(-i 2 pi (...)) (Eq.
+//          greens-time-reversed), planes 6-11 conj(kappa) u. The angular density dgamma (step a4)
+//          comes from the direction angles of the neighbouring transducers, kept in registers as
+//          the thread walks its transducers: the tables are read 1 + 2 / walk times and no
+//          array of dgamma is written or read.
+// Bound: HBM. Per entry 16 B are read and 24 B (12 B for KIND 0) written.
+template <int KIND>
+__global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict__ tab, const float2 *__restrict__ v, int N,
+                                                     int X, int x0, int nx, int xld, size_t pstride, float fhi, float flo,
+                                                     float C, __nv_bfloat16 *__restrict__ planes, int walk)
+{
+    const int xl = 2 * (blockIdx.x * blockDim.x + threadIdx.x), e0 = blockIdx.y * walk;
+    if (xl >= nx) return;
+    const bool two = xl + 1 < nx;
+    const TabEntry *t = tab + x0 + xl;
+    TabEntry none;
+    none.idk = kUncovered;
+    none.T = none.a = none.gam = 0.f;
+    TabEntry prev[2], cur[2], next[2];
+    auto row = [&](int e, TabEntry *o) {
+        o[0] = t[(size_t)e * X];
+        o[1] = two ? t[(size_t)e * X + 1] : none;
+    };
+    if (KIND == 2) row((e0 + N - 1) % N, prev);
+    row(e0, cur);
+    float2 w[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    if (KIND == 1) {
+        w[0] = v[x0 + xl];
+        if (two) w[1] = v[x0 + xl + 1];
+    }
+    const int e1 = min(N, e0 + walk);
+    for (int e = e0; e < e1; e++) {
+        if (KIND == 2 || e + 1 < e1) row((e + 1) % N, next);
+        float2 z[2], z2[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            z[q] = z2[q] = make_float2(0.f, 0.f);
+            if (cur[q].idk == kUncovered) continue;
+            float s, c;
+            sincospif(2.f * phase_cycles_(cur[q].T, (int)(cur[q].idk & 0xffu), fhi, flo), &s, &c);
+            if (KIND == 2) {
+                const float dg = (next[q].idk == kUncovered || prev[q].idk == kUncovered)
+                                     ? 0.f : dgamma_of(next[q].gam, prev[q].gam);
+                const float A = dg / (C * cur[q].a);
+                z[q] = make_float2(A * c, -A * s);
+                const float2 k = unit_of(cur[q].gam);
+                z2[q] = make_float2(k.x * z[q].x + k.y * z[q].y, k.x * z[q].y - k.y * z[q].x);
+            } else {
+                const float A = C * cur[q].a;
+                z[q] = make_float2(A * c, A * s);
+                if (KIND == 1)
+                    z2[q] = make_float2(z[q].x * w[q].x - z[q].y * w[q].y, z[q].x * w[q].y + z[q].y * w[q].x);
+            }
+        }
+        const size_t at = (size_t)e * xld + xl;
+        put_parts(planes, pstride, at, z);
+        if (KIND != 0) put_parts(planes + 6 * pstride, pstride, at, z2);
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            prev[q] = cur[q];
+            cur[q] = next[q];
+        }
+    }
+}
+
+// R_s (complex N x N) -> parts [6][N][rld]
+__global__ void k_rs_parts(const float2 *__restrict__ Rs, int N, int rld, __nv_bfloat16 *__restrict__ planes)
+{
+    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (i >= (size_t)N * N) return;
+    const size_t o = (i / N) * rld + i % N, P = (size_t)N * rld;
+    __nv_bfloat16 q[6];
+    const float2 v = Rs[i];
+    split3(v.x, q);
+    split3(v.y, q + 3);
+#pragma unroll
+    for (int k = 0; k < 6; k++) planes[k * P + o] = q[k];
+}
+
+// gpart[stack][x] = sum over emitter tiles, in order
+__global__ void k_bp_sum(const float2 *__restrict__ bpart, int ET, int X, float2 *__restrict__ gpart)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= X) return;
+    float2 s = make_float2(0.f, 0.f);
+    for (int t = 0; t < ET; t++) {
+        const float2 p = bpart[((size_t)blockIdx.y * ET + t) * X + x];
+        s.x += p.x;
+        s.y += p.y;
+    }
+    gpart[(size_t)blockIdx.y * X + x] = s;
+}
+
+void fsplit(double f, float &fhi, float &flo)
+{
+    fhi = (float)f;
+    flo = (float)(f - (double)fhi);
+}
+
+float green_const(double f, double c0)
+{
+    return (float)(1.0 / sqrt(8.0 * 3.14159265358979323846 * (2.0 * 3.14159265358979323846 * f) / c0));
+}
+
+// BF16 planes [planes][rows][cols], rows ld elements apart, read in boxes of `inner` columns,
+// `outer` rows and six planes
+bool make_map(CUtensorMap *m, void *base, size_t cols, size_t rows, size_t planes, size_t ld, unsigned inner,
+              unsigned outer)
+{
+    cuuint64_t dims[3] = {cols, rows, planes};
+    cuuint64_t strides[2] = {ld * 2, ld * rows * 2};
+    cuuint32_t box[3] = {inner, outer, PARTS}, estr[3] = {1, 1, 1};
+    return encode_tiled(m, base, 3, dims, strides, box, estr,
+                        inner * 2 == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+}
+
+template <int KIND>
+void synth(const F32Planes &p, const TabEntry *tab, const float2 *v, int x0, int nx, double f, double c0, cudaStream_t s)
+{
+    float fhi, flo;
+    fsplit(f, fhi, flo);
+    // a walk of 8 once that still gives every SM a full set of blocks; short ones on small
+    // problems, which a long walk leaves waiting on its chain of loads
+    const unsigned bx = (unsigned)((nx + 255) / 256);
+    const int walk = (size_t)bx * ((p.N + 7) / 8) >= 152 * 16 ? 8 : 2;
+    k_synth_parts<KIND><<<dim3(bx, (unsigned)((p.N + walk - 1) / walk)), 128, 0, s>>>(
+        tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo, green_const(f, c0), static_cast<__nv_bfloat16 *>(p.planes),
+        walk);
+}
+
+}  // namespace
+
+// Splits of the forward's K loop: the tile pairs fill the GPU once, at most 64 partials (the
+// bound of the job's memory estimate) and no split below three K chunks (the start of a CTA
+// and its drain cost about as much).
+int forward_splits(int N, int X)
+{
+    const int T = (N + BM - 1) / BM, pairs = T * (T + 1) / 2, nk = (X + BK - 1) / BK;
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int s = std::max(1, sms / pairs);
+    s = std::min(s, std::min(64, (nk + 2) / 3));
+    const int kper = (nk + s - 1) / s;
+    return (nk + kper - 1) / kper;
+}
+
+bool f32_setup(F32Planes &p, int N, int X, bool full, cudaStream_t st)
+{
+    p.N = N;
+    p.X = X;
+    p.full = full;
+    const int x8 = (X + 7) / 8 * 8;
+    // all nodes' forward or back-projection operands (24 B an entry), or on a tensor-core job,
+    // whose plain adjoint alone comes here, 8 B an entry and the nodes in slabs
+    p.xs = full ? x8 : std::max(std::min(x8, 64), X * 2 / 3 / 8 * 8);
+    p.xld = p.xs;
+    p.pstride = (size_t)N * p.xld;
+    p.rld = (N + 7) / 8 * 8;
+    const size_t bytes = (full ? 12 : 6) * p.pstride * sizeof(__nv_bfloat16);
+    const size_t ET = (N + BN - 1) / BN;
+    if (cudaMallocAsync(&p.planes, bytes, st) != cudaSuccess) return false;
+    if (cudaMallocAsync(&p.rs, PARTS * (size_t)N * p.rld * sizeof(__nv_bfloat16), st) != cudaSuccess) return false;
+    if (ET > 1 &&   // with one emitter tile the partial row-dots are the result
+        cudaMallocAsync(reinterpret_cast<void **>(&p.bpart), (full ? 2 : 1) * ET * X * sizeof(float2), st) != cudaSuccess)
+        return false;
+    if (cudaMallocAsync(reinterpret_cast<void **>(&p.err), sizeof(unsigned), st) != cudaSuccess) return false;
+    cudaMemsetAsync(p.err, 0, sizeof(unsigned), st);
+    const size_t cols = std::min(p.xs, X), planes = full ? 12 : 6;
+    return make_map(&p.fmap, p.planes, cols, N, planes, p.xld, BK, BM) &&
+           make_map(&p.amap, p.planes, cols, N, planes, p.xld, 64, BK) &&
+           make_map(&p.rmap, p.rs, N, N, PARTS, p.rld, BK, BN) &&
+           cudaFuncSetAttribute(k_cgemm_f32<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(k_cgemm_f32<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(k_cgemm_f32<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
+               cudaSuccess;
+}
+
+void f32_free(F32Planes &p, cudaStream_t st)
+{
+    void *ps[] = {p.planes, p.rs, p.bpart, p.err};
+    for (void *q : ps)
+        if (q) cudaFreeAsync(q, st);
+    p = F32Planes{};
+}
+
+void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
+{
+    synth<1>(p, tab, v, 0, p.X, f, c0, s);
+}
+
+void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s)
+{
+    synth<2>(p, tab, nullptr, 0, p.X, f, c0, s);
+}
+
+void launch_forward_f32(F32Planes &p, int splits, float2 *part, cudaStream_t s)
+{
+    const int T = (p.N + BM - 1) / BM, nk = (p.X + BK - 1) / BK;
+    GemmArgs g{};
+    g.a = g.b = p.fmap;
+    g.N = p.N;
+    g.ntile = T;
+    g.nk = nk;
+    g.kper = (nk + splits - 1) / splits;
+    g.part = part;
+    g.err = p.err;
+    k_cgemm_f32<false, false><<<dim3(T * (T + 1) / 2, splits), THREADS, G_SMEM, s>>>(g);
+}
+
+static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
+{
+    GemmArgs g{};
+    g.a = p.amap;
+    g.b = p.rmap;
+    g.N = p.N;
+    g.nk = (p.N + BK - 1) / BK;
+    g.tab = tab;
+    g.planes = static_cast<const __nv_bfloat16 *>(p.planes);
+    g.pstride = p.pstride;
+    g.xld = p.xld;
+    g.X = p.X;
+    g.bpart = p.bpart ? p.bpart : gpart;
+    g.err = p.err;
+    return g;
+}
+
+static void rs_parts(F32Planes &p, const float2 *Rs, cudaStream_t s)
+{
+    const size_t nn = (size_t)p.N * p.N;
+    k_rs_parts<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
+}
+
+// The preconditioned back-projection from the operands of launch_synth_bp: gpart[2][X].
+int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, float2 *gpart, cudaStream_t s)
+{
+    const int ET = (p.N + BN - 1) / BN;
+    rs_parts(p, Rs, s);
+    GemmArgs g = bp_args(p, tab, gpart);
+    g.nx = p.X;
+    k_cgemm_f32<true, false><<<dim3(ET, (p.X + BM - 1) / BM, 2), THREADS, G_SMEM, s>>>(g);
+    if (ET == 1) return 2;
+    k_bp_sum<<<dim3((p.X + 255) / 256, 2), 256, 0, s>>>(p.bpart, ET, p.X, gpart);
+    return 3;
+}
+
+// The plain adjoint's sum_{e,r} conj(G_e G_r) R_s: synthesis and contraction, slab by slab.
+int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, double f, double c0, float2 *gpart,
+                       cudaStream_t s)
+{
+    const int ET = (p.N + BN - 1) / BN;
+    int n = 1;
+    rs_parts(p, Rs, s);
+    for (int x0 = 0; x0 < p.X; x0 += p.xs, n += 2) {
+        GemmArgs g = bp_args(p, tab, gpart);
+        g.x0 = x0;
+        g.nx = std::min(p.xs, p.X - x0);
+        synth<0>(p, tab, nullptr, x0, g.nx, f, c0, s);
+        k_cgemm_f32<true, true><<<dim3(ET, (g.nx + BM - 1) / BM, 1), THREADS, G_SMEM, s>>>(g);
+    }
+    if (ET == 1) return n;
+    k_bp_sum<<<dim3((p.X + 255) / 256, 1), 256, 0, s>>>(p.bpart, ET, p.X, gpart);
+    return n + 1;
+}
+
+}  // namespace rbx

@@ -122,6 +122,16 @@ __global__ __launch_bounds__(256) void k_forward_tables_noalloc(const float *__r
         }
 }
 
+// About 2048 blocks, each of at least 256 nodes.
+int noalloc_splits(int N, int X)
+{
+    const int T = (N + TM - 1) / TM, pairs = T * (T + 1) / 2;
+    int s = (2048 + pairs - 1) / pairs;
+    const int smax = (X + 255) / 256;
+    if (s > smax) s = smax;
+    return s > 64 ? 64 : s;
+}
+
 std::mutex g_scratch_mu;
 float2 *g_scratch_ptr[64] = {};
 
@@ -174,7 +184,7 @@ extern "C" rbx_status rbx_forward_noalloc(const float *T_dev, const float *a_dev
         }
         scratch = g_scratch_ptr[dev];
     }
-    int splits = forward_splits(N, X);
+    int splits = noalloc_splits(N, X);
     int cap = (int)(kScratchElems / ((size_t)N * N));
     if (splits > cap) splits = cap;
     int Tn = (N + TM - 1) / TM, pairs = Tn * (Tn + 1) / 2;

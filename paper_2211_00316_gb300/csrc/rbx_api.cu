@@ -97,12 +97,12 @@ static cudaError_t dalloc(T *&p, size_t n, cudaStream_t s)
 
 static void free_ws(Workspace &w, cudaStream_t s)
 {
-    void *ps[] = {w.hist, w.node2x, w.idx, w.rows, w.c, w.ns, w.tmp, w.fields, w.ns64, w.tmp64, w.tab, w.dg, w.exits, w.G, w.U,
-                  w.kap, w.v, w.gdir, w.D, w.R, w.Rs, w.part, w.gpart, w.data, w.red, w.counters, w.alpha0, w.as64,
+    void *ps[] = {w.hist, w.node2x, w.idx, w.rows, w.c, w.ns, w.tmp, w.fields, w.ns64, w.tmp64, w.tab, w.dg, w.exits, w.v, w.gdir, w.D, w.R, w.Rs, w.part, w.gpart, w.data, w.red, w.counters, w.alpha0, w.as64,
                   w.dmacc, w.linked, w.beta};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, s);
     tc_free(w.tc, s);
+    f32_free(w.f32, s);
     w = Workspace{};
 }
 
@@ -269,10 +269,11 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.tab, NX);
     ALLOC(w.dg, NX);
     ALLOC(w.exits, N * (N - 1));
-    ALLOC(w.G, NX);
-    if (g.precision == RBX_FP32) {   // FP32 back-projection operands (the tensor-core path has its own)
-        ALLOC(w.U, NX);
-        ALLOC(w.kap, NX);
+    // FP32 jobs: the operands of both contractions; the others: those of the plain adjoint
+    if (!f32_setup(w.f32, w.N, X, g.precision == RBX_FP32, j->stream)) {
+        cudaGetLastError();
+        free_ws(w, j->stream);
+        return fail(j, RBX_ENOMEM, "FP32 operand set-up failed (allocation or TMA descriptor)");
     }
     ALLOC(w.v, X);
     ALLOC(w.gdir, N * N);
@@ -443,9 +444,8 @@ static rbx_status direct_green(rbx_job *j, double f, float2 *out)
     return RBX_OK;
 }
 
-// The angular density array w.dg (step a4), formed when first needed after the tables changed:
-// the FP32 back-projection and rbx_get_tables read it; the tensor-core operand synthesis forms
-// the same values from the tables itself.
+// The angular density array w.dg (step a4), formed when rbx_get_tables first asks for it after
+// the tables changed; the operand syntheses form the same values from the tables themselves.
 static rbx_status ensure_dgamma(rbx_job *j)
 {
     if (j->dg_valid) return RBX_OK;
@@ -487,7 +487,6 @@ static rbx_status trace_end(rbx_job *j)
     rbx_status st;
     j->linked_valid = j->dg_valid = false;
     if ((st = record(j, EV_TRACE))) return st;
-    if (j->g.precision == RBX_FP32 && (st = ensure_dgamma(j))) return st;
     if ((st = record(j, EV_TABLES))) return st;
     j->has_tables = true;
     return RBX_OK;
@@ -583,10 +582,10 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
         launch_forward_reduce(w.part, w.N, splits, w.D, j->stream);
         LAUNCHED(j, 2);
     } else {
-        launch_synth_fwd(w.tab, w.N, w.X, f, j->g.c0, w.G, j->stream);
+        launch_synth_fwd(w.f32, w.tab, w.v, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if (timed && (st = record(j, EV_SYNTH_F))) return st;
-        launch_forward_simt(w.G, w.v, w.N, w.X, w.fwd_splits, w.part, j->stream);
+        launch_forward_f32(w.f32, w.fwd_splits, w.part, j->stream);
         launch_forward_reduce(w.part, w.N, w.fwd_splits, w.D, j->stream);
         LAUNCHED(j, 2);
     }
@@ -642,17 +641,14 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
         launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
-        LAUNCHED(j, 1);
+        LAUNCHED(j, 4);
     } else if (preconditioned) {
-        rbx_status st = ensure_dgamma(j);
-        if (st) return st;
-        launch_synth_bp(w.tab, w.dg, w.N, w.X, f, j->g.c0, w.U, w.kap, j->stream);
-        launch_backproject_simt(w.U, w.kap, w.Rs, w.N, w.X, 0, w.gpart, j->stream);
+        launch_synth_bp(w.f32, w.tab, f, j->g.c0, j->stream);
+        LAUNCHED(j, launch_backproject_f32(w.f32, w.tab, w.Rs, w.gpart, j->stream));
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
     } else {
         double om = 2 * 3.14159265358979323846 * f;
-        launch_synth_fwd(w.tab, w.N, w.X, f, j->g.c0, w.G, j->stream);
-        launch_backproject_simt(w.G, nullptr, w.Rs, w.N, w.X, 1, w.gpart, j->stream);
+        LAUNCHED(j, launch_adjoint_f32(w.f32, w.tab, w.Rs, f, j->g.c0, w.gpart, j->stream));
         if (j->lossy)
             launch_combine_adjoint_lossy(w.gpart, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j),
                                          static_cast<float2 *>(out_dev), j->stream);
@@ -660,7 +656,7 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
             launch_combine_adjoint(w.gpart, w.X, 1, j->g.weight_mode, om * om * j->g.dx * j->g.dx,
                                    static_cast<float2 *>(out_dev), j->stream);
     }
-    LAUNCHED(j, 3);
+    LAUNCHED(j, 1);
     return RBX_OK;
 }
 
@@ -696,12 +692,10 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
         LAUNCHED(j, 3);
     } else {
-        if ((st = ensure_dgamma(j))) return st;
-        launch_synth_bp(w.tab, w.dg, w.N, w.X, f, j->g.c0, w.U, w.kap, j->stream);
+        launch_synth_bp(w.f32, w.tab, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if ((st = record(j, EV_SYNTH_B))) return st;
-        launch_backproject_simt(w.U, w.kap, w.Rs, w.N, w.X, 0, w.gpart, j->stream);
-        LAUNCHED(j, 1);
+        LAUNCHED(j, launch_backproject_f32(w.f32, w.tab, w.Rs, w.gpart, j->stream));
     }
     if ((st = record(j, EV_GEMM_B))) return st;
     const int roff = residual_blocks(w.N) + 8;
@@ -709,6 +703,12 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
                   w.counters, lossy_of(j), w.dmacc, mode, j->stream);
     LAUNCHED(j, 2);
     return RBX_OK;
+}
+
+// Where the kernels of an update's contractions record a bounded wait that gave up.
+static const unsigned *contraction_err(const rbx_job *j)
+{
+    return j->g.precision == RBX_FP32 ? j->w.f32.err : j->w.tc.err;
 }
 
 static rbx_status enqueue_update(rbx_job *j, double f, double df, const float2 *data, bool traced, int slot)
@@ -722,7 +722,7 @@ static rbx_status enqueue_update(rbx_job *j, double f, double df, const float2 *
     if ((st = enqueue_freq(j, f, df, data, 0))) return st;
     const int roff = residual_blocks(w.N) + 8;
     launch_snapshot(w.red + residual_blocks(w.N), w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters,
-                    w.tc.err, (unsigned long long)w.N * w.X, w.hist + (size_t)slot * kHistStride, j->stream);
+                    contraction_err(j), (unsigned long long)w.N * w.X, w.hist + (size_t)slot * kHistStride, j->stream);
     LAUNCHED(j, 1);
     if ((st = record(j, EV_UPDATE))) return st;
     j->ns_valid = false;   // the model changed
@@ -880,7 +880,7 @@ rbx_status rbx_update_set(rbx_job *j, const double *freqs, int nf, double df, co
         launch_acc_scalar(w.red + nb, w.red + nb + 4, k == 0, j->stream);
         LAUNCHED(j, 1);
     }
-    launch_snapshot(w.red + nb + 4, w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters, w.tc.err,
+    launch_snapshot(w.red + nb + 4, w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters, contraction_err(j),
                     (unsigned long long)w.N * w.X, w.hist, j->stream);
     LAUNCHED(j, 1);
     if ((st = record(j, EV_UPDATE))) return st;
@@ -1253,8 +1253,8 @@ size_t job_bytes_estimate(const rbx_geometry &g, int nf)
     const double r = g.mask_radius / g.dx;
     const size_t X = (size_t)(3.14159265358979 * r * r + 6.3 * r + 16);
     const size_t N = (size_t)g.n_xducers, NX = N * X, nxy = (size_t)g.nx * g.ny, NN = N * N;
-    size_t b = NX * (16 + 4 + 8);                                 // tables, angular density, G
-    if (g.precision == RBX_FP32) b += NX * 16;                    // U, kappa
+    size_t b = NX * (16 + 4 + 8);                                 // tables, angular density, FP32 operand planes
+    if (g.precision == RBX_FP32) b += NX * 16;                    // (24 B an entry in all)
     else {
         const size_t Np = (N + 127) / 128 * 128, Xk = (X + 63) / 64 * 64, Xm = (X + 127) / 128 * 128;
         const size_t m = g.precision == RBX_BF16X3 ? 2 : 1;

@@ -77,6 +77,19 @@ struct TcPlanes {
     bool ready = false;
 };
 
+// Operands of the FP32-accurate contractions of one job: FP32 values as three BF16 parts, their
+// TMA descriptors and the back-projection partials (k_gemm_f32.cu).
+struct F32Planes {
+    int N = 0, X = 0, xs = 0, xld = 0, rld = 0;   // xs nodes per slab, rows of xld (operands) and rld (R_s)
+    bool full = false;         // both operand sets of all nodes (FP32 jobs); else the plain adjoint's slab
+    size_t pstride = 0;
+    void *planes = nullptr;    // [12 or 6][N][xld] bf16
+    void *rs = nullptr;        // [6][N][rld] bf16
+    float2 *bpart = nullptr;   // [stacks][emitter tiles][X]; nullptr with one emitter tile
+    unsigned *err = nullptr;   // bounded-wait timeouts
+    CUtensorMap fmap, amap, rmap;   // K-major and M-major boxes of planes, K-major boxes of rs
+};
+
 // Device workspace of one job.
 struct Workspace {
     int N = 0, X = 0, nx = 0, ny = 0;
@@ -87,7 +100,6 @@ struct Workspace {
     TabEntry *tab = nullptr;
     float *dg = nullptr;
     float4 *exits = nullptr;
-    float2 *G = nullptr, *U = nullptr, *kap = nullptr;
     float2 *v = nullptr;        // Born weight Upsilon_m dA (m - m_s) per mask node (complex when lossy)
     float *alpha0 = nullptr;    // absorption map alpha0 [ny][nx], Np (rad/s)^-y m^-1 (lossy jobs only)
     double *as64 = nullptr;     // smoothed alpha0 (lossy jobs only)
@@ -101,6 +113,7 @@ struct Workspace {
     unsigned long long *counters = nullptr;   // [0] covered entries [1] clamped [2] bad rays [3] CAS bound [4] m <= 0 [5] bad model [6] mask count [7] uniform radius (float bits)
     int fwd_splits = 1;
     TcPlanes tc;
+    F32Planes f32;
 };
 
 // ---------------------------------------------------------------- kernels (launchers)
@@ -162,24 +175,31 @@ void launch_set_tables(const float *T, const float *a, const float *gam, const u
                        unsigned long long *counters, cudaStream_t s);
 void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, size_t n, cudaStream_t s);
 
-// k_gemm_simt.cu
-void launch_synth_fwd(const TabEntry *tab, int N, int X, double f, double c0, float2 *G, cudaStream_t s);
-void launch_synth_bp(const TabEntry *tab, const float *dg, int N, int X, double f, double c0, float2 *U,
-                     float2 *kap, cudaStream_t s);
+// k_born.cu
 // Born weights v[x] = Upsilon_m dA (m - m_s) (rough part) or Upsilon_m dA dm[x], with
 // Upsilon_m = omega c k~ at the node (omega^2 when lossless; c = current model).
 void launch_born_weights_rough(const float *c, const double *ns64, const int *idx, int X, double f, double dA,
                                const Lossy &ab, float2 *v, cudaStream_t s);
 void launch_born_weights_dm(const float *dm, const float *c, const int *idx, int X, double f, double dA,
                             const Lossy &ab, float2 *v, cudaStream_t s);
-int forward_splits(int N, int X);
-void launch_forward_simt(const float2 *G, const float2 *v, int N, int X, int splits, float2 *part, cudaStream_t s);
 void launch_forward_reduce(const float2 *part, int N, int splits, float2 *D, cudaStream_t s);
-// mode 0: preconditioned (A = U, conj(kap) U; W = U, kap U); mode 1: plain adjoint (A = W = conj(G))
-void launch_backproject_simt(const float2 *A, const float2 *kap, const float2 *Rs, int N, int X, int mode,
-                             float2 *gpart, cudaStream_t s);
+
+// k_gemm_f32.cu (FP32 accuracy on the tensor cores)
+int forward_splits(int N, int X);
+bool f32_setup(F32Planes &p, int N, int X, bool full, cudaStream_t s);
+void f32_free(F32Planes &p, cudaStream_t s);
+void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s);
+void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s);
+void launch_forward_f32(F32Planes &p, int splits, float2 *part, cudaStream_t s);
+// Both return the number of kernels launched. Preconditioned: the two stacks of the operands
+// that launch_synth_bp wrote. Plain adjoint: synthesis included.
+int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, float2 *gpart, cudaStream_t s);
+int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, double f, double c0, float2 *gpart,
+                       cudaStream_t s);
 
 // k_gemm_tc.cu (BF16 tensor cores)
+bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
+                  const cuuint32_t *box, const cuuint32_t *estr, CUtensorMapSwizzle swizzle);
 bool tc_setup(TcPlanes &p, int N, int X, bool split, cudaStream_t s);
 // Choose the forward K split by timing the candidates on this job's planes (once per shape
 // and process; later jobs of the shape reuse the choice). part holds fwd_max_splits partials.

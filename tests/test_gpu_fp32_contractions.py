@@ -1,0 +1,77 @@
+"""The FP32 contractions (three BF16 parts per operand on the tensor cores) at the edges of their
+tiles: transducer counts around one and two 128-wide tiles and 32-wide K chunks, odd node counts,
+and the plain adjoint of a tensor-core job, which goes through the nodes in slabs.
+
+Reference: the sums in complex128 on the same FP32 tables. Tolerance: an operand carries about six
+FP32 roundings (phase, sine, amplitude, products), two operands sqrt(12) 2^-24 = 2.1e-7 relative
+for rounding errors of random sign; sums of up to ~100 terms in FP32 add the same again; 1e-6
+leaves a factor of two and is below the 7.6e-6 that one lost low part (2^-17) would leave. The
+preconditioned operands divide by dgamma, a difference of FP32 angles of size 2 pi / N with an
+error of 2^-23: N 2^-24 on top.
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2211_00316_gb300 import phantoms as P
+from paper_2211_00316_gb300 import rbx
+
+pytestmark = pytest.mark.gpu
+
+F, C0 = 4e5, P.C_WATER
+
+
+def tables(g, seed):
+    rng = np.random.default_rng(seed)
+    X, Y = (v[g.mask()] for v in g.coords())
+    th = 2 * np.pi * np.arange(g.n_xducers) / g.n_xducers
+    dx, dy = X - g.ring_radius * np.cos(th)[:, None], Y - g.ring_radius * np.sin(th)[:, None]
+    s = np.hypot(dx, dy)
+    T = (s / C0 * (1 + 0.01 * np.sin(40 * X + th[:, None]))).astype(np.float32)
+    a = (s ** -0.5).astype(np.float32)
+    a[rng.random(a.shape) < 0.02] = 0.0                       # uncovered entries
+    gam = np.arctan2(dy, dx).astype(np.float32)
+    K = rng.integers(0, 3, a.shape).astype(np.uint8)
+    return T, a, gam, K
+
+
+def rel(x, y):
+    return float(np.linalg.norm(x - y) / np.linalg.norm(y))
+
+
+@pytest.mark.parametrize("n", [3, 16, 17, 31, 32, 33, 127, 128, 129, 144, 257])
+@pytest.mark.parametrize("nx,ny", [(24, 24), (41, 37)])
+def test_against_complex128(n, nx, ny):
+    g = P.Geometry(nx=nx, ny=ny, dx=1e-3, n_xducers=n, ring_radius=(min(nx, ny) - 1) * 0.5e-3 - 1.5e-3)
+    T, a, gam, K = tables(g, n)
+    rng = np.random.default_rng(7)
+    cov = a > 0
+    w = 2 * math.pi * F
+    Cg = (8 * math.pi * w / C0) ** -0.5
+    G = np.where(cov, Cg * a.astype(np.float64) * np.exp(2j * np.pi * (F * T.astype(np.float64) - K / 4 + 0.125)), 0)
+    gd = gam.astype(np.float64)
+    d = np.roll(gd, -1, 0) - np.roll(gd, 1, 0)
+    d = 0.5 * np.abs(np.mod(d + np.pi, 2 * np.pi) - np.pi)
+    d[~(np.roll(cov, -1, 0) & np.roll(cov, 1, 0))] = 0
+    U = np.where(cov, d / np.where(cov, G, 1), 0)
+    kap = np.exp(1j * gd)
+    dm = (1e-9 * rng.standard_normal((ny, nx))).astype(np.float32)
+    v = w * w * g.dx ** 2 * dm[g.mask()].astype(np.float64)
+    R = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    Rs = 0.5 * (R + R.T).astype(np.complex128)
+    want = {"forward": (G * v) @ G.T, "plain": w * w * g.dx ** 2 * (G.conj() * (Rs @ G.conj())).sum(0),
+            "pre": 2 * ((U * (Rs @ U)).sum(0) - (kap * U * (Rs @ (kap.conj() * U))).sum(0))}
+    dev = [torch.tensor(t, device="cuda") for t in (T, a, gam, K)]
+    exits = torch.zeros((n, n - 1, 4), device="cuda")
+    Rd, dmd = torch.tensor(R, device="cuda"), torch.tensor(dm, device="cuda")
+    for prec in (rbx.RBX_FP32, rbx.RBX_BF16):
+        job = rbx.Job()
+        job.set_geometry(g, precision=prec)
+        job.set_tables(*dev, exits)
+        assert rel(job.adjoint(F, Rd, False).cpu().numpy(), want["plain"]) <= 1e-6
+        if prec == rbx.RBX_FP32:
+            assert rel(job.forward(F, dmd).cpu().numpy(), want["forward"]) <= 1e-6
+            assert rel(job.adjoint(F, Rd, True).cpu().numpy(), want["pre"]) <= 1e-6 + n * 2.0 ** -24
+        job.close()
