@@ -32,6 +32,7 @@ struct RayParams {
     int N, X, nx, ny;
     float dx, x0, y0, R, ds, inv_dx, rmask;
     int maxs;
+    int lpr;              // lanes per ray of the trace (1: a warp traces 32 rays)
     const double *beta;   // [N] position angles of the transducers (device); nullptr: uniform ring 2 pi e / N
 };
 
@@ -154,7 +155,11 @@ struct TraceGroup {
     int njobs, total;
     TraceJob j[kMaxGroup];
 };
-// Work items of a job in the grouped trace (the per-job kernel's blocks).
+// Lanes per ray of a job's own trace: the most (up to 8) whose warps still fit the GPU at once
+// (152 SMs x 20). A small ring has too few rays to fill the GPU, so its rays' lanes share out
+// the rasterisation, which is most of a step's time there.
+int trace_lanes_per_ray(int N);
+// Work items of a job in the grouped trace (one lane per ray).
 int trace_items(int N, int *nwarps);
 // Resident blocks of the grouped trace on this device (its grid).
 int trace_grouped_blocks(bool lossy, bool raw, int max_ny);
