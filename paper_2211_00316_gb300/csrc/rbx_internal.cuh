@@ -157,7 +157,8 @@ struct TraceGroup {
 };
 // Lanes per ray of a job's own trace: the most (up to 8) whose warps still fit the GPU at once
 // (152 SMs x 20). A small ring has too few rays to fill the GPU, so its rays' lanes share out
-// the rasterisation, which is most of a step's time there.
+// the rasterisation, which is most of a step's time there (64 transducers: 0.63 -> 0.31 ms with
+// eight lanes and the two-stage rasteriser; 128: 0.94 -> 0.59 with four; 192: 1.17 -> 0.88 with two).
 int trace_lanes_per_ray(int N);
 // Work items of a job in the grouped trace (one lane per ray).
 int trace_items(int N, int *nwarps);
