@@ -419,7 +419,6 @@ static RayParams ray_params(const rbx_job *j)
     p.R = (float)j->g.ring_radius; p.ds = (float)j->g.ds; p.inv_dx = (float)(1.0 / j->g.dx);
     p.rmask = (float)j->g.mask_radius;
     p.maxs = max_steps(j->g);
-    p.lpr = trace_lanes_per_ray(w.N);
     p.beta = w.beta;
     return p;
 }
@@ -1104,7 +1103,6 @@ rbx_status rbx_batch_run(rbx_job *const *jobs, int n, const double *const *freqs
                 TraceJob &t = gr.j[gr.njobs++];
                 t.F = w.fields; t.rows = w.rows; t.tab = w.tab; t.exits = w.exits; t.counters = w.counters;
                 t.p = ray_params(jobs[i]);
-                t.p.lpr = 1;   // the group fills the GPU
                 t.item0 = gr.total;
                 gr.total += trace_items(w.N, &t.nwarps);
             }

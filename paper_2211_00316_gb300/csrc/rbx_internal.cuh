@@ -32,7 +32,6 @@ struct RayParams {
     int N, X, nx, ny;
     float dx, x0, y0, R, ds, inv_dx, rmask;
     int maxs;
-    int lpr;              // lanes per ray of the trace (1: a warp traces 32 rays)
     const double *beta;   // [N] position angles of the transducers (device); nullptr: uniform ring 2 pi e / N
 };
 
@@ -155,12 +154,7 @@ struct TraceGroup {
     int njobs, total;
     TraceJob j[kMaxGroup];
 };
-// Lanes per ray of a job's own trace: the most (up to 8) whose warps still fit the GPU at once
-// (152 SMs x 20). A small ring has too few rays to fill the GPU, so its rays' lanes share out
-// the rasterisation, which is most of a step's time there (64 transducers: 0.63 -> 0.31 ms with
-// eight lanes and the two-stage rasteriser; 128: 0.94 -> 0.59 with four; 192: 1.17 -> 0.88 with two).
-int trace_lanes_per_ray(int N);
-// Work items of a job in the grouped trace (one lane per ray).
+// Work items of a job in the grouped trace (the per-job kernel's blocks).
 int trace_items(int N, int *nwarps);
 // Resident blocks of the grouped trace on this device (its grid).
 int trace_grouped_blocks(bool lossy, bool raw, int max_ny);

@@ -1,6 +1,6 @@
 """The trace with one, two, four and eight lanes per ray (the transducer count decides), against the
-oracle's tables element by element with the bounds of the parity tests; the last warp of a fan is
-full, one ray short or nearly empty."""
+oracle's tables element by element with the bounds of the parity tests; the last 32 rays of a fan are
+all there, one short or nearly all missing."""
 import pytest
 
 from paper_2211_00316_gb300 import phantoms as P
