@@ -1313,98 +1313,6 @@ void launch_direct_green(const float4 *exits, int N, const double *beta, double 
 
 // ---------------------------------------------------------------- ray linking
 
-// One ray from (x, y) to the ring by one thread: the Heun and paraxial step of k_trace_raster
-// (same normalisations, the same compensated sums of the position and T and plain sums of
-// the momentum and the paraxial ray, the same reciprocals, the same final partial step)
-// without its rasterisation and straight-line shortcuts. The initial direction is formed in double so that a secant
-// iteration on it is not limited by FP32 rounding of the angle. Returns false when the ray
-// does not reach the ring within p.maxs steps.
-template <bool LOSSY, bool RAW>
-__device__ bool trace_one(const float *__restrict__ F, const RayParams &p, float x, float y, double gam0,
-                          float &theta, float &Tout, float &aout, int &Kout)
-{
-    const float ds = p.ds, hds = 0.5f * p.ds, R2 = p.R * p.R;
-    Fv F1;
-    field_eval<LOSSY, RAW>(F, p, x, y, F1);
-    double sd, cd;
-    sincos(gam0, &sd, &cd);
-    float px = F1.n * (float)cd, py = F1.n * (float)sd, dpx = -F1.n * (float)sd, dpy = F1.n * (float)cd;
-    float dxx = 0.f, dxy = 0.f, T = 0.f, Tc = 0.f, B = 0.f, Bc = 0.f;
-    float cx = 0.f, cy = 0.f;
-    float sc1 = 0.f, Jlast = 0.f;
-    int K = 0;
-    for (int i = 0; i < p.maxs; i++) {
-        const float n = F1.n, in = rcp_ap(n);
-        const float sc = n * rsqrtf(px * px + py * py);
-        px *= sc; py *= sc;
-        const float qx = px * in, qy = py * in;
-        Fv F2;
-        field_eval<LOSSY, RAW>(F, p, x + ds * qx, y + ds * qy, F2);
-        const float na = F2.n, ina = rcp_ap(na);
-        float pax = px + ds * F1.gx, pay = py + ds * F1.gy;
-        const float sca = na * rsqrtf(pax * pax + pay * pay);
-        pax *= sca; pay *= sca;
-        const float qax = pax * ina, qay = pay * ina;
-        const float sx = qx + qax, sy = qy + qay, rs = rsqrtf(sx * sx + sy * sy);
-        const float dirx = sx * rs, diry = sy * rs;
-        const float ddpx = hds * (F1.gx + F2.gx), ddpy = hds * (F1.gy + F2.gy);
-        const float gd = F1.gx * dxx + F1.gy * dxy, pd = px * dpx + py * dpy;
-        const float qdxx = in * (dpx - px * gd * in), qdxy = in * (dpy - py * gd * in);
-        const float w1 = in * (pd * in - gd);
-        const float qdpx = F1.hxx * dxx + F1.hxy * dxy + F1.gx * w1;
-        const float qdpy = F1.hxy * dxx + F1.hyy * dxy + F1.gy * w1;
-        const float dpax = dpx + ds * qdpx, dpay = dpy + ds * qdpy;
-        const float dxax = dxx + ds * qdxx, dxay = dxy + ds * qdxy;
-        const float gda = F2.gx * dxax + F2.gy * dxay, pda = pax * dpax + pay * dpay;
-        const float qdxax = ina * (dpax - pax * gda * ina), qdxay = ina * (dpay - pay * gda * ina);
-        const float w2 = ina * (pda * ina - gda);
-        const float qdpax = F2.hxx * dxax + F2.hxy * dxay + F2.gx * w2;
-        const float qdpay = F2.hxy * dxax + F2.hyy * dxay + F2.gy * w2;
-        const float ddxx = hds * (qdxx + qdxax), ddxy = hds * (qdxy + qdxay);
-        const float ddpx2 = hds * (qdpx + qdpax), ddpy2 = hds * (qdpy + qdpay);
-        const float xn = x + ds * dirx, yn = y + ds * diry;
-        field_eval<LOSSY, RAW>(F, p, xn, yn, F2);
-        float inc = hds * (F1.nr + F2.nr), incB = LOSSY ? hds * (F1.al + F2.al) : 0.f;
-        const bool last = xn * xn + yn * yn >= R2;
-        if (last) {
-            // as in k_trace_raster: a first step starts on the ring (|x|^2 - R^2 = 0)
-            float b = x * dirx + y * diry, cc = i == 0 ? 0.f : x * x + y * y - R2;
-            float disc = b * b - cc;
-            float t = -b + sqrtf(disc > 0.f ? disc : 0.f);
-            t = fminf(fmaxf(t, 0.f), ds);
-            float fr = t / ds;
-            x = x + t * dirx; y = y + t * diry;
-            inc *= fr;
-            incB *= fr;
-            dxx += fr * ddxx; dxy += fr * ddxy;
-            dpx += fr * ddpx2; dpy += fr * ddpy2;
-            px += fr * ddpx; py += fr * ddpy;
-            field_eval<LOSSY, RAW>(F, p, x, y, F2);
-        } else {
-            kadd(x, cx, ds * dirx); kadd(y, cy, ds * diry);
-            px += ddpx; py += ddpy;
-            dxx += ddxx; dxy += ddxy;
-            dpx += ddpx2; dpy += ddpy2;
-        }
-        kadd(T, Tc, inc);
-        if (LOSSY) kadd(B, Bc, incB);
-        F1 = F2;
-        const float rp = rsqrtf(px * px + py * py), tx = px * rp, ty = py * rp;
-        const float J = dxx * ty - dxy * tx;
-        if (i == 0) { sc1 = sqrtf(F1.nr * fabsf(J) / ds); Jlast = J; }
-        else if (J * Jlast < 0.f) K++;
-        if (J != 0.f) Jlast = J;
-        if (last) {
-            theta = atan2f(y, x);
-            Tout = T;
-            aout = sc1 * rsqrtf(F1.nr * fabsf(J)) * (LOSSY ? expf(-B) : 1.f);
-            Kout = K;
-            return true;
-        }
-    }
-    return false;
-}
-
 // Linked rays of the direct term (Sec. 4.4, Sec. 6.3.2), in two kernels.
 //
 // Linking, step 1, one block per transducer: the first bracketing pair of fan rays of every
@@ -1444,73 +1352,237 @@ __global__ void k_link_brackets(const float4 *__restrict__ exits, int N, const d
     }
 }
 
-// Linking, step 2, one thread per (transducer, receiver) pair; a block's four warps take the
-// same 32 receiver offsets m = r - e of four neighbouring transducers, so their rays, rotated
-// by one ring step, share L1 lines. From the bracketing fan rays a secant on the initial
+// Linking, step 2. A warp takes `chunk` consecutive receiver offsets m = r - e of one transducer, a
+// block's four warps the same offsets of four neighbouring ones, so their rays, rotated by one
+// ring step, share L1 lines. From the bracketing fan rays a secant on the initial
 // angle, kept inside the bracket (regula falsi with the Illinois weighting), stops when the
 // exit lies within tol radians of beta_r (at most maxit new rays); T and a are then
 // interpolated in exit angle between the two bracketing rays to beta_r exactly, K taken from
 // the nearer; linked[e][r] = (0, T, a, K) serves every frequency of the trace. Unbracketed
 // receivers take the nearest fan ray; those and the pairs that stopped on maxit are counted
 // in counters[1].
+//
+// A lane whose pair is linked takes the warp's next pair at once, and every lane's ray advances one
+// step per turn of the loop, whatever ray of whatever pair it is: rays of a warp differ in
+// length and pairs in their number of rays, and with one pair per lane half of the lanes waited
+// (16.5 of 32 at work). What happens between rays is in FP64, which is slow here, so it waits until
+// `wait` lanes need it; the secant's state lies in shared memory meanwhile. A warp with one pair
+// per lane (small rings) waits for all.
+// Linking alone, trace excluded: 256 transducers (288 x 288) 4.15 -> 2.19 ms, 512 (256 x 256, lossy)
+// 3.8 -> 2.6, 1024 (192 x 192) 9.05 -> 7.27; eight steps between looks at the other lanes (3.0 ms at
+// 512 with a look at every step).
+// The step is k_trace_raster's; the initial direction is formed in double so that the secant is not
+// limited by FP32 rounding of the angle.
 template <bool LOSSY, bool RAW>
 __global__ __launch_bounds__(128, 4) void k_link_rays(const float *__restrict__ F, RayParams p,
-                                                   const float4 *__restrict__ exits, int maxit, double tol,
+                                                   const float4 *__restrict__ exits, int maxit, double tol, int chunk,
                                                    float4 *__restrict__ linked, unsigned long long *counters)
 {
-    const int N = p.N;
-    const int e = blockIdx.y * 4 + (threadIdx.x >> 5), m = blockIdx.x * 32 + (threadIdx.x & 31) + 1;
-    if (e >= N || m > N - 1) return;
-    const int r = (e + m) % N;
+    enum { GA, GB, FA, FB, WA, WB, TA, TB, AA, AB, ND };
+    __shared__ double sd[ND][128];
+    __shared__ int sk[3][128];   // Ka, Kb, side
+    const unsigned FULL = 0xffffffffu;
+    const int N = p.N, q = threadIdx.x, lane = q & 31;
+    const int e = blockIdx.x * 4 + (q >> 5);
+    if (e >= N) return;
     const double PI = 3.14159265358979323846, TWO_PI = 2.0 * PI;
     const double step = TWO_PI / N, be = xducer_angle(e, N, step, p.beta);
-    const double td = recv_rel_m(m, e, N, step, p.beta, be);
-    float4 *slot = linked + (size_t)e * N + r;
-    const int code = __float_as_int(slot->x);
     const float4 *ex = exits + (size_t)e * (N - 1);
     auto rel = [&](double ang) { return wrap_turn(ang - be); };
-    double T, a;
-    int K;
-    if (code > 0) {
-        const int found = code;
-        const float xe = (float)(p.R * cos(be)), ye = (float)(p.R * sin(be));
-        const float4 A = ex[found - 1], Bq = ex[found];
-        // bracketing secant (regula falsi, Illinois weighting): every new ray starts between
-        // the two bracketing rays, so it points inward like the fan's
-        double ga = be + PI / 2 + PI * found / N, gb = be + PI / 2 + PI * (found + 1) / N;
-        double fa = rel(A.x) - td, fb = rel(Bq.x) - td, wa = fa, wb = fb;
-        double Ta = A.y, Tb = Bq.y, aa = A.z, ab = Bq.z;
-        int Ka = (int)A.w, Kb = (int)Bq.w, it = 0, side = 0;
-        while (fabs(fa) > tol && fabs(fb) > tol && it < maxit && wb != wa) {
-            const double gc = (ga * wb - gb * wa) / (wb - wa);
-            float thc, Tc, ac;
-            int Kc;
-            if (!trace_one<LOSSY, RAW>(F, p, xe, ye, gc, thc, Tc, ac, Kc)) break;
-            double fc = rel(thc) - td;
-            if (fc > PI) fc -= TWO_PI;
-            if (fc < -PI) fc += TWO_PI;
-            it++;
-            if ((fc > 0) == (fb > 0)) {
-                gb = gc; fb = fc; wb = fc; Tb = Tc; ab = ac; Kb = Kc;
-                if (side == -1) wa *= 0.5;
-                side = -1;
-            } else {
-                ga = gc; fa = fc; wa = fc; Ta = Tc; aa = ac; Ka = Kc;
-                if (side == 1) wb *= 0.5;
-                side = 1;
-            }
+    const float xe = (float)(p.R * cos(be)), ye = (float)(p.R * sin(be));
+    int next = 1 + warp_of_rank(blockIdx.y, gridDim.y) * chunk;   // the warp's next pair
+    const int end = min(N, next + chunk);
+
+    // the pair, its rays so far, and the ray on its way
+    bool has = false, busy = false, reached = false;
+    int m = 0, it = 0, i = 0, K = 0;
+    double td = 0.0, gc = 0.0;
+    float an = 0.f;
+    float x = 0.f, y = 0.f, px = 0.f, py = 0.f, dpx = 0.f, dpy = 0.f;
+    float dxx = 0.f, dxy = 0.f, T = 0.f, Tc = 0.f, B = 0.f, Bc = 0.f, cx = 0.f, cy = 0.f, sc1 = 0.f, Jlast = 0.f;
+    Fv F1{};
+    const float ds = p.ds, hds = 0.5f * p.ds, R2 = p.R * p.R;
+
+    // the next ray of the pair, or its result when it is linked or out of rays
+    auto advance = [&]() {
+        const double ga = sd[GA][q], gb = sd[GB][q], fa = sd[FA][q], fb = sd[FB][q], wa = sd[WA][q], wb = sd[WB][q];
+        if (fabs(fa) > tol && fabs(fb) > tol && it < maxit && wb != wa) {
+            gc = (ga * wb - gb * wa) / (wb - wa);
+            x = xe;
+            y = ye;
+            field_eval<LOSSY, RAW>(F, p, x, y, F1);
+            double sn, cd;
+            sincos(gc, &sn, &cd);
+            px = F1.n * (float)cd; py = F1.n * (float)sn; dpx = -F1.n * (float)sn; dpy = F1.n * (float)cd;
+            dxx = 0.f; dxy = 0.f; T = 0.f; Tc = 0.f; B = 0.f; Bc = 0.f;
+            cx = 0.f; cy = 0.f;
+            sc1 = 0.f; Jlast = 0.f;
+            K = 0;
+            i = 0;
+            busy = true;
+            return;
         }
         if (fabs(fa) > tol && fabs(fb) > tol) atomicAdd(&counters[1], 1ull);
         const double fr = (fb == fa) ? 0.0 : -fa / (fb - fa);
-        T = Ta + fr * (Tb - Ta);
-        a = aa + fr * (ab - aa);
-        K = fabs(fa) <= fabs(fb) ? Ka : Kb;
-    } else {
-        const float4 A = ex[-code - 1];
-        T = A.y; a = A.z; K = (int)A.w;
-        atomicAdd(&counters[1], 1ull);
+        const double To = sd[TA][q] + fr * (sd[TB][q] - sd[TA][q]);
+        const double ao = sd[AA][q] + fr * (sd[AB][q] - sd[AA][q]);
+        const int Ko = fabs(fa) <= fabs(fb) ? sk[0][q] : sk[1][q];
+        linked[(size_t)e * N + (e + m) % N] = make_float4(0.f, (float)To, (float)ao, (float)Ko);
+        has = false;
+    };
+    // the bracket after a ray (a ray that does not reach the ring ends the pair as it stands)
+    auto narrow = [&]() {
+        if (!reached) {
+            it = maxit;
+            return;
+        }
+        const float thc = atan2f(y, x);
+        double fc = rel(thc) - td;
+        if (fc > PI) fc -= TWO_PI;
+        if (fc < -PI) fc += TWO_PI;
+        it++;
+        if ((fc > 0) == (sd[FB][q] > 0)) {
+            sd[GB][q] = gc; sd[FB][q] = fc; sd[WB][q] = fc; sd[TB][q] = T; sd[AB][q] = an; sk[1][q] = K;
+            if (sk[2][q] == -1) sd[WA][q] *= 0.5;
+            sk[2][q] = -1;
+        } else {
+            sd[GA][q] = gc; sd[FA][q] = fc; sd[WA][q] = fc; sd[TA][q] = T; sd[AA][q] = an; sk[0][q] = K;
+            if (sk[2][q] == 1) sd[WB][q] *= 0.5;
+            sk[2][q] = 1;
+        }
+    };
+
+    const int wait = chunk > 32 ? 12 : 32;
+    for (;;) {
+        unsigned b = __ballot_sync(FULL, busy);
+        if (__popc(b) <= 32 - wait && (next < end || __any_sync(FULL, has && !busy))) {
+            if (has && !busy) narrow();
+            for (;;) {
+                // lanes without a pair take the next ones
+                const unsigned idle = __ballot_sync(FULL, !has);
+                const int mine = next + __popc(idle & ((1u << lane) - 1));
+                next += __popc(idle);
+                if (!has && mine < end) {
+                    m = mine;
+                    const int r = (e + m) % N, code = __float_as_int(linked[(size_t)e * N + r].x);
+                    if (code > 0) {
+                        const float4 A = ex[code - 1], Bq = ex[code];
+                        td = recv_rel_m(m, e, N, step, p.beta, be);
+                        // every new ray starts between the two bracketing rays, so it points inward
+                        // like the fan's
+                        sd[GA][q] = be + PI / 2 + PI * code / N;
+                        sd[GB][q] = be + PI / 2 + PI * (code + 1) / N;
+                        const double fa = rel(A.x) - td, fb = rel(Bq.x) - td;
+                        sd[FA][q] = sd[WA][q] = fa;
+                        sd[FB][q] = sd[WB][q] = fb;
+                        sd[TA][q] = A.y; sd[TB][q] = Bq.y; sd[AA][q] = A.z; sd[AB][q] = Bq.z;
+                        sk[0][q] = (int)A.w; sk[1][q] = (int)Bq.w; sk[2][q] = 0;
+                        it = 0;
+                        has = true;
+                    } else {
+                        const float4 A = ex[-code - 1];
+                        atomicAdd(&counters[1], 1ull);
+                        linked[(size_t)e * N + r] = make_float4(0.f, (float)(double)A.y, (float)(double)A.z, (float)(int)A.w);
+                    }
+                }
+                __syncwarp();
+                if (has && !busy) advance();
+                __syncwarp();
+                if (next >= end || !__any_sync(FULL, !has)) break;
+            }
+            b = __ballot_sync(FULL, busy);
+        }
+        if (!b) break;
+        if (busy) {
+            int k = 0;   // eight steps between looks at the other lanes (all, where the warp waits for all)
+            do {
+                const float n = F1.n, in = rcp_ap(n);
+                const float sc = n * rsqrtf(px * px + py * py);
+                px *= sc; py *= sc;
+                const float qx = px * in, qy = py * in;
+                Fv F2;
+                Cell<LOSSY, RAW> cell;   // one cell for both points, as in k_trace_raster
+                {
+                    const float ax = x + ds * qx, ay = y + ds * qy;
+                    const float u = (ax - p.x0) * p.inv_dx, v = (ay - p.y0) * p.inv_dx;
+                    cell_load<LOSSY, RAW>(F, p, u, v, cell);
+                    cell_eval<LOSSY, RAW>(cell, u - cell.i, v - cell.j, F2);
+                }
+                const float na = F2.n, ina = rcp_ap(na);
+                float pax = px + ds * F1.gx, pay = py + ds * F1.gy;
+                const float sca = na * rsqrtf(pax * pax + pay * pay);
+                pax *= sca; pay *= sca;
+                const float qax = pax * ina, qay = pay * ina;
+                const float sx = qx + qax, sy = qy + qay, rs = rsqrtf(sx * sx + sy * sy);
+                const float dirx = sx * rs, diry = sy * rs;
+                const float ddpx = hds * (F1.gx + F2.gx), ddpy = hds * (F1.gy + F2.gy);
+                const float gd = F1.gx * dxx + F1.gy * dxy, pd = px * dpx + py * dpy;
+                const float qdxx = in * (dpx - px * gd * in), qdxy = in * (dpy - py * gd * in);
+                const float w1 = in * (pd * in - gd);
+                const float qdpx = F1.hxx * dxx + F1.hxy * dxy + F1.gx * w1;
+                const float qdpy = F1.hxy * dxx + F1.hyy * dxy + F1.gy * w1;
+                const float dpax = dpx + ds * qdpx, dpay = dpy + ds * qdpy;
+                const float dxax = dxx + ds * qdxx, dxay = dxy + ds * qdxy;
+                const float gda = F2.gx * dxax + F2.gy * dxay, pda = pax * dpax + pay * dpay;
+                const float qdxax = ina * (dpax - pax * gda * ina), qdxay = ina * (dpay - pay * gda * ina);
+                const float w2 = ina * (pda * ina - gda);
+                const float qdpax = F2.hxx * dxax + F2.hxy * dxay + F2.gx * w2;
+                const float qdpay = F2.hxy * dxax + F2.hyy * dxay + F2.gy * w2;
+                const float ddxx = hds * (qdxx + qdxax), ddxy = hds * (qdxy + qdxay);
+                const float ddpx2 = hds * (qdpx + qdpax), ddpy2 = hds * (qdpy + qdpay);
+                const float xn = x + ds * dirx, yn = y + ds * diry;
+                Fv Fn;
+                {
+                    const float u = (xn - p.x0) * p.inv_dx, v = (yn - p.y0) * p.inv_dx;
+                    float tx = u - cell.i, ty = v - cell.j;
+                    if (!(tx >= 0.f && tx < 1.f && ty >= 0.f && ty < 1.f)) {
+                        cell_load<LOSSY, RAW>(F, p, u, v, cell);
+                        tx = u - cell.i; ty = v - cell.j;
+                    }
+                    cell_eval<LOSSY, RAW>(cell, tx, ty, Fn);
+                }
+                float inc = hds * (F1.nr + Fn.nr), incB = LOSSY ? hds * (F1.al + Fn.al) : 0.f;
+                const bool last = xn * xn + yn * yn >= R2;
+                if (last) {
+                    // as in k_trace_raster: a first step starts on the ring (|x|^2 - R^2 = 0)
+                    float b = x * dirx + y * diry, cc = i == 0 ? 0.f : __fsub_rn(__fmaf_rn(y, y, __fmul_rn(x, x)), R2);
+                    float disc = b * b - cc;
+                    float t = -b + sqrtf(disc > 0.f ? disc : 0.f);
+                    t = fminf(fmaxf(t, 0.f), ds);
+                    float fr = t / ds;
+                    x = x + t * dirx; y = y + t * diry;
+                    inc *= fr;
+                    incB *= fr;
+                    dxx += fr * ddxx; dxy += fr * ddxy;
+                    dpx += fr * ddpx2; dpy += fr * ddpy2;
+                    px += fr * ddpx; py += fr * ddpy;
+                    field_eval<LOSSY, RAW>(F, p, x, y, Fn);
+                } else {
+                    kadd(x, cx, ds * dirx); kadd(y, cy, ds * diry);
+                    px += ddpx; py += ddpy;
+                    dxx += ddxx; dxy += ddxy;
+                    dpx += ddpx2; dpy += ddpy2;
+                }
+                kadd(T, Tc, inc);
+                if (LOSSY) kadd(B, Bc, incB);
+                F1 = Fn;
+                const float rp = rsqrtf(px * px + py * py), tx = px * rp, ty = py * rp;
+                const float J = dxx * ty - dxy * tx;
+                if (i == 0) { sc1 = sqrtf(F1.nr * fabsf(J) / ds); Jlast = J; }
+                else if (J * Jlast < 0.f) K++;
+                if (J != 0.f) Jlast = J;
+                if (last) {
+                    an = sc1 * rsqrtf(F1.nr * fabsf(J)) * (LOSSY ? expf(-B) : 1.f);
+                    reached = true;
+                    busy = false;
+                } else if (++i == p.maxs) {
+                    reached = false;
+                    busy = false;
+                }
+            } while (busy && (wait == 32 || ++k < 8));
+        }
+        __syncwarp();
     }
-    *slot = make_float4(0.f, (float)T, (float)a, (float)K);
 }
 
 // g[e][r] = C a exp(i 2 pi (f T - K/4 + 1/8)) from the linked rays' (-, T, a, K); 0 on the diagonal
@@ -1541,15 +1613,18 @@ void launch_link_rays(const float *fields, const RayParams &p, const float4 *exi
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_link_brackets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_link_brackets<<<p.N, 256, smem, s>>>(exits, p.N, p.beta, linked);
     const double tol = 1e-6;
-    const dim3 grd((p.N - 1 + 31) / 32, (p.N + 3) / 4);
+    // two sets of warps for the GPU (152 SMs x 16), at least a pair and at most eight pairs per lane
+    int chunk = (int)((size_t)p.N * (p.N - 1) / (2 * 152 * 16) + 31) / 32 * 32;
+    chunk = chunk < 32 ? 32 : (chunk > 256 ? 256 : chunk);
+    const dim3 grd((p.N + 3) / 4, (p.N - 1 + chunk - 1) / chunk);
     if (lossy && raw)
-        k_link_rays<true, true><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, linked, counters);
+        k_link_rays<true, true><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, chunk, linked, counters);
     else if (lossy)
-        k_link_rays<true, false><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, linked, counters);
+        k_link_rays<true, false><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, chunk, linked, counters);
     else if (raw)
-        k_link_rays<false, true><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, linked, counters);
+        k_link_rays<false, true><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, chunk, linked, counters);
     else
-        k_link_rays<false, false><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, linked, counters);
+        k_link_rays<false, false><<<grd, 128, 0, s>>>(fields, p, exits, maxit, tol, chunk, linked, counters);
 }
 
 // ---------------------------------------------------------------- table I/O
