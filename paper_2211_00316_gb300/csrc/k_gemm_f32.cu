@@ -1,5 +1,6 @@
 // Steps a6-a8 at FP32 accuracy on the tensor cores: Green's function synthesis and the two
-// complex contractions of an FP32 job (and the plain adjoint of every job).
+// complex contractions of an FP32 job (and the plain adjoint of every job), and the same with
+// split BF16 (hi + lo).
 //
 //  forward (Eqs. perturb1, derivative):  D[e,r] = sum_x G_e[x] G_r[x] v[x]
 //  back-projection (Eq. sound_speed_update2), exact two-term factorisation:
@@ -16,7 +17,8 @@
 // to nearest, so a long sum there drifts; here a sum in tensor memory covers 32 terms of K (one
 // pipeline stage, the five small products before hi hi so that only four additions meet the
 // full-size sum) and is then added to FP32 registers, rounded to nearest, by the epilogue warps.
-// Two accumulator buffers alternate, so the MMAs do not wait for that. Sums over 16 terms gave
+// Two accumulator buffers alternate, so the MMAs do not wait for that. Split BF16 takes two parts
+// and three products in the same way. Sums over 16 terms gave
 // no smaller error (twice as many FP32 additions follow) and ran 7 % slower.
 #include "rbx_internal.cuh"
 #include "tc_sm100.cuh"
@@ -31,11 +33,16 @@ using namespace tc;
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 32;
-constexpr int PARTS = 6;                                   // re hi, mid, lo, im hi, mid, lo
 constexpr uint32_t PLANE = BM * BK * 2;                    // 8 KB: one part of one operand tile
-constexpr uint32_t OPER = PARTS * PLANE;                   // 48 KB: an operand's tile, all parts
-constexpr int STAGES = 2;
-constexpr size_t G_SMEM = 1024 + (size_t)STAGES * 2 * OPER + 4352;
+// NP parts per real number: planes re hi (, mid), lo, im hi (, mid), lo
+template <int NP>
+struct Form {
+    static constexpr int PLANES = 2 * NP;
+    static constexpr uint32_t OPER = PLANES * PLANE;       // an operand's tile, all parts: 48 or 32 KB
+    static constexpr int STAGES = NP == 3 ? 2 : 3;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * 2 * OPER + 4352;
+    static constexpr int PRODUCTS = NP == 3 ? 6 : 3;
+};
 constexpr int EPI = 256;                                   // epilogue threads (warps 2..9)
 constexpr int THREADS = 64 + EPI;
 
@@ -64,11 +71,12 @@ __device__ __forceinline__ uint64_t desc_k64(uint32_t saddr)
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
-// M-major, 128-byte swizzle: 64 rows of M contiguous, the next 64 rows PARTS * 4 KB on, groups
+// M-major, 128-byte swizzle: 64 rows of M contiguous, the next 64 rows half an operand on, groups
 // of 8 K 1024 B apart.
+template <int NP>
 __device__ __forceinline__ uint64_t desc_m128(uint32_t saddr)
 {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((OPER / 2) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((Form<NP>::OPER / 2) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
@@ -98,6 +106,10 @@ struct GemmArgs {
 // BP false: the forward's upper tile pair (te, tr) over the K chunks of one split.
 // BP true: for 128 nodes, 128 emitters and one stack, P = A^T R_s over all receivers and the
 // row-dot with the weights. CONJ: the plain adjoint, A = W = conj(G).
+// NP = 3: FP32 accuracy, six products. NP = 2 (split BF16): hi hi + hi lo + lo hi; against kernels
+// that drained long sums to global memory (forward) or stopped for the drain (back-projection),
+// 768 transducers, 59,800 nodes: an update from tables 3.24 -> 2.60 ms, forward error 2.7e-6 ->
+// 1.1e-6.
 //
 // Bound: shared-memory bandwidth of the tensor cores. A 128 x 128 x 16 MMA reads 8 KB in the 64
 // clocks it takes at the peak rate (128 B per clock, all an SM has), the tile loads write 31 B
@@ -108,9 +120,11 @@ struct GemmArgs {
 // transducers, 19,760 nodes: plain adjoint 2915 -> 384 us. Error against 64 bits no larger at any
 // size from 48 transducers on (N = 1024, 20,000 nodes: forward 6.0e-7 -> 2.2e-7, plain adjoint
 // 6.1e-7 -> 1.7e-7).
-template <bool BP, bool CONJ>
+template <int NP, bool BP, bool CONJ>
 __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant__ GemmArgs g)
 {
+    constexpr int STAGES = Form<NP>::STAGES, PLANES = Form<NP>::PLANES;
+    constexpr uint32_t OPER = Form<NP>::OPER;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(tiles + (size_t)STAGES * 2 * OPER);
@@ -160,12 +174,12 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
             const uint32_t base = smem_u32(tiles + (size_t)s * 2 * OPER);
             const int k = (c0 + c) * BK;
             if (BP) {
-                tma_load_3d(base, &g.a, full + s, ta * BM, k, PARTS * stack);
-                tma_load_3d(base + OPER / 2, &g.a, full + s, ta * BM + 64, k, PARTS * stack);
+                tma_load_3d(base, &g.a, full + s, ta * BM, k, PLANES * stack);
+                tma_load_3d(base + OPER / 2, &g.a, full + s, ta * BM + 64, k, PLANES * stack);
                 tma_load_3d(base + OPER, &g.b, full + s, k, tb * BN, 0);
             } else {
                 tma_load_3d(base, &g.a, full + s, k, ta * BM, 0);
-                tma_load_3d(base + OPER, &g.a, full + s, k, tb * BN, PARTS);
+                tma_load_3d(base + OPER, &g.a, full + s, k, tb * BN, PLANES);
             }
             issued++;
         }
@@ -187,16 +201,17 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
                 const uint32_t a = smem_u32(tiles + (size_t)s * 2 * OPER), b = a + OPER;
                 constexpr uint32_t APART = BP ? PLANE / 2 : PLANE, AK = BP ? 2048 : 32;
 #pragma unroll
-                for (int p = 0; p < 6; p++) {
-                    // (hi, lo), (lo, hi), (mid, mid), (hi, mid), (mid, hi), (hi, hi)
+                for (int p = 6 - Form<NP>::PRODUCTS; p < 6; p++) {
+                    // three parts: (hi, lo), (lo, hi), (mid, mid), (hi, mid), (mid, hi), (hi, hi); of
+                    // two parts, hi and lo, the last three
                     constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};
 #pragma unroll
                     for (int k = 0; k < BK / 16; k++) {
                         const uint32_t ar = a + PA[p] * APART + k * AK, br = b + PB[p] * PLANE + k * 32;
-                        const uint64_t a0 = BP ? desc_m128(ar) : desc_k64(ar);
-                        const uint64_t a1 = BP ? desc_m128(ar + 3 * APART) : desc_k64(ar + 3 * APART);
-                        const uint64_t b0 = desc_k64(br), b1 = desc_k64(br + 3 * PLANE);
-                        const uint32_t acc = (p > 0 || k > 0) ? 1u : 0u;
+                        const uint64_t a0 = BP ? desc_m128<NP>(ar) : desc_k64(ar);
+                        const uint64_t a1 = BP ? desc_m128<NP>(ar + NP * APART) : desc_k64(ar + NP * APART);
+                        const uint64_t b0 = desc_k64(br), b1 = desc_k64(br + NP * PLANE);
+                        const uint32_t acc = (p > 6 - Form<NP>::PRODUCTS || k > 0) ? 1u : 0u;
                         mma_bf16(dre, a0, b0, ip, acc);
                         mma_bf16(dre, a1, b1, i_re, 1u);
                         mma_bf16(dim, a0, b1, ip, acc);
@@ -270,13 +285,13 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
                 // and a chain of single rows waits for each
 #pragma unroll 1
                 for (int i0 = 0; i0 < ne; i0 += 8) {
-                    __nv_bfloat162 q[8][6];
+                    __nv_bfloat162 q[8][PLANES];
                     float gam[8][2];
 #pragma unroll
                     for (int k = 0; k < 8; k++) {
                         const int i = min(i0 + k, ne - 1);
 #pragma unroll
-                        for (int m = 0; m < 6; m++)
+                        for (int m = 0; m < PLANES; m++)
                             q[k][m] = *reinterpret_cast<const __nv_bfloat162 *>(w + (size_t)i * g.xld + m * g.pstride);
                         if (!CONJ && stack == 1) {
                             // an uncovered entry's weight is zero and its direction not a number
@@ -292,10 +307,13 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
                         const float4 p = *reinterpret_cast<const float4 *>(P + (quarter * 32 + i0 + k) * BM + r2);
 #pragma unroll
                         for (int h = 0; h < 2; h++) {
-                            float v[6];   // the parts add up to the FP32 weight exactly
+                            // the parts add up to the weight (three: the FP32 weight) exactly
+                            float wr = 0.f, wi = 0.f;
 #pragma unroll
-                            for (int m = 0; m < 6; m++) v[m] = h ? __high2float(q[k][m]) : __low2float(q[k][m]);
-                            float wr = v[0] + v[1] + v[2], wi = v[3] + v[4] + v[5];
+                            for (int m = 0; m < NP; m++) {
+                                wr += h ? __high2float(q[k][m]) : __low2float(q[k][m]);
+                                wi += h ? __high2float(q[k][NP + m]) : __low2float(q[k][NP + m]);
+                            }
                             if (CONJ) wi = -wi;
                             if (!CONJ && stack == 1) {
                                 const float2 kap = unit_of(gam[k][h]);
@@ -343,40 +361,43 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
     }
 }
 
-// v = hi + mid + lo, each BF16
-__device__ __forceinline__ void split3(float v, __nv_bfloat16 *q)
+// v = hi (+ mid) + lo, each BF16
+template <int NP>
+__device__ __forceinline__ void split(float v, __nv_bfloat16 *q)
 {
-    q[0] = __float2bfloat16_rn(v);
-    v -= __bfloat162float(q[0]);
-    q[1] = __float2bfloat16_rn(v);
-    v -= __bfloat162float(q[1]);
-    q[2] = __float2bfloat16_rn(v);
+#pragma unroll
+    for (int k = 0; k < NP; k++) {
+        q[k] = __float2bfloat16_rn(v);
+        v -= __bfloat162float(q[k]);
+    }
 }
 
-// The six parts of two neighbouring complex values to [plane][N][xld]
+// The parts of two neighbouring complex values to [plane][N][xld]
+template <int NP>
 __device__ __forceinline__ void put_parts(__nv_bfloat16 *planes, size_t pstride, size_t at, const float2 *z)
 {
-    __nv_bfloat16 a[6], b[6];
-    split3(z[0].x, a);
-    split3(z[0].y, a + 3);
-    split3(z[1].x, b);
-    split3(z[1].y, b + 3);
+    __nv_bfloat16 a[2 * NP], b[2 * NP];
+    split<NP>(z[0].x, a);
+    split<NP>(z[0].y, a + NP);
+    split<NP>(z[1].x, b);
+    split<NP>(z[1].y, b + NP);
 #pragma unroll
-    for (int k = 0; k < 6; k++)
+    for (int k = 0; k < 2 * NP; k++)
         *reinterpret_cast<__nv_bfloat162 *>(planes + k * pstride + at) = __halves2bfloat162(a[k], b[k]);
 }
 
 // Operands of the contractions from the tables, two nodes and `walk` transducers per thread, as
 // parts in [plane][N][xld] for the slab of nx nodes from x0 on.
-//  KIND 0: planes 0-5 G_e[x] = (8 pi omega/c0)^(-1/2) a exp(i 2 pi (f T - K/4 + 1/8)) (Eq. 2D_greens)
-//  KIND 1: planes 0-5 G, planes 6-11 G v (the forward)
-//  KIND 2: planes 0-5 u_e[x] = dgamma / ((8 pi omega/c0)^(-1/2) a) exp(-i 2 pi (...)) (Eq.
-//          greens-time-reversed), planes 6-11 conj(kappa) u. The angular density dgamma (step a4)
+//  KIND 0: first operand G_e[x] = (8 pi omega/c0)^(-1/2) a exp(i 2 pi (f T - K/4 + 1/8)) (Eq. 2D_greens)
+//  KIND 1: first G, second G v (the forward)
+//  KIND 2: first u_e[x] = dgamma / ((8 pi omega/c0)^(-1/2) a) exp(-i 2 pi (...)) (Eq.
+//          greens-time-reversed), second conj(kappa) u. The angular density dgamma (step a4)
 //          comes from the direction angles of the neighbouring transducers, kept in registers as
 //          the thread walks its transducers: the tables are read 1 + 2 / walk times and no
 //          array of dgamma is written or read.
-// Bound: HBM. Per entry 16 B are read and 24 B (12 B for KIND 0) written.
-template <int KIND>
+// Bound: HBM. Per entry 16 B are read and 8 NP B (4 NP for KIND 0) written; 512 transducers, 47,660
+// nodes, NP = 3: 0.98 GB in 147 us.
+template <int KIND, int NP>
 __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict__ tab, const float2 *__restrict__ v, int N,
                                                      int X, int x0, int nx, int xld, size_t pstride, float fhi, float flo,
                                                      float C, __nv_bfloat16 *__restrict__ planes, int walk)
@@ -425,8 +446,8 @@ __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict_
             }
         }
         const size_t at = (size_t)e * xld + xl;
-        put_parts(planes, pstride, at, z);
-        if (KIND != 0) put_parts(planes + 6 * pstride, pstride, at, z2);
+        put_parts<NP>(planes, pstride, at, z);
+        if (KIND != 0) put_parts<NP>(planes + 2 * NP * pstride, pstride, at, z2);
 #pragma unroll
         for (int q = 0; q < 2; q++) {
             prev[q] = cur[q];
@@ -435,18 +456,19 @@ __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict_
     }
 }
 
-// R_s (complex N x N) -> parts [6][N][rld]
+// R_s (complex N x N) -> parts [2 NP][N][rld]
+template <int NP>
 __global__ void k_rs_parts(const float2 *__restrict__ Rs, int N, int rld, __nv_bfloat16 *__restrict__ planes)
 {
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= (size_t)N * N) return;
     const size_t o = (i / N) * rld + i % N, P = (size_t)N * rld;
-    __nv_bfloat16 q[6];
+    __nv_bfloat16 q[2 * NP];
     const float2 v = Rs[i];
-    split3(v.x, q);
-    split3(v.y, q + 3);
+    split<NP>(v.x, q);
+    split<NP>(v.y, q + NP);
 #pragma unroll
-    for (int k = 0; k < 6; k++) planes[k * P + o] = q[k];
+    for (int k = 0; k < 2 * NP; k++) planes[k * P + o] = q[k];
 }
 
 // gpart[stack][x] = sum over emitter tiles, in order
@@ -475,13 +497,13 @@ float green_const(double f, double c0)
 }
 
 // BF16 planes [planes][rows][cols], rows ld elements apart, read in boxes of `inner` columns,
-// `outer` rows and six planes
+// `outer` rows and `deep` planes
 bool make_map(CUtensorMap *m, void *base, size_t cols, size_t rows, size_t planes, size_t ld, unsigned inner,
-              unsigned outer)
+              unsigned outer, unsigned deep)
 {
     cuuint64_t dims[3] = {cols, rows, planes};
     cuuint64_t strides[2] = {ld * 2, ld * rows * 2};
-    cuuint32_t box[3] = {inner, outer, PARTS}, estr[3] = {1, 1, 1};
+    cuuint32_t box[3] = {inner, outer, deep}, estr[3] = {1, 1, 1};
     return encode_tiled(m, base, 3, dims, strides, box, estr,
                         inner * 2 == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
@@ -495,9 +517,14 @@ void synth(const F32Planes &p, const TabEntry *tab, const float2 *v, int x0, int
     // problems, which a long walk leaves waiting on its chain of loads
     const unsigned bx = (unsigned)((nx + 255) / 256);
     const int walk = (size_t)bx * ((p.N + 7) / 8) >= 152 * 16 ? 8 : 2;
-    k_synth_parts<KIND><<<dim3(bx, (unsigned)((p.N + walk - 1) / walk)), 128, 0, s>>>(
-        tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo, green_const(f, c0), static_cast<__nv_bfloat16 *>(p.planes),
-        walk);
+    const dim3 grd(bx, (unsigned)((p.N + walk - 1) / walk));
+    __nv_bfloat16 *planes = static_cast<__nv_bfloat16 *>(p.planes);
+    if (p.parts == 3)
+        k_synth_parts<KIND, 3><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo,
+                                                   green_const(f, c0), planes, walk);
+    else
+        k_synth_parts<KIND, 2><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo,
+                                                   green_const(f, c0), planes, walk);
 }
 
 }  // namespace
@@ -516,37 +543,44 @@ int forward_splits(int N, int X)
     return (nk + kper - 1) / kper;
 }
 
-bool f32_setup(F32Planes &p, int N, int X, bool full, cudaStream_t st)
+template <int NP>
+static bool allow_smem()
+{
+    return cudaFuncSetAttribute(k_cgemm_f32<NP, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Form<NP>::SMEM) == cudaSuccess &&
+           cudaFuncSetAttribute(k_cgemm_f32<NP, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Form<NP>::SMEM) == cudaSuccess &&
+           (NP != 3 ||   // the plain adjoint always takes three parts
+            cudaFuncSetAttribute(k_cgemm_f32<3, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)Form<3>::SMEM) == cudaSuccess);
+}
+
+bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st)
 {
     p.N = N;
     p.X = X;
+    p.parts = parts;
     p.full = full;
     const int x8 = (X + 7) / 8 * 8;
-    // all nodes' forward or back-projection operands (24 B an entry), or on a tensor-core job,
+    // all nodes' forward or back-projection operands (24 or 16 B an entry), or on a tensor-core job,
     // whose plain adjoint alone comes here, 8 B an entry and the nodes in slabs
     p.xs = full ? x8 : std::max(std::min(x8, 64), X * 2 / 3 / 8 * 8);
     p.xld = p.xs;
     p.pstride = (size_t)N * p.xld;
     p.rld = (N + 7) / 8 * 8;
-    const size_t bytes = (full ? 12 : 6) * p.pstride * sizeof(__nv_bfloat16);
+    const size_t deep = 2 * parts, planes = full ? 2 * deep : deep;
     const size_t ET = (N + BN - 1) / BN;
-    if (cudaMallocAsync(&p.planes, bytes, st) != cudaSuccess) return false;
-    if (cudaMallocAsync(&p.rs, PARTS * (size_t)N * p.rld * sizeof(__nv_bfloat16), st) != cudaSuccess) return false;
+    if (cudaMallocAsync(&p.planes, planes * p.pstride * sizeof(__nv_bfloat16), st) != cudaSuccess) return false;
+    if (cudaMallocAsync(&p.rs, deep * N * p.rld * sizeof(__nv_bfloat16), st) != cudaSuccess) return false;
     if (ET > 1 &&   // with one emitter tile the partial row-dots are the result
         cudaMallocAsync(reinterpret_cast<void **>(&p.bpart), (full ? 2 : 1) * ET * X * sizeof(float2), st) != cudaSuccess)
         return false;
     if (cudaMallocAsync(reinterpret_cast<void **>(&p.err), sizeof(unsigned), st) != cudaSuccess) return false;
     cudaMemsetAsync(p.err, 0, sizeof(unsigned), st);
-    const size_t cols = std::min(p.xs, X), planes = full ? 12 : 6;
-    return make_map(&p.fmap, p.planes, cols, N, planes, p.xld, BK, BM) &&
-           make_map(&p.amap, p.planes, cols, N, planes, p.xld, 64, BK) &&
-           make_map(&p.rmap, p.rs, N, N, PARTS, p.rld, BK, BN) &&
-           cudaFuncSetAttribute(k_cgemm_f32<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_cgemm_f32<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_cgemm_f32<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM) ==
-               cudaSuccess;
+    const size_t cols = std::min(p.xs, X);
+    return make_map(&p.fmap, p.planes, cols, N, planes, p.xld, BK, BM, deep) &&
+           make_map(&p.amap, p.planes, cols, N, planes, p.xld, 64, BK, deep) &&
+           make_map(&p.rmap, p.rs, N, N, deep, p.rld, BK, BN, deep) && (parts == 3 ? allow_smem<3>() : allow_smem<2>());
 }
 
 void f32_free(F32Planes &p, cudaStream_t st)
@@ -578,7 +612,11 @@ void launch_forward_f32(F32Planes &p, int splits, float2 *part, cudaStream_t s)
     g.kper = (nk + splits - 1) / splits;
     g.part = part;
     g.err = p.err;
-    k_cgemm_f32<false, false><<<dim3(T * (T + 1) / 2, splits), THREADS, G_SMEM, s>>>(g);
+    const dim3 grd(T * (T + 1) / 2, splits);
+    if (p.parts == 3)
+        k_cgemm_f32<3, false, false><<<grd, THREADS, Form<3>::SMEM, s>>>(g);
+    else
+        k_cgemm_f32<2, false, false><<<grd, THREADS, Form<2>::SMEM, s>>>(g);
 }
 
 static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
@@ -601,7 +639,11 @@ static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
 static void rs_parts(F32Planes &p, const float2 *Rs, cudaStream_t s)
 {
     const size_t nn = (size_t)p.N * p.N;
-    k_rs_parts<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
+    const unsigned nb = (unsigned)((nn + 255) / 256);
+    if (p.parts == 3)
+        k_rs_parts<3><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
+    else
+        k_rs_parts<2><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
 }
 
 // The preconditioned back-projection from the operands of launch_synth_bp: gpart[2][X].
@@ -611,7 +653,11 @@ int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, 
     rs_parts(p, Rs, s);
     GemmArgs g = bp_args(p, tab, gpart);
     g.nx = p.X;
-    k_cgemm_f32<true, false><<<dim3(ET, (p.X + BM - 1) / BM, 2), THREADS, G_SMEM, s>>>(g);
+    const dim3 grd(ET, (p.X + BM - 1) / BM, 2);
+    if (p.parts == 3)
+        k_cgemm_f32<3, true, false><<<grd, THREADS, Form<3>::SMEM, s>>>(g);
+    else
+        k_cgemm_f32<2, true, false><<<grd, THREADS, Form<2>::SMEM, s>>>(g);
     if (ET == 1) return 2;
     k_bp_sum<<<dim3((p.X + 255) / 256, 2), 256, 0, s>>>(p.bpart, ET, p.X, gpart);
     return 3;
@@ -629,7 +675,7 @@ int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, doub
         g.x0 = x0;
         g.nx = std::min(p.xs, p.X - x0);
         synth<0>(p, tab, nullptr, x0, g.nx, f, c0, s);
-        k_cgemm_f32<true, true><<<dim3(ET, (g.nx + BM - 1) / BM, 1), THREADS, G_SMEM, s>>>(g);
+        k_cgemm_f32<3, true, true><<<dim3(ET, (g.nx + BM - 1) / BM, 1), THREADS, Form<3>::SMEM, s>>>(g);   // parts == 3
     }
     if (ET == 1) return n;
     k_bp_sum<<<dim3((p.X + 255) / 256, 1), 256, 0, s>>>(p.bpart, ET, p.X, gpart);

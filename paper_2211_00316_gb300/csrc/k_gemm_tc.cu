@@ -36,6 +36,7 @@ namespace {
 constexpr int BM = 128, BN = 128, BK = 64;
 constexpr uint32_t TILE = BM * BK * 2;        // 16 KB: 128 rows x 64 BF16 (128 B per row)
 
+constexpr int kSynWalk = 8;                   // transducers a thread of the forward's synthesis walks
 constexpr int F_STAGES = 3, F_TILES = 4;     // forward: Gre, Gim | Gvre, Gvim
 constexpr size_t F_SMEM = 1024 + (size_t)F_STAGES * F_TILES * TILE + 256;
 constexpr int B_STAGES = 2, B_TILES = 6;     // back-projection: Ure, Uim, Vre, Vim | Rsre, Rsim
@@ -71,30 +72,20 @@ __device__ __forceinline__ uint8_t *align1024(uint8_t *p)
 
 // ---------------------------------------------------------------- forward
 
-// Operand maps of one K pass: A (re, im) and B (re, im).
+// Operand maps: A (re, im) and B (re, im).
 struct Maps4 {
     CUtensorMap are, aim, bre, bim;
 };
 
-// passes = 1: A_hi B_hi. passes = 3 (split BF16): A_hi B_hi + A_hi B_lo + A_lo B_hi.
-// With split BF16 the tensor-memory accumulators are drained every kSeg K chunks into the
-// CTA's FP32 partial tile in global memory (the CTA owns that tile), so no accumulation in
-// tensor memory runs over more than kSeg x 64 mask nodes (its long-K rounding would
-// otherwise exceed the split's own error); two accumulator buffers alternate so the MMAs
-// never wait for the drain. Plain BF16, whose error is its input rounding, uses one segment.
-constexpr int kSeg = 16;
-
-__global__ __launch_bounds__(192, 1) void k_forward_tc(const __grid_constant__ Maps4 hi, const __grid_constant__ Maps4 lo,
-                                                       int passes, int N, int ntile, int nk, int kper,
-                                                       float2 *__restrict__ part, unsigned *__restrict__ err)
+__global__ __launch_bounds__(192, 1) void k_forward_tc(const __grid_constant__ Maps4 maps, int N, int ntile, int nk,
+                                                       int kper, float2 *__restrict__ part, unsigned *__restrict__ err)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *tiles = align1024(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(tiles + (size_t)F_STAGES * F_TILES * TILE);
     uint64_t *empty = full + F_STAGES;
-    uint64_t *accf = empty + F_STAGES;     // [2] accumulator buffer ready to drain
-    uint64_t *acce = accf + 2;             // [2] accumulator buffer drained
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + 2);
+    uint64_t *accf = empty + F_STAGES;     // accumulators ready to drain
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(accf + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     int b = blockIdx.x, te = 0;
@@ -102,36 +93,31 @@ __global__ __launch_bounds__(192, 1) void k_forward_tc(const __grid_constant__ M
     const int tr = te + b;
     const int split = blockIdx.y;
     const int c0 = split * kper, nc = min(nk, c0 + kper) - c0;
-    const int ntot = passes * nc;
-    const int seglen = passes == 3 ? kSeg : (ntot > 0 ? ntot : 1);
-    const int nseg = (ntot + seglen - 1) / seglen;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < F_STAGES; s++) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
-        for (int q = 0; q < 2; q++) { mbar_init(accf + q, 1); mbar_init(acce + q, 128); }
+        mbar_init(accf, 1);
         fence_mbar_init();
     }
-    if (warp == 1) tmem_alloc(tslot, 512);
+    if (warp == 1) tmem_alloc(tslot, 256);
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tslot;
 
     if (warp == 0 && lane == 0) {
-        prefetch_tmap(&hi.are); prefetch_tmap(&hi.aim); prefetch_tmap(&hi.bre); prefetch_tmap(&hi.bim);
+        prefetch_tmap(&maps.are); prefetch_tmap(&maps.aim); prefetch_tmap(&maps.bre); prefetch_tmap(&maps.bim);
         int issued = 0;
-        for (int c = 0; c < ntot; c++) {
-            int s = c % F_STAGES;
+        for (int c = 0; c < nc; c++) {
+            const int s = c % F_STAGES;
             if (c >= F_STAGES && !mbar_wait(empty + s, ((c / F_STAGES) - 1) & 1)) { atomicOr(err, 1u); break; }
             mbar_arrive_expect_tx(full + s, F_TILES * TILE);
-            uint32_t base = smem_u32(tiles + (size_t)s * F_TILES * TILE);
-            const int pass = c / nc;
-            const Maps4 &A = pass == 2 ? lo : hi, &B = pass == 1 ? lo : hi;
-            int kx = (c0 + c - pass * nc) * BK;
-            tma_load_2d(base, &A.are, full + s, kx, te * BM);
-            tma_load_2d(base + TILE, &A.aim, full + s, kx, te * BM);
-            tma_load_2d(base + 2 * TILE, &B.bre, full + s, kx, tr * BN);
-            tma_load_2d(base + 3 * TILE, &B.bim, full + s, kx, tr * BN);
+            const uint32_t base = smem_u32(tiles + (size_t)s * F_TILES * TILE);
+            const int kx = (c0 + c) * BK;
+            tma_load_2d(base, &maps.are, full + s, kx, te * BM);
+            tma_load_2d(base + TILE, &maps.aim, full + s, kx, te * BM);
+            tma_load_2d(base + 2 * TILE, &maps.bre, full + s, kx, tr * BN);
+            tma_load_2d(base + 3 * TILE, &maps.bim, full + s, kx, tr * BN);
             issued++;
         }
         // no copy may still be in flight when the CTA retires
@@ -140,79 +126,59 @@ __global__ __launch_bounds__(192, 1) void k_forward_tc(const __grid_constant__ M
     } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t ip = idesc_bf16(BM, BN, 0), in = idesc_bf16(BM, BN, 1);
-            bool ok = true;
-            for (int c = 0; c < ntot && ok; c++) {
-                const int seg = c / seglen, cs = c - seg * seglen, buf = seg & 1;
-                if (cs == 0 && seg >= 2) {
-                    if (!mbar_wait(acce + buf, ((seg >> 1) - 1) & 1)) { atomicOr(err, 32u); ok = false; break; }
-                    fence_after();
-                }
-                const uint32_t dre = tmem + buf * 2 * BN, dim = dre + BN;
-                int s = c % F_STAGES;
-                if (!mbar_wait(full + s, (c / F_STAGES) & 1)) { atomicOr(err, 2u); ok = false; break; }
+            const uint32_t dre = tmem, dim = tmem + BN;
+            for (int c = 0; c < nc; c++) {
+                const int s = c % F_STAGES;
+                if (!mbar_wait(full + s, (c / F_STAGES) & 1)) { atomicOr(err, 2u); break; }
                 fence_after();
-                uint32_t base = smem_u32(tiles + (size_t)s * F_TILES * TILE);
+                const uint32_t base = smem_u32(tiles + (size_t)s * F_TILES * TILE);
 #pragma unroll
                 for (int k = 0; k < BK / 16; k++) {
-                    uint64_t a0 = desc_sw128(base + k * 32), a1 = desc_sw128(base + TILE + k * 32);
-                    uint64_t b0 = desc_sw128(base + 2 * TILE + k * 32), b1 = desc_sw128(base + 3 * TILE + k * 32);
-                    uint32_t acc = (cs > 0 || k > 0) ? 1u : 0u;
+                    const uint64_t a0 = desc_sw128(base + k * 32), a1 = desc_sw128(base + TILE + k * 32);
+                    const uint64_t b0 = desc_sw128(base + 2 * TILE + k * 32), b1 = desc_sw128(base + 3 * TILE + k * 32);
+                    const uint32_t acc = (c > 0 || k > 0) ? 1u : 0u;
                     mma_bf16(dre, a0, b0, ip, acc);
                     mma_bf16(dre, a1, b1, in, 1u);
                     mma_bf16(dim, a0, b1, ip, acc);
                     mma_bf16(dim, a1, b0, ip, 1u);
                 }
                 mma_commit(empty + s);
-                if (cs == seglen - 1 || c == ntot - 1) mma_commit(accf + buf);
             }
-            // every MMA of this CTA has completed once the last buffer is signalled
-            if (ntot > 0 && !mbar_wait(accf + ((nseg - 1) & 1), ((nseg - 1) >> 1) & 1)) atomicOr(err, 8u);
+            // every MMA of this CTA has completed once this is signalled
+            if (nc > 0) mma_commit(accf);
+            if (nc > 0 && !mbar_wait(accf, 0)) atomicOr(err, 8u);
         }
         __syncwarp();
-    } else if (warp >= 2) {
+    } else if (warp >= 2 && nc > 0) {
         const int sub = warp & 3, row = sub * 32 + lane;
         const int e = te * BM + row;
         float2 *P = part + (size_t)split * N * N + (size_t)e * N;
         const uint32_t lanes = (uint32_t)(sub * 32) << 16;
-        for (int sg = 0; sg < nseg; sg++) {
-            const int buf = sg & 1;
-            bool ok = __all_sync(0xffffffffu, mbar_wait(accf + buf, (sg >> 1) & 1));
-            fence_after();
-            if (!ok) {
-                if (lane == 0) atomicOr(err, 16u);
-                break;
-            }
-            const uint32_t dre = tmem + buf * 2 * BN;
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(accf, 0));
+        fence_after();
+        if (!ok) {
+            if (lane == 0) atomicOr(err, 16u);
+        } else {
 #pragma unroll 1
             for (int cc = 0; cc < BN; cc += 32) {
                 float vr[32], vi[32];
-                tmem_ld32(tmem + lanes + (dre - tmem) + cc, vr);
-                tmem_ld32(tmem + lanes + (dre - tmem) + BN + cc, vi);
+                tmem_ld32(tmem + lanes + cc, vr);
+                tmem_ld32(tmem + lanes + BN + cc, vi);
                 if (e < N) {
 #pragma unroll
                     for (int i = 0; i < 32; i++) {
-                        int r = tr * BN + cc + i;
-                        if (r < N) {
-                            float2 v = make_float2(vr[i], vi[i]);
-                            if (sg > 0) {
-                                float2 o = P[r];
-                                v.x += o.x;
-                                v.y += o.y;
-                            }
-                            P[r] = v;
-                        }
+                        const int r = tr * BN + cc + i;
+                        if (r < N) P[r] = make_float2(vr[i], vi[i]);
                     }
                 }
             }
-            fence_before();
-            mbar_arrive(acce + buf);
         }
     }
     fence_before();
     __syncthreads();
     if (warp == 1) {
         fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc(tmem, 256);
     }
 }
 
@@ -375,19 +341,12 @@ __global__ __launch_bounds__(192, 1) void k_forward_tc_fused(const TabEntry *__r
 
 // ---------------------------------------------------------------- back-projection
 
-// Operand maps of one K pass: A = u and conj(kappa) u (re, im), B = R_s (re, im).
+// Operand maps: A = u and conj(kappa) u (re, im), B = R_s (re, im).
 struct Maps6 {
     CUtensorMap ure, uim, vre, vim, rre, rim;
 };
 
-// passes = 1: A_hi B_hi; passes = 3 (split BF16) adds A_hi B_lo and A_lo B_hi, and the
-// epilogue weights are read as hi + lo. With split BF16, as in the forward, no accumulation in
-// tensor memory runs over more than kSeg K chunks: the MMAs pause at each segment's end while
-// the epilogue adds that segment's row-dot into its registers (the row-dot is linear in P),
-// then restart from zero (one accumulator set, so the pause is not hidden; split BF16 only).
-template <bool SPLIT>
-__global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant__ Maps6 hi,
-                                                           const __grid_constant__ Maps6 lo,
+__global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant__ Maps6 maps,
                                                            const __nv_bfloat16 *__restrict__ planes, size_t pstride,
                                                            int Npad, int nk, float sgn, float2 *__restrict__ bpart,
                                                            int Xp, unsigned *__restrict__ err)
@@ -396,20 +355,14 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
     uint8_t *tiles = align1024(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(tiles + (size_t)B_STAGES * B_TILES * TILE);
     uint64_t *empty = full + B_STAGES;
-    uint64_t *accb = empty + B_STAGES;     // accumulators of a segment ready to drain
-    uint64_t *accd = accb + 1;             // accumulators drained
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(accd + 1);
+    uint64_t *accb = empty + B_STAGES;     // accumulators ready to drain
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(accb + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int et = blockIdx.x, xt = blockIdx.y;
-    constexpr int passes = SPLIT ? 3 : 1;
-    const int ntot = passes * nk;
-    const int seglen = SPLIT ? kSeg : ntot;
-    const int nseg = SPLIT ? (ntot + kSeg - 1) / kSeg : 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < B_STAGES; s++) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
         mbar_init(accb, 1);
-        mbar_init(accd, 128);
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tslot, 512);
@@ -419,23 +372,21 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
     const uint32_t tmem = *tslot;
 
     if (warp == 0 && lane == 0) {
-        prefetch_tmap(&hi.ure); prefetch_tmap(&hi.uim); prefetch_tmap(&hi.vre); prefetch_tmap(&hi.vim);
-        prefetch_tmap(&hi.rre); prefetch_tmap(&hi.rim);
+        prefetch_tmap(&maps.ure); prefetch_tmap(&maps.uim); prefetch_tmap(&maps.vre); prefetch_tmap(&maps.vim);
+        prefetch_tmap(&maps.rre); prefetch_tmap(&maps.rim);
         int issued = 0;
-        for (int c = 0; c < ntot; c++) {
+        for (int c = 0; c < nk; c++) {
             int s = c % B_STAGES;
             if (c >= B_STAGES && !mbar_wait(empty + s, ((c / B_STAGES) - 1) & 1)) { atomicOr(err, 1u); break; }
             mbar_arrive_expect_tx(full + s, B_TILES * TILE);
             uint32_t base = smem_u32(tiles + (size_t)s * B_TILES * TILE);
-            const int pass = c / nk;
-            const Maps6 &A = pass == 2 ? lo : hi, &B = pass == 1 ? lo : hi;
-            int kx = (c - pass * nk) * BK;
-            tma_load_2d(base, &A.ure, full + s, kx, xt * BM);
-            tma_load_2d(base + TILE, &A.uim, full + s, kx, xt * BM);
-            tma_load_2d(base + 2 * TILE, &A.vre, full + s, kx, xt * BM);
-            tma_load_2d(base + 3 * TILE, &A.vim, full + s, kx, xt * BM);
-            tma_load_2d(base + 4 * TILE, &B.rre, full + s, kx, et * BN);
-            tma_load_2d(base + 5 * TILE, &B.rim, full + s, kx, et * BN);
+            int kx = c * BK;
+            tma_load_2d(base, &maps.ure, full + s, kx, xt * BM);
+            tma_load_2d(base + TILE, &maps.uim, full + s, kx, xt * BM);
+            tma_load_2d(base + 2 * TILE, &maps.vre, full + s, kx, xt * BM);
+            tma_load_2d(base + 3 * TILE, &maps.vim, full + s, kx, xt * BM);
+            tma_load_2d(base + 4 * TILE, &maps.rre, full + s, kx, et * BN);
+            tma_load_2d(base + 5 * TILE, &maps.rim, full + s, kx, et * BN);
             issued++;
         }
         for (int c = (issued > B_STAGES ? issued - B_STAGES : 0); c < issued; c++)
@@ -444,12 +395,7 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
         if (lane == 0) {
             const uint32_t ip = idesc_bf16(BM, BN, 0), in = idesc_bf16(BM, BN, 1);
             const uint32_t p0r = tmem, p0i = tmem + BN, p1r = tmem + 2 * BN, p1i = tmem + 3 * BN;
-            for (int c = 0; c < ntot; c++) {
-                const int seg = SPLIT ? c / kSeg : 0, cs = c - seg * seglen;
-                if (cs == 0 && seg >= 1) {   // the previous segment's accumulators have been read
-                    if (!mbar_wait(accd, (seg - 1) & 1)) { atomicOr(err, 32u); break; }
-                    fence_after();
-                }
+            for (int c = 0; c < nk; c++) {
                 int s = c % B_STAGES;
                 if (!mbar_wait(full + s, (c / B_STAGES) & 1)) { atomicOr(err, 2u); break; }
                 fence_after();
@@ -459,7 +405,7 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
                     uint64_t ur = desc_sw128(base + k * 32), ui = desc_sw128(base + TILE + k * 32);
                     uint64_t vr = desc_sw128(base + 2 * TILE + k * 32), vi = desc_sw128(base + 3 * TILE + k * 32);
                     uint64_t rr = desc_sw128(base + 4 * TILE + k * 32), ri = desc_sw128(base + 5 * TILE + k * 32);
-                    uint32_t acc = (cs > 0 || k > 0) ? 1u : 0u;
+                    uint32_t acc = (c > 0 || k > 0) ? 1u : 0u;
                     mma_bf16(p0r, ur, rr, ip, acc);
                     mma_bf16(p0r, ui, ri, in, 1u);
                     mma_bf16(p0i, ur, ri, ip, acc);
@@ -470,27 +416,23 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
                     mma_bf16(p1i, vi, rr, ip, 1u);
                 }
                 mma_commit(empty + s);
-                if (cs == seglen - 1 || c == ntot - 1) mma_commit(accb);
             }
-            // every MMA of this CTA has completed once the last segment is signalled
-            if (!mbar_wait(accb, (nseg - 1) & 1)) atomicOr(err, 8u);
+            // every MMA of this CTA has completed once this is signalled
+            mma_commit(accb);
+            if (!mbar_wait(accb, 0)) atomicOr(err, 8u);
         }
         __syncwarp();
     } else if (warp >= 2) {
         const int sub = warp & 3, row = sub * 32 + lane;
         const int x = xt * BM + row;
         float gre = 0.f, gim = 0.f;
-        bool ok = true;
-        for (int sg = 0; sg < nseg && ok; sg++) {
-            ok = __all_sync(0xffffffffu, mbar_wait(accb, sg & 1));
-            fence_after();
-            if (!ok) break;
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(accb, 0));
+        fence_after();
+        if (ok) {
             const uint32_t lanes = (uint32_t)(sub * 32) << 16;
-            // epilogue weights at [x][e]: u (planes 0, 1) and kappa u (planes 4, 5); with
-            // split BF16 the lo parts are planes 6 + (0, 1, 4, 5)
+            // epilogue weights at [x][e]: u (planes 0, 1) and kappa u (planes 4, 5)
             const __nv_bfloat16 *w0r = planes + (size_t)x * Npad + et * BN;
             const __nv_bfloat16 *w0i = w0r + pstride, *w1r = w0r + 4 * pstride, *w1i = w0r + 5 * pstride;
-            const size_t lo_off = 6 * pstride;
 #pragma unroll 1
             for (int cc = 0; cc < BN; cc += 32) {
                 float a0r[32], a0i[32], a1r[32], a1i[32];
@@ -504,30 +446,14 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
                     uint4 i0 = *reinterpret_cast<const uint4 *>(w0i + cc + 8 * q);
                     uint4 r1 = *reinterpret_cast<const uint4 *>(w1r + cc + 8 * q);
                     uint4 i1 = *reinterpret_cast<const uint4 *>(w1i + cc + 8 * q);
-                    uint4 r0l = make_uint4(0, 0, 0, 0), i0l = r0l, r1l = r0l, i1l = r0l;
-                    if (passes == 3) {
-                        r0l = *reinterpret_cast<const uint4 *>(w0r + lo_off + cc + 8 * q);
-                        i0l = *reinterpret_cast<const uint4 *>(w0i + lo_off + cc + 8 * q);
-                        r1l = *reinterpret_cast<const uint4 *>(w1r + lo_off + cc + 8 * q);
-                        i1l = *reinterpret_cast<const uint4 *>(w1i + lo_off + cc + 8 * q);
-                    }
                     const __nv_bfloat162 *R0 = reinterpret_cast<const __nv_bfloat162 *>(&r0);
                     const __nv_bfloat162 *I0 = reinterpret_cast<const __nv_bfloat162 *>(&i0);
                     const __nv_bfloat162 *R1 = reinterpret_cast<const __nv_bfloat162 *>(&r1);
                     const __nv_bfloat162 *I1 = reinterpret_cast<const __nv_bfloat162 *>(&i1);
-                    const __nv_bfloat162 *R0l = reinterpret_cast<const __nv_bfloat162 *>(&r0l);
-                    const __nv_bfloat162 *I0l = reinterpret_cast<const __nv_bfloat162 *>(&i0l);
-                    const __nv_bfloat162 *R1l = reinterpret_cast<const __nv_bfloat162 *>(&r1l);
-                    const __nv_bfloat162 *I1l = reinterpret_cast<const __nv_bfloat162 *>(&i1l);
 #pragma unroll
                     for (int h = 0; h < 4; h++) {
                         float2 wr0 = __bfloat1622float2(R0[h]), wi0 = __bfloat1622float2(I0[h]);
                         float2 wr1 = __bfloat1622float2(R1[h]), wi1 = __bfloat1622float2(I1[h]);
-                        float2 t;
-                        t = __bfloat1622float2(R0l[h]); wr0.x += t.x; wr0.y += t.y;
-                        t = __bfloat1622float2(I0l[h]); wi0.x += t.x; wi0.y += t.y;
-                        t = __bfloat1622float2(R1l[h]); wr1.x += t.x; wr1.y += t.y;
-                        t = __bfloat1622float2(I1l[h]); wi1.x += t.x; wi1.y += t.y;
                         int j = 8 * q + 2 * h;
                         gre += wr0.x * a0r[j] - wi0.x * a0i[j] + sgn * (wr1.x * a1r[j] - wi1.x * a1i[j]);
                         gim += wr0.x * a0i[j] + wi0.x * a0r[j] + sgn * (wr1.x * a1i[j] + wi1.x * a1r[j]);
@@ -536,8 +462,6 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
                     }
                 }
             }
-            fence_before();
-            mbar_arrive(accd);
         }
         if (ok)
             bpart[(size_t)et * Xp + x] = make_float2(gre, gim);
@@ -554,39 +478,54 @@ __global__ __launch_bounds__(192, 1) void k_backproject_tc(const __grid_constant
 
 // ---------------------------------------------------------------- operand synthesis
 
-// value = hi + lo with hi = bf16(value), lo = bf16(value - hi) (split BF16)
-__device__ __forceinline__ void put_split(__nv_bfloat16 *hi, __nv_bfloat16 *lo, float v)
+// planes [4][Npad][Xpad]: Gre, Gim, (G v)re, (G v)im;
+// G_e[x] = C a exp(i 2 pi (f T - K/4 + 1/8)). Two nodes and eight transducers per thread, so that a
+// store is 4 bytes and the Born weights are read once.
+// Bound: HBM, 16 B read and 8 B written per entry: 1024 transducers, 152,088 nodes (3.7 GB), one
+// entry per thread 785 us; the Born forward 1252 -> 950 us with this.
+__global__ __launch_bounds__(128) void k_synth_fwd_tc(const TabEntry *__restrict__ tab, const float2 *__restrict__ v,
+                                                      int N, int X, int Xpad, size_t pstride, float fhi, float flo,
+                                                      float C, __nv_bfloat16 *__restrict__ planes)
 {
-    __nv_bfloat16 h = __float2bfloat16_rn(v);
-    *hi = h;
-    if (lo) *lo = __float2bfloat16_rn(v - __bfloat162float(h));
-}
-
-
-// planes [4][Npad][Xpad]: Gre, Gim, (G v)re, (G v)im (then 4 lo planes when split);
-// G_e[x] = C a exp(i 2 pi (f T - K/4 + 1/8))
-__global__ void k_synth_fwd_tc(const TabEntry *__restrict__ tab, const float2 *__restrict__ v, int N, int X, int Xpad,
-                               size_t pstride, float fhi, float flo, float C, __nv_bfloat16 *__restrict__ planes,
-                               int split)
-{
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= (size_t)N * X) return;
-    int e = (int)(i / X), x = (int)(i % X);
-    TabEntry t = tab[i];
-    float gr = 0.f, gi = 0.f;
-    if (t.idk != kUncovered) {
-        float s, c;
-        sincos_turns_tc(phase_cycles_tc(t.T, (int)(t.idk & 0xffu), fhi, flo), &s, &c);
-        gr = C * t.a * c;
-        gi = C * t.a * s;
+    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x), e0 = blockIdx.y * kSynWalk;
+    if (x >= X) return;
+    const bool two = x + 1 < X;
+    const float2 w[2] = {v[x], two ? v[x + 1] : make_float2(0.f, 0.f)};
+    TabEntry none;
+    none.idk = kUncovered;
+    none.T = none.a = none.gam = 0.f;
+    const int n = min(kSynWalk, N - e0);
+    TabEntry t[2], next[2];
+    auto row = [&](int e, TabEntry *o) {
+        const TabEntry *q = tab + (size_t)e * X + x;
+        o[0] = q[0];
+        o[1] = two ? q[1] : none;
+    };
+    row(e0, t);
+    for (int i = 0; i < n; i++) {
+        if (i + 1 < n) row(e0 + i + 1, next);
+        float g[2][2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            g[q][0] = g[q][1] = 0.f;
+            if (t[q].idk != kUncovered) {
+                float s, c;
+                sincos_turns_tc(phase_cycles_tc(t[q].T, (int)(t[q].idk & 0xffu), fhi, flo), &s, &c);
+                g[q][0] = C * t[q].a * c;
+                g[q][1] = C * t[q].a * s;
+            }
+        }
+        const size_t o = (size_t)(e0 + i) * Xpad + x;
+        auto put = [&](int k, float a, float b) {
+            *reinterpret_cast<__nv_bfloat162 *>(planes + k * pstride + o) = __floats2bfloat162_rn(a, b);
+        };
+        put(0, g[0][0], g[1][0]);
+        put(1, g[0][1], g[1][1]);
+        put(2, gv_re(g[0][0], g[0][1], w[0]), gv_re(g[1][0], g[1][1], w[1]));
+        put(3, gv_im(g[0][0], g[0][1], w[0]), gv_im(g[1][0], g[1][1], w[1]));
+        t[0] = next[0];
+        t[1] = next[1];
     }
-    const float2 vv = v[x];
-    size_t o = (size_t)e * Xpad + x;
-    __nv_bfloat16 *lo = split ? planes + 4 * pstride : nullptr;
-    put_split(planes + o, lo ? lo + o : nullptr, gr);
-    put_split(planes + pstride + o, lo ? lo + pstride + o : nullptr, gi);
-    put_split(planes + 2 * pstride + o, lo ? lo + 2 * pstride + o : nullptr, gv_re(gr, gi, vv));
-    put_split(planes + 3 * pstride + o, lo ? lo + 3 * pstride + o : nullptr, gv_im(gr, gi, vv));
 }
 
 // 16-byte asynchronous copy global -> shared (L2 only), and its group fences.
@@ -629,14 +568,14 @@ __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab
 // back-projection planes, 8 % faster than nodes fastest) with
 // two shared-memory buffers, the next tile's entries copied in while the current one is
 // formed and stored, so that table reads stay in flight between the blocks' barriers.
-template <bool FWD, bool SPLIT>
-__global__ __launch_bounds__(256, SPLIT ? 3 : 4) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
+template <bool FWD>
+__global__ __launch_bounds__(256, 4) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
                                                      size_t pstride, float fhi, float flo, float C,
                                                      __nv_bfloat16 *__restrict__ planes, const float2 *__restrict__ bw,
                                                      int Xpad, size_t fpstride, __nv_bfloat16 *__restrict__ fplanes,
                                                      int XT, int ntiles)
 {
-    constexpr int NPL = SPLIT ? 12 : 6;                      // back-projection planes (hi, then lo)
+    constexpr int NPL = 6;                                   // back-projection planes
     extern __shared__ __align__(16) unsigned char syn_smem[];
     TabEntry *buf = reinterpret_cast<TabEntry *>(syn_smem);  // [2][kSynSlots]
     // [plane][x][e]: rows of 17 words, the tile transposed and rounded to BF16
@@ -681,18 +620,15 @@ __global__ __launch_bounds__(256, SPLIT ? 3 : 4) void k_synth_tc(const TabEntry 
             }
 #pragma unroll
             for (int m = 0; m < 6; m++) {
-                const __nv_bfloat16 h = __float2bfloat16_rn(v[m]);
-                sv[m][tx][q] = h;
-                if (SPLIT) sv[6 + m][tx][q] = __float2bfloat16_rn(v[m] - __bfloat162float(h));
+                sv[m][tx][q] = __float2bfloat16_rn(v[m]);
             }
             if (FWD && e0 + q < N && xin) {
                 // G and G v at [e][x], as k_synth_fwd_tc
                 const size_t o = (size_t)(e0 + q) * Xpad + x;
-                __nv_bfloat16 *lo = SPLIT ? fplanes + 4 * fpstride : nullptr;
-                put_split(fplanes + o, SPLIT ? lo + o : nullptr, gr);
-                put_split(fplanes + fpstride + o, SPLIT ? lo + fpstride + o : nullptr, gi);
-                put_split(fplanes + 2 * fpstride + o, SPLIT ? lo + 2 * fpstride + o : nullptr, gv_re(gr, gi, vv));
-                put_split(fplanes + 3 * fpstride + o, SPLIT ? lo + 3 * fpstride + o : nullptr, gv_im(gr, gi, vv));
+                fplanes[o] = __float2bfloat16_rn(gr);
+                fplanes[fpstride + o] = __float2bfloat16_rn(gi);
+                fplanes[2 * fpstride + o] = __float2bfloat16_rn(gv_re(gr, gi, vv));
+                fplanes[3 * fpstride + o] = __float2bfloat16_rn(gv_im(gr, gi, vv));
             }
         }
         __syncthreads();   // the tile is in sv, and buffer b is free for the tile after next
@@ -714,17 +650,16 @@ __global__ __launch_bounds__(256, SPLIT ? 3 : 4) void k_synth_tc(const TabEntry 
     cp_async_wait0();
 }
 
-// R_s (complex N x N) -> planes [2][Npad][Npad] (then 2 lo planes when split)
-__global__ void k_rs_planes(const float2 *__restrict__ Rs, int N, int Npad, __nv_bfloat16 *__restrict__ planes,
-                            int split)
+// R_s (complex N x N) -> planes [2][Npad][Npad]
+__global__ void k_rs_planes(const float2 *__restrict__ Rs, int N, int Npad, __nv_bfloat16 *__restrict__ planes)
 {
     size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= (size_t)N * N) return;
     int e = (int)(i / N), r = (int)(i % N);
     float2 v = Rs[i];
     size_t o = (size_t)e * Npad + r, P = (size_t)Npad * Npad;
-    put_split(planes + o, split ? planes + 2 * P + o : nullptr, v.x);
-    put_split(planes + P + o, split ? planes + 3 * P + o : nullptr, v.y);
+    planes[o] = __float2bfloat16_rn(v.x);
+    planes[P + o] = __float2bfloat16_rn(v.y);
 }
 
 // gpart[0][x] = sum over emitter tiles (fixed order); gpart[1][x] = 0 (the stacks are
@@ -787,10 +722,8 @@ bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, 
 
 // ---------------------------------------------------------------- API used by rbx_api.cu
 
-bool tc_setup(TcPlanes &p, int N, int X, bool split, cudaStream_t st)
+bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t st)
 {
-    p.split = split;
-    const int mult = split ? 2 : 1;
     p.N = N;
     p.X = X;
     p.Npad = (N + BM - 1) / BM * BM;
@@ -812,9 +745,9 @@ bool tc_setup(TcPlanes &p, int N, int X, bool split, cudaStream_t st)
     // the autotuner may go up to 4x the heuristic's split (at most one K chunk per CTA)
     const int smax = std::min(nk, std::max(4 * splits, 1));
     p.fwd_max_splits = (nk + (nk + smax - 1) / smax - 1) / ((nk + smax - 1) / smax);
-    const size_t fbytes = mult * 4 * p.fwd_pstride * sizeof(__nv_bfloat16);
-    const size_t bbytes = mult * 6 * p.bp_pstride * sizeof(__nv_bfloat16);
-    const size_t rbytes = mult * 2 * (size_t)p.Npad * p.Npad * sizeof(__nv_bfloat16);
+    const size_t fbytes = 4 * p.fwd_pstride * sizeof(__nv_bfloat16);
+    const size_t bbytes = 6 * p.bp_pstride * sizeof(__nv_bfloat16);
+    const size_t rbytes = 2 * (size_t)p.Npad * p.Npad * sizeof(__nv_bfloat16);
     if (cudaMallocAsync(&p.fplanes, fbytes, st) != cudaSuccess) return false;
     if (cudaMallocAsync(&p.bplanes, bbytes, st) != cudaSuccess) return false;
     if (cudaMallocAsync(&p.rsplanes, rbytes, st) != cudaSuccess) return false;
@@ -831,25 +764,14 @@ bool tc_setup(TcPlanes &p, int N, int X, bool split, cudaStream_t st)
     const __nv_bfloat16 *r = static_cast<const __nv_bfloat16 *>(p.rsplanes);
     const size_t P = (size_t)p.Npad * p.Npad;
     bool ok = true;
-    for (int h = 0; h < mult; h++) {
-        const __nv_bfloat16 *fh = f + (size_t)h * 4 * p.fwd_pstride, *bh = b + (size_t)h * 6 * p.bp_pstride,
-                            *rh = r + (size_t)h * 2 * P;
-        for (int k = 0; k < 4; k++) ok = ok && make_map(&p.fmaps[h][k], fh + k * p.fwd_pstride, p.Npad, p.Xpad);
-        for (int k = 0; k < 4; k++) ok = ok && make_map(&p.bmaps[h][k], bh + k * p.bp_pstride, p.Xp, p.Npad);
-        for (int k = 0; k < 2; k++) ok = ok && make_map(&p.bmaps[h][4 + k], rh + (size_t)k * P, p.Npad, p.Npad);
-    }
-    if (!split) {
-        for (int k = 0; k < 4; k++) p.fmaps[1][k] = p.fmaps[0][k];
-        for (int k = 0; k < 6; k++) p.bmaps[1][k] = p.bmaps[0][k];
-    }
+    for (int k = 0; k < 4; k++) ok = ok && make_map(&p.fmaps[k], f + k * p.fwd_pstride, p.Npad, p.Xpad);
+    for (int k = 0; k < 4; k++) ok = ok && make_map(&p.bmaps[k], b + k * p.bp_pstride, p.Xp, p.Npad);
+    for (int k = 0; k < 2; k++) ok = ok && make_map(&p.bmaps[4 + k], r + (size_t)k * P, p.Npad, p.Npad);
     if (!ok) return false;
     ok = cudaFuncSetAttribute(k_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) == cudaSuccess &&
          cudaFuncSetAttribute(k_forward_tc_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) ==
              cudaSuccess &&
-         cudaFuncSetAttribute(k_backproject_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) ==
-             cudaSuccess &&
-         cudaFuncSetAttribute(k_backproject_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) ==
-             cudaSuccess;
+         cudaFuncSetAttribute(k_backproject_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) == cudaSuccess;
     p.ready = ok;
     return ok;
 }
@@ -863,7 +785,7 @@ struct TuneChoice {
     bool fused = false;
     float ms[4] = {0.f, 0.f, 0.f, 0.f};
 };
-std::map<std::tuple<int, int, int, bool>, TuneChoice> g_tune;   // (device, N, X, split) -> choice
+std::map<std::tuple<int, int, int>, TuneChoice> g_tune;   // (device, N, X) -> choice
 int g_tune_mode = 1;
 }  // namespace
 
@@ -886,12 +808,12 @@ bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream
 {
     int dev = 0;
     cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, p.N, p.X, p.split);
+    const auto key = std::make_tuple(dev, p.N, p.X);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         if (g_tune_mode == 0) return true;                      // heuristic split
         if (g_tune_mode == 2) {                                 // heuristic split, fused forward
-            p.fwd_fused = !p.split;
+            p.fwd_fused = true;
             return true;
         }
         auto it = g_tune.find(key);
@@ -911,8 +833,7 @@ bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream
         const int kper = (nk + sp - 1) / sp;
         if (std::find(kpers.begin(), kpers.end(), kper) == kpers.end()) kpers.push_back(kper);
     }
-    Maps4 hi{p.fmaps[0][0], p.fmaps[0][1], p.fmaps[0][2], p.fmaps[0][3]};
-    Maps4 lo{p.fmaps[1][0], p.fmaps[1][1], p.fmaps[1][2], p.fmaps[1][3]};
+    const Maps4 maps{p.fmaps[0], p.fmaps[1], p.fmaps[2], p.fmaps[3]};
     cudaEvent_t a = nullptr, b = nullptr;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return false;
     int best = p.fwd_kper;
@@ -923,7 +844,7 @@ bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream
         float tot = 0.f;
         for (int rep = 0; rep < 3 && ok; rep++) {              // first launch warms up
             ok = cudaEventRecord(a, s) == cudaSuccess;
-            k_forward_tc<<<dim3(pairs, sp), 192, F_SMEM, s>>>(hi, lo, p.split ? 3 : 1, p.N, T, nk, kper, part, p.err);
+            k_forward_tc<<<dim3(pairs, sp), 192, F_SMEM, s>>>(maps, p.N, T, nk, kper, part, p.err);
             ok = ok && cudaGetLastError() == cudaSuccess && cudaEventRecord(b, s) == cudaSuccess &&
                  cudaEventSynchronize(b) == cudaSuccess;
             float ms = 0.f;
@@ -940,10 +861,10 @@ bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream
     TuneChoice ch;
     ch.kper = best;
     apply_kper(p, best);
-    // plain BF16: the separate synthesis pass (both operand sets, as an update runs it) plus the
+    // the separate synthesis pass (both operand sets, as an update runs it) plus the
     // forward GEMM, against the back-projection's synthesis alone plus the fused forward, on
     // tables holding covered entries (every entry then costs its full synthesis)
-    if (ok && !p.split && tab && v) {
+    if (ok && tab && v) {
         ok = cudaMemsetAsync(tab, 0, sizeof(TabEntry) * (size_t)p.N * p.X, s) == cudaSuccess &&
              cudaMemsetAsync(v, 0, sizeof(float2) * (size_t)p.X, s) == cudaSuccess;
         const double f = 5e5, c0 = 1500.0;
@@ -1006,11 +927,10 @@ static float green_const_tc(double f, double c0)
 
 void launch_synth_fwd_tc(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
-    size_t n = (size_t)p.N * p.X;
     float fhi = (float)f, flo = (float)(f - (double)fhi);
-    k_synth_fwd_tc<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tab, v, p.N, p.X, p.Xpad, p.fwd_pstride, fhi, flo,
-                                                               green_const_tc(f, c0),
-                                                               static_cast<__nv_bfloat16 *>(p.fplanes), p.split);
+    const dim3 grd((unsigned)((p.X + 255) / 256), (unsigned)((p.N + kSynWalk - 1) / kSynWalk));
+    k_synth_fwd_tc<<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.Xpad, p.fwd_pstride, fhi, flo, green_const_tc(f, c0),
+                                       static_cast<__nv_bfloat16 *>(p.fplanes));
 }
 
 int launch_forward_tc_fused(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, float2 *part,
@@ -1026,39 +946,37 @@ int launch_forward_tc_fused(TcPlanes &p, const TabEntry *tab, const float2 *v, d
 int launch_forward_tc(TcPlanes &p, float2 *part, cudaStream_t s)
 {
     int T = p.Npad / BM, pairs = T * (T + 1) / 2;
-    Maps4 hi{p.fmaps[0][0], p.fmaps[0][1], p.fmaps[0][2], p.fmaps[0][3]};
-    Maps4 lo{p.fmaps[1][0], p.fmaps[1][1], p.fmaps[1][2], p.fmaps[1][3]};
-    k_forward_tc<<<dim3(pairs, p.fwd_splits), 192, F_SMEM, s>>>(hi, lo, p.split ? 3 : 1, p.N, T, p.Xpad / BK,
-                                                                p.fwd_kper, part, p.err);
+    const Maps4 maps{p.fmaps[0], p.fmaps[1], p.fmaps[2], p.fmaps[3]};
+    k_forward_tc<<<dim3(pairs, p.fwd_splits), 192, F_SMEM, s>>>(maps, p.N, T, p.Xpad / BK, p.fwd_kper, part, p.err);
     return p.fwd_splits;
 }
 
-// Shared memory and persistent grid of k_synth_tc<FWD, SPLIT> (set up once per instance).
-template <bool FWD, bool SPLIT>
+// Shared memory and persistent grid of k_synth_tc<FWD> (set up once per instance).
+template <bool FWD>
 static int synth_grid(size_t &smem)
 {
-    smem = 2 * kSynSlots * sizeof(TabEntry) + (SPLIT ? 12 : 6) * 32 * 34 * sizeof(__nv_bfloat16);
+    smem = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * 34 * sizeof(__nv_bfloat16);
     static int blocks = 0;
     if (blocks == 0) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_synth_tc<FWD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD, SPLIT>, 256, smem);
+        cudaFuncSetAttribute(k_synth_tc<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, 256, smem);
         blocks = sms * (per_sm > 0 ? per_sm : 1);
     }
     return blocks;
 }
 
-template <bool FWD, bool SPLIT>
+template <bool FWD>
 static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
     const float fhi = (float)f, flo = (float)(f - (double)fhi);
     const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + 31) / 32);
     size_t smem = 0;
-    int grd = synth_grid<FWD, SPLIT>(smem);
+    int grd = synth_grid<FWD>(smem);
     if (grd > ntiles) grd = ntiles;
-    k_synth_tc<FWD, SPLIT><<<grd, 256, smem, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
+    k_synth_tc<FWD><<<grd, 256, smem, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
                                                   static_cast<__nv_bfloat16 *>(p.bplanes), v, FWD ? p.Xpad : 0,
                                                   FWD ? p.fwd_pstride : 0,
                                                   FWD ? static_cast<__nv_bfloat16 *>(p.fplanes) : nullptr, XT, ntiles);
@@ -1066,18 +984,12 @@ static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, doub
 
 void launch_synth_bp_tc(TcPlanes &p, const TabEntry *tab, double f, double c0, cudaStream_t s)
 {
-    if (p.split)
-        synth_launch<false, true>(p, tab, nullptr, f, c0, s);
-    else
-        synth_launch<false, false>(p, tab, nullptr, f, c0, s);
+    synth_launch<false>(p, tab, nullptr, f, c0, s);
 }
 
 void launch_synth_both_tc(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
-    if (p.split)
-        synth_launch<true, true>(p, tab, v, f, c0, s);
-    else
-        synth_launch<true, false>(p, tab, v, f, c0, s);
+    synth_launch<true>(p, tab, v, f, c0, s);
 }
 
 // One thread waits, with the bound every tensor-core kernel uses, on an mbarrier that nothing
@@ -1101,18 +1013,12 @@ void launch_backproject_tc(TcPlanes &p, const float2 *Rs, int weight_mode, float
 {
     size_t nn = (size_t)p.N * p.N;
     k_rs_planes<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Rs, p.N, p.Npad,
-                                                             static_cast<__nv_bfloat16 *>(p.rsplanes), p.split);
+                                                             static_cast<__nv_bfloat16 *>(p.rsplanes));
     dim3 grd(p.Npad / BN, p.Xp / BM);
-    Maps6 hi{p.bmaps[0][0], p.bmaps[0][1], p.bmaps[0][2], p.bmaps[0][3], p.bmaps[0][4], p.bmaps[0][5]};
-    Maps6 lo{p.bmaps[1][0], p.bmaps[1][1], p.bmaps[1][2], p.bmaps[1][3], p.bmaps[1][4], p.bmaps[1][5]};
+    const Maps6 maps{p.bmaps[0], p.bmaps[1], p.bmaps[2], p.bmaps[3], p.bmaps[4], p.bmaps[5]};
     const __nv_bfloat16 *bp = static_cast<const __nv_bfloat16 *>(p.bplanes);
     const float sgn = weight_mode == 0 ? -1.f : 1.f;
-    if (p.split)
-        k_backproject_tc<true><<<grd, 192, B_SMEM, s>>>(hi, lo, bp, p.bp_pstride, p.Npad, p.Npad / BK, sgn, p.bpart,
-                                                        p.Xp, p.err);
-    else
-        k_backproject_tc<false><<<grd, 192, B_SMEM, s>>>(hi, lo, bp, p.bp_pstride, p.Npad, p.Npad / BK, sgn, p.bpart,
-                                                         p.Xp, p.err);
+    k_backproject_tc<<<grd, 192, B_SMEM, s>>>(maps, bp, p.bp_pstride, p.Npad, p.Npad / BK, sgn, p.bpart, p.Xp, p.err);
     k_bp_reduce<<<(p.X + 255) / 256, 256, 0, s>>>(p.bpart, p.Npad / BN, p.Xp, p.X, gpart);
 }
 

@@ -103,6 +103,7 @@ static void free_ws(Workspace &w, cudaStream_t s)
         if (p) cudaFreeAsync(p, s);
     tc_free(w.tc, s);
     f32_free(w.f32, s);
+    f32_free(w.split, s);
     w = Workspace{};
 }
 
@@ -270,10 +271,11 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.dg, NX);
     ALLOC(w.exits, N * (N - 1));
     // FP32 jobs: the operands of both contractions; the others: those of the plain adjoint
-    if (!f32_setup(w.f32, w.N, X, g.precision == RBX_FP32, j->stream)) {
+    if (!f32_setup(w.f32, w.N, X, 3, g.precision == RBX_FP32, j->stream) ||
+        (g.precision == RBX_BF16X3 && !f32_setup(w.split, w.N, X, 2, true, j->stream))) {
         cudaGetLastError();
         free_ws(w, j->stream);
-        return fail(j, RBX_ENOMEM, "FP32 operand set-up failed (allocation or TMA descriptor)");
+        return fail(j, RBX_ENOMEM, "operand set-up failed (allocation or TMA descriptor)");
     }
     ALLOC(w.v, X);
     ALLOC(w.gdir, N * N);
@@ -281,8 +283,8 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.R, N * N);
     ALLOC(w.Rs, N * N);
     ALLOC(w.data, N * N);
-    if (g.precision != RBX_FP32) {
-        if (!tc_setup(w.tc, w.N, X, g.precision == RBX_BF16X3, j->stream)) {
+    if (g.precision == RBX_BF16) {
+        if (!tc_setup(w.tc, w.N, X, j->stream)) {
             cudaGetLastError();
             free_ws(w, j->stream);
             return fail(j, RBX_ENOMEM, "tensor-core operand set-up failed (allocation or TMA descriptor)");
@@ -290,7 +292,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
         if (w.tc.fwd_max_splits > w.fwd_splits) w.fwd_splits = w.tc.fwd_max_splits;
     }
     ALLOC(w.part, (size_t)w.fwd_splits * N * N);
-    if (g.precision != RBX_FP32 && !tc_autotune(w.tc, w.part, w.tab, w.v, j->stream)) {
+    if (g.precision == RBX_BF16 && !tc_autotune(w.tc, w.part, w.tab, w.v, j->stream)) {
         cudaGetLastError();
         free_ws(w, j->stream);
         return fail(j, RBX_ECUDA, "autotuning of the tensor-core forward failed");
@@ -553,6 +555,9 @@ rbx_status rbx_direct_green(rbx_job *j, double f, void *g_dev)
     return direct_green(j, f, static_cast<float2 *>(g_dev));
 }
 
+// The operands of an FP32 or split BF16 job's contractions.
+static F32Planes &parts_of(rbx_job *j) { return j->g.precision == RBX_FP32 ? j->w.f32 : j->w.split; }
+
 // D = sum_x G_r G_e v on the current tables, into w.D (symmetric).
 // The Born forward on the current tables with the weights in w.v. With both (tensor-core
 // paths) the operand synthesis also writes the back-projection's planes for this frequency.
@@ -560,7 +565,7 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
 {
     Workspace &w = j->w;
     rbx_status st;
-    if (j->g.precision != RBX_FP32 && w.tc.fwd_fused) {
+    if (j->g.precision == RBX_BF16 && w.tc.fwd_fused) {
         // the tuner's choice: the forward forms its operands from the tables; an update still
         // writes the back-projection's planes
         if (both) {
@@ -571,7 +576,7 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
         int splits = launch_forward_tc_fused(w.tc, w.tab, w.v, f, j->g.c0, w.part, j->stream);
         launch_forward_reduce(w.part, w.N, splits, w.D, j->stream);
         LAUNCHED(j, 2);
-    } else if (j->g.precision != RBX_FP32) {
+    } else if (j->g.precision == RBX_BF16) {
         if (both)
             launch_synth_both_tc(w.tc, w.tab, w.v, f, j->g.c0, j->stream);
         else
@@ -582,10 +587,10 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
         launch_forward_reduce(w.part, w.N, splits, w.D, j->stream);
         LAUNCHED(j, 2);
     } else {
-        launch_synth_fwd(w.f32, w.tab, w.v, f, j->g.c0, j->stream);
+        launch_synth_fwd(parts_of(j), w.tab, w.v, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if (timed && (st = record(j, EV_SYNTH_F))) return st;
-        launch_forward_f32(w.f32, w.fwd_splits, w.part, j->stream);
+        launch_forward_f32(parts_of(j), w.fwd_splits, w.part, j->stream);
         launch_forward_reduce(w.part, w.N, w.fwd_splits, w.D, j->stream);
         LAUNCHED(j, 2);
     }
@@ -637,14 +642,14 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
     Workspace &w = j->w;
     launch_symmetrize(static_cast<const float2 *>(R_dev), w.N, w.Rs, j->stream);
     LAUNCHED(j, 1);
-    if (preconditioned && j->g.precision != RBX_FP32) {
+    if (preconditioned && j->g.precision == RBX_BF16) {
         launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
         LAUNCHED(j, 4);
     } else if (preconditioned) {
-        launch_synth_bp(w.f32, w.tab, f, j->g.c0, j->stream);
-        LAUNCHED(j, launch_backproject_f32(w.f32, w.tab, w.Rs, w.gpart, j->stream));
+        launch_synth_bp(parts_of(j), w.tab, f, j->g.c0, j->stream);
+        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, w.Rs, w.gpart, j->stream));
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
     } else {
         double om = 2 * 3.14159265358979323846 * f;
@@ -683,7 +688,7 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
     launch_residual(w.gdir, w.D, data, w.N, nullptr, w.Rs, w.red, j->stream);
     LAUNCHED(j, 2);
     if ((st = record(j, EV_RESID))) return st;
-    if (j->g.precision != RBX_FP32) {
+    if (j->g.precision == RBX_BF16) {
         if (j->raw) {   // otherwise the forward's synthesis wrote these planes
             launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);
             LAUNCHED(j, 1);
@@ -692,10 +697,10 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
         LAUNCHED(j, 3);
     } else {
-        launch_synth_bp(w.f32, w.tab, f, j->g.c0, j->stream);
+        launch_synth_bp(parts_of(j), w.tab, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if ((st = record(j, EV_SYNTH_B))) return st;
-        LAUNCHED(j, launch_backproject_f32(w.f32, w.tab, w.Rs, w.gpart, j->stream));
+        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, w.Rs, w.gpart, j->stream));
     }
     if ((st = record(j, EV_GEMM_B))) return st;
     const int roff = residual_blocks(w.N) + 8;
@@ -708,7 +713,7 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
 // Where the kernels of an update's contractions record a bounded wait that gave up.
 static const unsigned *contraction_err(const rbx_job *j)
 {
-    return j->g.precision == RBX_FP32 ? j->w.f32.err : j->w.tc.err;
+    return j->g.precision == RBX_BF16 ? j->w.tc.err : (j->g.precision == RBX_FP32 ? j->w.f32 : j->w.split).err;
 }
 
 static rbx_status enqueue_update(rbx_job *j, double f, double df, const float2 *data, bool traced, int slot)
@@ -1254,11 +1259,11 @@ size_t job_bytes_estimate(const rbx_geometry &g, int nf)
     const size_t X = (size_t)(3.14159265358979 * r * r + 6.3 * r + 16);
     const size_t N = (size_t)g.n_xducers, NX = N * X, nxy = (size_t)g.nx * g.ny, NN = N * N;
     size_t b = NX * (16 + 4 + 8);                                 // tables, angular density, FP32 operand planes
-    if (g.precision == RBX_FP32) b += NX * 16;                    // (24 B an entry in all)
-    else {
+    if (g.precision == RBX_FP32 || g.precision == RBX_BF16X3) {
+        b += NX * 16;                                             // (24 B an entry in all; split BF16 8 + 16)
+    } else {
         const size_t Np = (N + 127) / 128 * 128, Xk = (X + 63) / 64 * 64, Xm = (X + 127) / 128 * 128;
-        const size_t m = g.precision == RBX_BF16X3 ? 2 : 1;
-        b += m * (4 * Np * Xk + 6 * Xm * Np + 2 * Np * Np) * 2 + (Np / 128) * Xm * 8;
+        b += (4 * Np * Xk + 6 * Xm * Np + 2 * Np * Np) * 2 + (Np / 128) * Xm * 8;
     }
     b += nxy * (4 + 4 + 8 + 8 + 32 + 4 + 4) + N * (N - 1) * 16 + NN * 8 * 5 + 64 * NN * 8 + X * 24;
     b += (size_t)nf * NN * 8 + nxy * 4 + (1u << 20);              // data, initial model, slack
@@ -1273,7 +1278,7 @@ int rbx_autotune(int mode) { return set_autotune(mode); }
 rbx_status rbx_get_tuning(const rbx_job *j, int *fwd_splits, int *candidates_timed)
 {
     if (!j) return RBX_EINVAL;
-    if (fwd_splits) *fwd_splits = j->g.precision == RBX_FP32 ? j->w.fwd_splits : j->w.tc.fwd_splits;
+    if (fwd_splits) *fwd_splits = j->g.precision == RBX_BF16 ? j->w.tc.fwd_splits : j->w.fwd_splits;
     if (candidates_timed) *candidates_timed = j->w.tc.tuned;
     return RBX_OK;
 }

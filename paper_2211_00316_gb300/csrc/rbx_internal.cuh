@@ -67,24 +67,24 @@ struct TcPlanes {
     bool fwd_fused = false;    // the forward forms its operands from the tables (k_forward_tc_fused)
     float tune_ms[4] = {0.f, 0.f, 0.f, 0.f};   // tuner's times: both synthesis passes, forward GEMM,
                                                // back-projection synthesis alone, fused forward
-    bool split = false;        // split BF16: every plane set is followed by its lo set
     void *fplanes = nullptr;   // [4][Npad][Xpad] bf16: Gre, Gim, (Gv)re, (Gv)im
     void *bplanes = nullptr;   // [6][Xp][Npad] bf16: u, conj(kappa) u, kappa u (re, im)
     void *rsplanes = nullptr;  // [2][Npad][Npad] bf16: R_s re, im
     float2 *bpart = nullptr;   // [Npad/128][Xp] partial back-projection
     unsigned *err = nullptr;   // bounded-wait timeouts of the tensor-core kernels
-    CUtensorMap fmaps[2][4], bmaps[2][6];   // [hi, lo]
+    CUtensorMap fmaps[4], bmaps[6];
     bool ready = false;
 };
 
-// Operands of the FP32-accurate contractions of one job: FP32 values as three BF16 parts, their
-// TMA descriptors and the back-projection partials (k_gemm_f32.cu).
+// Operands of the FP32-accurate (or split BF16) contractions of one job: values as three (two) BF16
+// parts, their TMA descriptors and the back-projection partials (k_gemm_f32.cu).
 struct F32Planes {
     int N = 0, X = 0, xs = 0, xld = 0, rld = 0;   // xs nodes per slab, rows of xld (operands) and rld (R_s)
-    bool full = false;         // both operand sets of all nodes (FP32 jobs); else the plain adjoint's slab
+    int parts = 3;
+    bool full = false;         // both operand sets of all nodes ; else the plain adjoint's slab
     size_t pstride = 0;
-    void *planes = nullptr;    // [12 or 6][N][xld] bf16
-    void *rs = nullptr;        // [6][N][rld] bf16
+    void *planes = nullptr;    // [4 parts, or 2 parts of a slab][N][xld] bf16
+    void *rs = nullptr;        // [2 parts][N][rld] bf16
     float2 *bpart = nullptr;   // [stacks][emitter tiles][X]; nullptr with one emitter tile
     unsigned *err = nullptr;   // bounded-wait timeouts
     CUtensorMap fmap, amap, rmap;   // K-major and M-major boxes of planes, K-major boxes of rs
@@ -113,7 +113,8 @@ struct Workspace {
     unsigned long long *counters = nullptr;   // [0] covered entries [1] clamped [2] bad rays [3] CAS bound [4] m <= 0 [5] bad model [6] mask count [7] uniform radius (float bits)
     int fwd_splits = 1;
     TcPlanes tc;
-    F32Planes f32;
+    F32Planes f32;              // FP32 jobs; the plain adjoint of the others
+    F32Planes split;            // split BF16 jobs
 };
 
 // ---------------------------------------------------------------- kernels (launchers)
@@ -186,7 +187,7 @@ void launch_forward_reduce(const float2 *part, int N, int splits, float2 *D, cud
 
 // k_gemm_f32.cu (FP32 accuracy on the tensor cores)
 int forward_splits(int N, int X);
-bool f32_setup(F32Planes &p, int N, int X, bool full, cudaStream_t s);
+bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t s);
 void f32_free(F32Planes &p, cudaStream_t s);
 void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s);
 void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s);
@@ -200,7 +201,7 @@ int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, doub
 // k_gemm_tc.cu (BF16 tensor cores)
 bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
                   const cuuint32_t *box, const cuuint32_t *estr, CUtensorMapSwizzle swizzle);
-bool tc_setup(TcPlanes &p, int N, int X, bool split, cudaStream_t s);
+bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t s);
 // Choose the forward K split by timing the candidates on this job's planes (once per shape
 // and process; later jobs of the shape reuse the choice). part holds fwd_max_splits partials.
 bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream_t s);
