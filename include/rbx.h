@@ -282,9 +282,9 @@ rbx_status rbx_reconstruct(rbx_job *job, const double *freqs_hz, int nf, const v
  * weights v_dev (n_nodes float32, v = omega^2 dA dm per mask node); D_dev is N x N complex64.
  * It allocates nothing: the split partial sums live in a fixed 8 MiB array inside the
  * library, so n_xducers must be <= 1024 (RBX_EINVAL otherwise). The contraction splits the
- * mask nodes over at most floor(2^20 / N^2) CTAs per tile pair (the array holds that many
- * N x N partial sums): at N = 1024 it runs unsplit, one CTA per upper 64 x 64 tile pair
- * (136 CTAs), each looping over all nodes, so the largest sizes run well below the speed of
+ * mask nodes over at most floor(2^20 / N^2) partial sums per tile pair (the array holds that many
+ * N x N ones), each shared by a cluster of up to four CTAs; every CTA forms its own operands, so the
+ * largest sizes run below the speed of
  * rbx_forward. The first call on each
  * device looks up that array's device address (it may load the module): make it before any
  * stream capture. All calls share the array; calls that overlap on the GPU race and must be

@@ -1,6 +1,7 @@
 """The FP32 contractions (three BF16 parts per operand on the tensor cores) at the edges of their
 tiles: transducer counts around one and two 128-wide tiles and 32-wide K chunks, odd node counts,
-and the plain adjoint of a tensor-core job, which goes through the nodes in slabs.
+and the plain adjoint of a tensor-core job, which goes through the nodes in slabs; and the forward that
+allocates nothing (its operands formed in the kernel, one CTA or a cluster per tile).
 
 Reference: the sums in complex128 on the same FP32 tables. Tolerance: an operand carries about six
 FP32 roundings (phase, sine, amplitude, products), two operands sqrt(12) 2^-24 = 2.1e-7 relative
@@ -9,6 +10,7 @@ leaves a factor of two and is below the 7.6e-6 that one lost low part (2^-17) wo
 preconditioned operands divide by dgamma, a difference of FP32 angles of size 2 pi / N with an
 error of 2^-23: N 2^-24 on top.
 """
+import ctypes
 import math
 
 import numpy as np
@@ -66,6 +68,11 @@ def test_against_complex128(n, nx, ny):
     dev = [torch.tensor(t, device="cuda") for t in (T, a, gam, K)]
     exits = torch.zeros((n, n - 1, 4), device="cuda")
     Rd, dmd = torch.tensor(R, device="cuda"), torch.tensor(dm, device="cuda")
+    D = torch.empty((n, n), dtype=torch.complex64, device="cuda")
+    vd, err = torch.tensor(v.astype(np.float32), device="cuda"), ctypes.create_string_buffer(256)
+    assert rbx.load().rbx_forward_noalloc(dev[0].data_ptr(), dev[1].data_ptr(), dev[3].data_ptr(), vd.data_ptr(), n, a.shape[1],
+                                          F, C0, D.data_ptr(), torch.cuda.current_stream().cuda_stream or None, err, 256) == 0
+    assert rel(D.cpu().numpy(), want["forward"]) <= 1e-6
     for prec in (rbx.RBX_FP32, rbx.RBX_BF16):
         job = rbx.Job()
         job.set_geometry(g, precision=prec)
