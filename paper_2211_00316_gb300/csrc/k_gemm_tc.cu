@@ -538,16 +538,17 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// One synthesis tile: 32 nodes x 32 transducers, with a halo row of transducers on each side.
-constexpr int kSynSlots = 34 * 32;   // slot s holds row (e0 - 1 + s) mod N, nodes x0 .. x0 + 31
+// One synthesis tile: 32 nodes x 64 transducers, with a halo row of transducers on each side.
+constexpr int kSynE = 64, kSynThreads = 512;
+constexpr int kSynSlots = (kSynE + 2) * 32;   // slot s holds row (e0 - 1 + s) mod N, nodes x0 .. x0 + 31
 
 // Queue the copies of tile t's table entries into buf (entries past the last node are not
 // copied; the consumer treats them as uncovered).
 __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab, int N, int X, int XT, int t,
                                                 TabEntry *buf)
 {
-    const int ET = (N + 31) / 32, x0 = (t / ET) * 32, e0 = (t % ET) * 32;
-    for (int idx = threadIdx.x; idx < kSynSlots; idx += 256) {
+    const int ET = (N + kSynE - 1) / kSynE, x0 = (t / ET) * 32, e0 = (t % ET) * kSynE;
+    for (int idx = threadIdx.x; idx < kSynSlots; idx += kSynThreads) {
         const int slot = idx >> 5, x = x0 + (idx & 31);
         if (x < X) {
             const int e = (e0 - 1 + slot + N) % N;
@@ -559,8 +560,9 @@ __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab
 // planes [6][Xp][Npad] at [x][e]: u, conj(kappa) u, kappa u (re, im each);
 // u_e[x] = dgamma / (C a) exp(-i 2 pi (f T - K/4 + 1/8)), kappa = exp(i gamma).
 // The angular density dgamma (step a4) is formed here from the direction angles of the
-// neighbouring transducers: a 32-transducer tile reads one halo row on each side (rows wrap
-// around the ring), so the tables are read once more by 1/16 instead of a separate pass.
+// neighbouring transducers: a 64-transducer tile reads one halo row on each side (rows wrap
+// around the ring), so the tables are read once more by 1/32 instead of a separate pass, and a
+// row of a back-projection plane is written in 128-byte pieces.
 // With FWD the same pass also writes the forward's planes (those of k_synth_fwd_tc, from the
 // same phase): an update reads its tables once for both contractions' operands.
 // Persistent: each block walks the tiles t = blockIdx.x, + gridDim.x, ... (transducer blocks
@@ -569,7 +571,7 @@ __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab
 // two shared-memory buffers, the next tile's entries copied in while the current one is
 // formed and stored, so that table reads stay in flight between the blocks' barriers.
 template <bool FWD>
-__global__ __launch_bounds__(256, 4) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
+__global__ __launch_bounds__(kSynThreads, 2) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
                                                      size_t pstride, float fhi, float flo, float C,
                                                      __nv_bfloat16 *__restrict__ planes, const float2 *__restrict__ bw,
                                                      int Xpad, size_t fpstride, __nv_bfloat16 *__restrict__ fplanes,
@@ -578,9 +580,9 @@ __global__ __launch_bounds__(256, 4) void k_synth_tc(const TabEntry *__restrict_
     constexpr int NPL = 6;                                   // back-projection planes
     extern __shared__ __align__(16) unsigned char syn_smem[];
     TabEntry *buf = reinterpret_cast<TabEntry *>(syn_smem);  // [2][kSynSlots]
-    // [plane][x][e]: rows of 17 words, the tile transposed and rounded to BF16
-    __nv_bfloat16(*sv)[32][34] = reinterpret_cast<__nv_bfloat16(*)[32][34]>(syn_smem + 2 * kSynSlots * sizeof(TabEntry));
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
+    // [plane][x][e]: rows of 33 words, the tile transposed and rounded to BF16
+    __nv_bfloat16(*sv)[32][kSynE + 2] = reinterpret_cast<__nv_bfloat16(*)[32][kSynE + 2]>(syn_smem + 2 * kSynSlots * sizeof(TabEntry));
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 16
     int t = blockIdx.x, b = 0;
     if (t < ntiles) synth_tile_load(tab, N, X, XT, t, buf);
     cp_async_commit();
@@ -590,14 +592,14 @@ __global__ __launch_bounds__(256, 4) void k_synth_tc(const TabEntry *__restrict_
         cp_async_wait1();   // this thread's copies of tile t have landed
         __syncthreads();    // and every thread's
         const TabEntry *B = buf + b * kSynSlots;
-        const int ET = (N + 31) / 32, x0 = (t / ET) * 32, e0 = (t % ET) * 32;
+        const int ET = (N + kSynE - 1) / kSynE, x0 = (t / ET) * 32, e0 = (t % ET) * kSynE;
         const int x = x0 + tx;
         const bool xin = x < X;
         float2 vv = make_float2(0.f, 0.f);
         if (FWD && xin) vv = bw[x];   // Born weights of node x
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const int q = ty + 8 * k;
+            const int q = ty + 16 * k;
             float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             float gr = 0.f, gi = 0.f;
             const TabEntry r = B[(q + 1) * 32 + tx];   // row e0 + q
@@ -638,12 +640,12 @@ __global__ __launch_bounds__(256, 4) void k_synth_tc(const TabEntry *__restrict_
         const uint32_t *sw = reinterpret_cast<const uint32_t *>(&sv[0][0][0]);
 #pragma unroll
         for (int j = 0; j < 2; j++) {
-            const int item = threadIdx.x + 256 * j, xr = item >> 4, pr = item & 15;
+            const int item = threadIdx.x + kSynThreads * j, xr = item >> 5, pr = item & 31;
             if (x0 + xr < X) {
                 const size_t o = (size_t)(x0 + xr) * Npad + e0 + 2 * pr;
 #pragma unroll
                 for (int m = 0; m < NPL; m++)
-                    *reinterpret_cast<uint32_t *>(planes + m * pstride + o) = sw[(m * 32 + xr) * 17 + pr];
+                    *reinterpret_cast<uint32_t *>(planes + m * pstride + o) = sw[(m * 32 + xr) * (kSynE / 2 + 1) + pr];
             }
         }
     }
@@ -955,14 +957,14 @@ int launch_forward_tc(TcPlanes &p, float2 *part, cudaStream_t s)
 template <bool FWD>
 static int synth_grid(size_t &smem)
 {
-    smem = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * 34 * sizeof(__nv_bfloat16);
+    smem = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * (kSynE + 2) * sizeof(__nv_bfloat16);
     static int blocks = 0;
     if (blocks == 0) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaFuncSetAttribute(k_synth_tc<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, 256, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, kSynThreads, smem);
         blocks = sms * (per_sm > 0 ? per_sm : 1);
     }
     return blocks;
@@ -972,11 +974,11 @@ template <bool FWD>
 static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
     const float fhi = (float)f, flo = (float)(f - (double)fhi);
-    const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + 31) / 32);
+    const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + kSynE - 1) / kSynE);
     size_t smem = 0;
     int grd = synth_grid<FWD>(smem);
     if (grd > ntiles) grd = ntiles;
-    k_synth_tc<FWD><<<grd, 256, smem, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
+    k_synth_tc<FWD><<<grd, kSynThreads, smem, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
                                                   static_cast<__nv_bfloat16 *>(p.bplanes), v, FWD ? p.Xpad : 0,
                                                   FWD ? p.fwd_pstride : 0,
                                                   FWD ? static_cast<__nv_bfloat16 *>(p.fplanes) : nullptr, XT, ntiles);
