@@ -384,7 +384,7 @@ __device__ __forceinline__ void raster_quad_warp(bool valid, const Vtx &P00, con
     }
 }
 
-// Warps per block, each tracing the same rays of a neighbouring transducer; 20 warps per SM.
+// Warps per block, each tracing the same rays of a neighbouring transducer.
 constexpr int kFansPerBlock = 4;
 
 // The per-warp hit queues of a block (shared memory).
@@ -677,8 +677,8 @@ __device__ __forceinline__ void trace_block(const float *__restrict__ F, const i
     if (lane == 0 && *hq.cov) atomicAdd(&counters[0], (unsigned long long)*hq.cov);
 }
 
-template <bool LOSSY, bool RAW>
-__global__ __launch_bounds__(32 * kFansPerBlock, 20 / kFansPerBlock) void k_trace_raster(const float *__restrict__ F, const int4 *__restrict__ rows_g,
+template <bool LOSSY, bool RAW, int WARPS>
+__global__ __launch_bounds__(32 * kFansPerBlock, WARPS / kFansPerBlock) void k_trace_raster(const float *__restrict__ F, const int4 *__restrict__ rows_g,
                                                          TabEntry *__restrict__ tab, float4 *__restrict__ exits,
                                                          RayParams p, unsigned long long *counters)
 {
@@ -1082,14 +1082,24 @@ void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, f
         else wide(std::integral_constant<int, 2>{});
         return;
     }
-    if (lossy && raw)
-        k_trace_raster<true, true><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
-    else if (lossy)
-        k_trace_raster<true, false><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
-    else if (raw)
-        k_trace_raster<false, true><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+    auto go = [&](auto w) {
+        constexpr int W = decltype(w)::value;
+        if (lossy && raw)
+            k_trace_raster<true, true, W><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+        else if (lossy)
+            k_trace_raster<true, false, W><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+        else if (raw)
+            k_trace_raster<false, true, W><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+        else
+            k_trace_raster<false, false, W><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+    };
+    // 16 warps per SM with 128 registers each while they hold the whole grid (to about 260
+    // transducers: 256 on 288 x 288 1.86 -> 1.75 ms), else 20 with 96 and a few spills (1024 on 512 x 512
+    // 15.6 ms against 16.4)
+    if ((size_t)p.N * nwarps <= 152 * 16)
+        go(std::integral_constant<int, 16>{});
     else
-        k_trace_raster<false, false><<<grd, 32 * kFansPerBlock, sm, s>>>(fields, rows, tab, exits, p, counters);
+        go(std::integral_constant<int, 20>{});
 }
 
 int trace_items(int N, int *nwarps)
