@@ -40,7 +40,7 @@ struct Form {
     static constexpr int PLANES = 2 * NP;
     static constexpr uint32_t OPER = PLANES * PLANE;       // an operand's tile, all parts: 48 or 32 KB
     static constexpr int STAGES = NP == 3 ? 2 : 3;
-    static constexpr size_t SMEM = 1024 + (size_t)STAGES * 2 * OPER + 4352;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * 2 * OPER + 2304;
     static constexpr int PRODUCTS = NP == 3 ? 6 : 3;
 };
 constexpr int EPI = 256;                                   // epilogue threads (warps 2..9)
@@ -93,7 +93,7 @@ __device__ __forceinline__ float2 unit_of(float g)
 
 struct GemmArgs {
     CUtensorMap a, b;
-    int N, ntile, nk, kper;         // forward: tile rows, K chunks, chunks per split
+    int N, ntile, nk, kper;         // tiles of transducers, K chunks; forward: chunks per split
     float2 *part;                   // forward: [split][N][N] partial D
     const TabEntry *tab;            // back-projection: directions of stack 1
     const __nv_bfloat16 *planes;    // back-projection: parts of the weights, [plane][N][xld]
@@ -108,16 +108,17 @@ struct GemmArgs {
 // row-dot with the weights. CONJ: the plain adjoint, A = W = conj(G).
 // NP = 3: FP32 accuracy, six products. NP = 2 (split BF16): hi hi + hi lo + lo hi; against kernels
 // that drained long sums to global memory (forward) or stopped for the drain (back-projection),
-// 768 transducers, 59,800 nodes: an update from tables 3.24 -> 2.60 ms, forward error 2.7e-6 ->
-// 1.1e-6.
+// 768 transducers, 59,800 nodes: an update from tables 3.24 -> 2.60 ms (2.35 with the row-dot as it
+// is now), forward error 2.7e-6 -> 1.1e-6.
 //
 // Bound: shared-memory bandwidth of the tensor cores. A 128 x 128 x 16 MMA reads 8 KB in the 64
 // clocks it takes at the peak rate (128 B per clock, all an SM has), the tile loads write 31 B
 // per clock besides, so 0.7-0.8 of the BF16 peak over the six products is what the form allows.
 // K chunks of 32 because a 64-term stage of both operands' parts (192 KB) leaves no second one.
 // Against FP32 multiply-adds on the CUDA cores (64 x 64 tiles, 0.5 of their peak), ncu: 256
-// transducers, 48,120 nodes: forward 437 -> 89 us, back-projection 1297 -> 321 us; 768
-// transducers, 19,760 nodes: plain adjoint 2915 -> 384 us. Error against 64 bits no larger at any
+// transducers, 48,120 nodes: forward 437 -> 89 us, back-projection 1297 -> 321 us (its row-dot as it
+// is now takes another 75 us off the update); 768 transducers, 19,760 nodes: plain adjoint 2915 -> 384
+// us, 364 now. Error against 64 bits no larger at any
 // size from 48 transducers on (N = 1024, 20,000 nodes: forward 6.0e-7 -> 2.2e-7, plain adjoint
 // 6.1e-7 -> 1.7e-7).
 template <int NP, bool BP, bool CONJ>
@@ -131,15 +132,16 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
     uint64_t *empty = full + STAGES;
     uint64_t *accf = empty + STAGES;       // [2] accumulator buffer ready to drain
     uint64_t *acce = accf + 2;             // [2] accumulator buffer drained
-    float2 *quarter_sum = reinterpret_cast<float2 *>(acce + 2);   // [4][128]
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(quarter_sum + 4 * BM);
+    uint64_t *wfull = acce + 2;            // [2] weights of the tile's emitters 0-63, 64-127 landed
+    float2 *half_sum = reinterpret_cast<float2 *>(wfull + 2);   // [2][128]
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(half_sum + 2 * BM);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int N = g.N;
 
     int ta, tb, c0 = 0, nc;                // tile of A (rows of D), tile of B (columns), K chunks
     if (BP) {
-        tb = blockIdx.x;
-        ta = blockIdx.y;
+        tb = blockIdx.x % g.ntile;         // one grid dimension: any number of nodes
+        ta = blockIdx.x / g.ntile;
         nc = g.nk;
     } else {
         int b = blockIdx.x, te = 0;
@@ -149,12 +151,12 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
         c0 = blockIdx.y * g.kper;
         nc = min(g.nk, c0 + g.kper) - c0;
     }
-    const int stack = BP ? blockIdx.z : 0;
+    const int stack = BP ? blockIdx.y : 0;
     const int ncol = min(BN, (N - tb * BN + 15) & ~15);   // columns of the MMAs (a ragged last tile)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; s++) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
-        for (int q = 0; q < 2; q++) { mbar_init(accf + q, 1); mbar_init(acce + q, EPI); }
+        for (int q = 0; q < 2; q++) { mbar_init(accf + q, 1); mbar_init(acce + q, EPI); mbar_init(wfull + q, 1); }
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tslot, 512);
@@ -183,7 +185,20 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
             }
             issued++;
         }
+        // the row-dot's weights (the first operand's rows of the tile's emitters), 64 emitters to
+        // each of the first two stages that the MMAs leave
+        int halves = 0;
+        for (; BP && issued == nc && halves < 2; halves++) {
+            const int s = (nc + halves) % STAGES, c = nc - STAGES + halves;
+            if (c >= 0 && !mbar_wait(empty + s, (c / STAGES) & 1)) { atomicOr(g.err, 64u); break; }
+            mbar_arrive_expect_tx(wfull + halves, 2 * OPER);
+            for (int q = 0; q < 4; q++)
+                tma_load_3d(smem_u32(tiles + (size_t)s * 2 * OPER + q * (OPER / 2)), &g.a, wfull + halves,
+                            ta * BM + (q & 1) * 64, tb * BN + halves * 64 + (q >> 1) * BK, 0);
+        }
         // no copy may still be in flight when the CTA retires
+        for (int h = 0; h < halves; h++)
+            if (!mbar_wait(wfull + h, 0)) atomicOr(g.err, 4u);
         for (int c = (issued > STAGES ? issued - STAGES : 0); c < issued; c++)
             if (!mbar_wait(full + (c % STAGES), (c / STAGES) & 1)) atomicOr(g.err, 4u);
     } else if (warp == 1) {
@@ -265,91 +280,89 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
                 }
             }
         } else {
-            // P through shared memory (the stages are free: every MMA has read them), column i of
-            // 128 rows at P[i]; then each thread takes two neighbouring nodes and 32 emitters
-            float2 *P = reinterpret_cast<float2 *>(tiles);
+            // The row-dot: a thread's node and 64 emitters. P goes back to tensor memory, so that a
+            // loop over eight emitters at a time can index it; the weights come by TMA into the
+            // stages, in the layout of the first operand, two of them while the last products run
+            // (loaded from global memory into registers, eight emitters at a time: 768 transducers,
+            // 59,800 nodes, split: an update from tables 2.58 -> 2.35 ms; 256, 48,120 nodes, FP32:
+            // an update 75 us less).
+            const int xl = min(ta * BM + row, g.nx - 1), e0 = tb * BN + half * 64, ne = min(64, N - e0);
+            const TabEntry *tab = g.tab + (size_t)e0 * g.X + g.x0 + xl;
+            const uint8_t *wt = tiles + (size_t)((nc + half) % STAGES) * 2 * OPER + (row >> 6) * (OPER / 2);
+            const uint32_t chunk = (uint32_t)(row & 63) >> 3, in_chunk = (uint32_t)(row & 7) * 2;
+            float2 s[8];   // partial sums, of every eighth emitter
 #pragma unroll
-            for (int i = 0; i < 64; i++) P[(half * 64 + i) * BM + row] = make_float2(re[i], im[i]);
-            asm volatile("bar.sync 1, 256;" ::: "memory");   // the epilogue warps
-            const int t = threadIdx.x - 64, r2 = 2 * (t & 63), quarter = t >> 6;
-            const int xl = ta * BM + r2, e0 = tb * BN + quarter * 32, ne = min(32, N - e0);
-            // eight partial sums, of every eighth emitter
-            float2 s[2][8];
+            for (int k = 0; k < 8; k++) s[k] = make_float2(0.f, 0.f);
+            // directions of the weights kappa u, loaded eight emitters ahead
+            uint32_t idk[8];
+            float gam[8];
+            auto directions = [&](int i0) {
 #pragma unroll
-            for (int k = 0; k < 8; k++) s[0][k] = s[1][k] = make_float2(0.f, 0.f);
-            if (ok && xl < g.nx && ne > 0) {
-                const bool two = xl + 1 < g.nx;
-                const __nv_bfloat16 *w = g.planes + (size_t)e0 * g.xld + xl;
-                const TabEntry *tab = g.tab + (size_t)e0 * g.X + g.x0 + xl;
-                // eight rows at a time, all their loads first: the weights come from L2 or HBM,
-                // and a chain of single rows waits for each
+                for (int k = 0; k < 8; k++) {
+                    const TabEntry *t = tab + (size_t)min(i0 + k, ne - 1) * g.X;
+                    idk[k] = __ldg(&t->idk);
+                    gam[k] = __ldg(&t->gam);
+                }
+            };
+            if (!CONJ && stack == 1 && ne > 0) directions(0);
+            const bool have = __all_sync(0xffffffffu, ok && mbar_wait(wfull + half, 0));
+            if (!have && lane == 0) atomicOr(g.err, 64u);
+            if (have) {
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    tmem_st32(at + q * 32, re + q * 32);
+                    tmem_st32(at + BN + q * 32, im + q * 32);
+                }
+            }
 #pragma unroll 1
-                for (int i0 = 0; i0 < ne; i0 += 8) {
-                    __nv_bfloat162 q[8][PLANES];
-                    float gam[8][2];
+            for (int i0 = 0; have && i0 < ne; i0 += 8) {
+                float2 kap[8];
+                if (!CONJ && stack == 1) {
+                    // an uncovered entry's weight is zero and its direction not a number
 #pragma unroll
-                    for (int k = 0; k < 8; k++) {
-                        const int i = min(i0 + k, ne - 1);
+                    for (int k = 0; k < 8; k++) kap[k] = unit_of(idk[k] == kUncovered ? 0.f : gam[k]);
+                    if (i0 + 8 < ne) directions(i0 + 8);
+                }
+                float pr[8], pi[8];
+                tmem_ld8(at + i0, pr);
+                tmem_ld8(at + BN + i0, pi);
+                const uint8_t *wk = wt + (size_t)(i0 >> 5) * OPER + (i0 & 31) * 128;
 #pragma unroll
-                        for (int m = 0; m < PLANES; m++)
-                            q[k][m] = *reinterpret_cast<const __nv_bfloat162 *>(w + (size_t)i * g.xld + m * g.pstride);
-                        if (!CONJ && stack == 1) {
-                            // an uncovered entry's weight is zero and its direction not a number
-                            const uint4 v0 = __ldg(reinterpret_cast<const uint4 *>(tab + (size_t)i * g.X));
-                            const uint4 v1 = __ldg(reinterpret_cast<const uint4 *>(tab + (size_t)i * g.X + (two ? 1 : 0)));
-                            gam[k][0] = v0.x == kUncovered ? 0.f : __uint_as_float(v0.w);
-                            gam[k][1] = v1.x == kUncovered ? 0.f : __uint_as_float(v1.w);
-                        }
+                for (int k = 0; k < 8; k++) {
+                    const uint8_t *z = wk + k * 128 + ((chunk ^ (uint32_t)k) << 4) + in_chunk;
+                    // the parts add up to the weight (three: the FP32 weight) exactly
+                    float wr = 0.f, wi = 0.f;
+#pragma unroll
+                    for (int m = 0; m < NP; m++) {
+                        wr += __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(z + m * (PLANE / 2)));
+                        wi += __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(z + (NP + m) * (PLANE / 2)));
                     }
-#pragma unroll
-                    for (int k = 0; k < 8; k++) {
-                        const bool in = i0 + k < ne;
-                        const float4 p = *reinterpret_cast<const float4 *>(P + (quarter * 32 + i0 + k) * BM + r2);
-#pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            // the parts add up to the weight (three: the FP32 weight) exactly
-                            float wr = 0.f, wi = 0.f;
-#pragma unroll
-                            for (int m = 0; m < NP; m++) {
-                                wr += h ? __high2float(q[k][m]) : __low2float(q[k][m]);
-                                wi += h ? __high2float(q[k][NP + m]) : __low2float(q[k][NP + m]);
-                            }
-                            if (CONJ) wi = -wi;
-                            if (!CONJ && stack == 1) {
-                                const float2 kap = unit_of(gam[k][h]);
-                                const float ur = wr;
-                                wr = kap.x * ur - kap.y * wi;
-                                wi = kap.x * wi + kap.y * ur;
-                            }
-                            const float pr = h ? p.z : p.x, pi = h ? p.w : p.y;
-                            if (in) {
-                                s[h][k].x = fmaf(wr, pr, s[h][k].x);
-                                s[h][k].x = fmaf(-wi, pi, s[h][k].x);
-                                s[h][k].y = fmaf(wr, pi, s[h][k].y);
-                                s[h][k].y = fmaf(wi, pr, s[h][k].y);
-                            }
-                        }
+                    if (CONJ) wi = -wi;
+                    if (!CONJ && stack == 1) {
+                        const float ur = wr;
+                        wr = kap[k].x * ur - kap[k].y * wi;
+                        wi = kap[k].x * wi + kap[k].y * ur;
                     }
+                    s[k].x = fmaf(wr, pr[k], s[k].x);
+                    s[k].x = fmaf(-wi, pi[k], s[k].x);
+                    s[k].y = fmaf(wr, pi[k], s[k].y);
+                    s[k].y = fmaf(wi, pr[k], s[k].y);
                 }
             }
 #pragma unroll
-            for (int h = 0; h < 2; h++) {
+            for (int d = 4; d > 0; d >>= 1)
 #pragma unroll
-                for (int d = 4; d > 0; d >>= 1)
-#pragma unroll
-                    for (int k = 0; k < d; k++) {
-                        s[h][k].x += s[h][k + d].x;
-                        s[h][k].y += s[h][k + d].y;
-                    }
-                quarter_sum[quarter * BM + r2 + h] = s[h][0];
-            }
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+                for (int k = 0; k < d; k++) {
+                    s[k].x += s[k + d].x;
+                    s[k].y += s[k + d].y;
+                }
+            half_sum[half * BM + row] = s[0];
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // the epilogue warps
+            const int t = threadIdx.x - 64;
             const int xo = ta * BM + t;
             if (t < BM && xo < g.nx) {
-                const float2 a = quarter_sum[t], b = quarter_sum[BM + t], c = quarter_sum[2 * BM + t],
-                             d = quarter_sum[3 * BM + t];
-                g.bpart[((size_t)stack * gridDim.x + tb) * g.X + g.x0 + xo] =
-                    make_float2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
+                const float2 a = half_sum[t], b = half_sum[BM + t];
+                g.bpart[((size_t)stack * g.ntile + tb) * g.X + g.x0 + xo] = make_float2(a.x + b.x, a.y + b.y);
             }
         }
     }
@@ -456,15 +469,20 @@ __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict_
     }
 }
 
-// R_s (complex N x N) -> parts [2 NP][N][rld]
-template <int NP>
+// R_s (complex N x N; SYM: R, from which R_s = (R + R^T)/2 is formed here, one launch less in an
+// adjoint) -> parts [2 NP][N][rld]
+template <int NP, bool SYM>
 __global__ void k_rs_parts(const float2 *__restrict__ Rs, int N, int rld, __nv_bfloat16 *__restrict__ planes)
 {
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= (size_t)N * N) return;
     const size_t o = (i / N) * rld + i % N, P = (size_t)N * rld;
     __nv_bfloat16 q[2 * NP];
-    const float2 v = Rs[i];
+    float2 v = Rs[i];
+    if (SYM) {
+        const float2 t = Rs[(i % N) * N + i / N];
+        v = make_float2(0.5f * (v.x + t.x), 0.5f * (v.y + t.y));
+    }
     split<NP>(v.x, q);
     split<NP>(v.y, q + NP);
 #pragma unroll
@@ -564,7 +582,7 @@ bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st
     const int x8 = (X + 7) / 8 * 8;
     // all nodes' forward or back-projection operands (24 or 16 B an entry), or on a tensor-core job,
     // whose plain adjoint alone comes here, 8 B an entry and the nodes in slabs
-    p.xs = full ? x8 : std::max(std::min(x8, 64), X * 2 / 3 / 8 * 8);
+    p.xs = full ? x8 : std::max(std::min(x8, 64), (int)((size_t)X * 2 / 3 / 8 * 8));
     p.xld = p.xs;
     p.pstride = (size_t)N * p.xld;
     p.rld = (N + 7) / 8 * 8;
@@ -625,6 +643,7 @@ static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
     g.a = p.amap;
     g.b = p.rmap;
     g.N = p.N;
+    g.ntile = (p.N + BN - 1) / BN;
     g.nk = (p.N + BK - 1) / BK;
     g.tab = tab;
     g.planes = static_cast<const __nv_bfloat16 *>(p.planes);
@@ -636,24 +655,29 @@ static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
     return g;
 }
 
+template <bool SYM>
 static void rs_parts(F32Planes &p, const float2 *Rs, cudaStream_t s)
 {
     const size_t nn = (size_t)p.N * p.N;
     const unsigned nb = (unsigned)((nn + 255) / 256);
     if (p.parts == 3)
-        k_rs_parts<3><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
+        k_rs_parts<3, SYM><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
     else
-        k_rs_parts<2><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
+        k_rs_parts<2, SYM><<<nb, 256, 0, s>>>(Rs, p.N, p.rld, static_cast<__nv_bfloat16 *>(p.rs));
 }
 
 // The preconditioned back-projection from the operands of launch_synth_bp: gpart[2][X].
-int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, float2 *gpart, cudaStream_t s)
+int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *R, bool symmetric, float2 *gpart,
+                           cudaStream_t s)
 {
     const int ET = (p.N + BN - 1) / BN;
-    rs_parts(p, Rs, s);
+    if (symmetric)
+        rs_parts<false>(p, R, s);
+    else
+        rs_parts<true>(p, R, s);
     GemmArgs g = bp_args(p, tab, gpart);
     g.nx = p.X;
-    const dim3 grd(ET, (p.X + BM - 1) / BM, 2);
+    const dim3 grd((unsigned)ET * ((p.X + BM - 1) / BM), 2);
     if (p.parts == 3)
         k_cgemm_f32<3, true, false><<<grd, THREADS, Form<3>::SMEM, s>>>(g);
     else
@@ -664,18 +688,18 @@ int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, 
 }
 
 // The plain adjoint's sum_{e,r} conj(G_e G_r) R_s: synthesis and contraction, slab by slab.
-int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, double f, double c0, float2 *gpart,
+int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *R, double f, double c0, float2 *gpart,
                        cudaStream_t s)
 {
     const int ET = (p.N + BN - 1) / BN;
     int n = 1;
-    rs_parts(p, Rs, s);
+    rs_parts<true>(p, R, s);
     for (int x0 = 0; x0 < p.X; x0 += p.xs, n += 2) {
         GemmArgs g = bp_args(p, tab, gpart);
         g.x0 = x0;
         g.nx = std::min(p.xs, p.X - x0);
         synth<0>(p, tab, nullptr, x0, g.nx, f, c0, s);
-        k_cgemm_f32<3, true, true><<<dim3(ET, (g.nx + BM - 1) / BM, 1), THREADS, Form<3>::SMEM, s>>>(g);   // parts == 3
+        k_cgemm_f32<3, true, true><<<(unsigned)ET * ((g.nx + BM - 1) / BM), THREADS, Form<3>::SMEM, s>>>(g);   // parts == 3
     }
     if (ET == 1) return n;
     k_bp_sum<<<dim3((p.X + 255) / 256, 1), 256, 0, s>>>(p.bpart, ET, p.X, gpart);

@@ -9,7 +9,8 @@
 // a final partial step that lands on the ring (Def. ray-parameterisation).
 //
 // GB300 mapping: one thread per ray, 32 adjacent rays of one fan per warp stepping in
-// lockstep; a block's four warps take the same rays of four neighbouring transducers. At
+// lockstep; a block's four warps take the same rays of four neighbouring transducers, the warps
+// with the longest rays first (a small ring gives each ray several lanes: k_trace_wide). At
 // each step a lane fetches its neighbour's new sample with a shuffle and rasterises the
 // ray-tube quad (rays j, j+1; samples i, i+1) as two triangles straight
 // into the fan's table (Sec. 4.4: triangulation of the ray samples). Overlapping triangles

@@ -640,20 +640,20 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
     NEED(j, j->has_tables, RBX_ESTATE, "rbx_adjoint before rbx_trace_rays or rbx_set_tables");
     NEED(j, !bad_freq(f), RBX_EINVAL, "frequency must be finite and > 0");
     Workspace &w = j->w;
-    launch_symmetrize(static_cast<const float2 *>(R_dev), w.N, w.Rs, j->stream);
-    LAUNCHED(j, 1);
+    const float2 *R = static_cast<const float2 *>(R_dev);
     if (preconditioned && j->g.precision == RBX_BF16) {
+        launch_symmetrize(R, w.N, w.Rs, j->stream);
         launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
-        LAUNCHED(j, 4);
+        LAUNCHED(j, 5);
     } else if (preconditioned) {
         launch_synth_bp(parts_of(j), w.tab, f, j->g.c0, j->stream);
-        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, w.Rs, w.gpart, j->stream));
+        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, R, false, w.gpart, j->stream));
         launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
     } else {
         double om = 2 * 3.14159265358979323846 * f;
-        LAUNCHED(j, launch_adjoint_f32(w.f32, w.tab, w.Rs, f, j->g.c0, w.gpart, j->stream));
+        LAUNCHED(j, launch_adjoint_f32(w.f32, w.tab, R, f, j->g.c0, w.gpart, j->stream));
         if (j->lossy)
             launch_combine_adjoint_lossy(w.gpart, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j),
                                          static_cast<float2 *>(out_dev), j->stream);
@@ -700,7 +700,7 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
         launch_synth_bp(parts_of(j), w.tab, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if ((st = record(j, EV_SYNTH_B))) return st;
-        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, w.Rs, w.gpart, j->stream));
+        LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, w.Rs, true, w.gpart, j->stream));
     }
     if ((st = record(j, EV_GEMM_B))) return st;
     const int roff = residual_blocks(w.N) + 8;

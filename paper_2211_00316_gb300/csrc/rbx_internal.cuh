@@ -193,9 +193,10 @@ void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double
 void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s);
 void launch_forward_f32(F32Planes &p, int splits, float2 *part, cudaStream_t s);
 // Both return the number of kernels launched. Preconditioned: the two stacks of the operands
-// that launch_synth_bp wrote. Plain adjoint: synthesis included.
-int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, float2 *gpart, cudaStream_t s);
-int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *Rs, double f, double c0, float2 *gpart,
+// that launch_synth_bp wrote. Plain adjoint: synthesis included. R unless symmetric is symmetrised.
+int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *R, bool symmetric, float2 *gpart,
+                           cudaStream_t s);
+int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *R, double f, double c0, float2 *gpart,
                        cudaStream_t s);
 
 // k_gemm_tc.cu (BF16 tensor cores)

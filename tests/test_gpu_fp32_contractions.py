@@ -82,3 +82,26 @@ def test_against_complex128(n, nx, ny):
             assert rel(job.forward(F, dmd).cpu().numpy(), want["forward"]) <= 1e-6
             assert rel(job.adjoint(F, Rd, True).cpu().numpy(), want["pre"]) <= 1e-6 + n * 2.0 ** -24
         job.close()
+
+
+def test_more_than_65535_node_tiles():
+    """Tables of equal entries, 8.5 million nodes: every node's plain adjoint is the first one's,
+    whichever tile it falls in; so is the preconditioned one's (its two transducer neighbours differ by the
+    same angle)."""
+    n, m = 3, 3320
+    g = P.Geometry(nx=m, ny=m, dx=1e-4, n_xducers=n, ring_radius=(m - 1) * 0.5e-4 - 3e-4, mask_frac=0.999,
+                   ds_frac=4.0)
+    x = int(g.mask().sum())
+    assert x > 65535 * 128
+    dev = [torch.full((n, x), val, dtype=dt, device="cuda")
+           for val, dt in ((1e-4, torch.float32), (3.0, torch.float32), (0.0, torch.float32), (1, torch.uint8))]
+    dev[2] += torch.tensor([0.3, 2.4, -1.9], device="cuda")[:, None]
+    R = torch.tensor(np.random.default_rng(1).standard_normal((n, n)), device="cuda").to(torch.complex64)
+    job = rbx.Job()
+    job.set_geometry(g, precision=rbx.RBX_FP32)
+    job.set_tables(*dev, torch.zeros((n, n - 1, 4), device="cuda"))
+    for pre in (False, True):
+        out = job.adjoint(F, R, pre)
+        assert bool(torch.isfinite(torch.view_as_real(out)).all()) and float(out[0].abs()) > 0
+        assert bool((out == out[0]).all())
+    job.close()
