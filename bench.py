@@ -30,9 +30,6 @@ sys.path.insert(0, ROOT)
 
 METRIC = "ray-Born freq-updates/s at 1024 xducers, 512² grid; p50/p99 request latency"
 UNIT = "freq-updates/s"
-SM_COUNT = 152
-SM_MAX_MHZ = 2070.0
-FP32_LANES_PER_SM = 128
 
 
 def workload(name: str, seed: int):
@@ -73,10 +70,10 @@ def peaks():
 # the sources it was taken on)
 KERNEL_SRC = {
     "trace": ["k_rays.cu"],
-    "gemm_fwd": ["k_gemm_tc.cu", "tc_sm100.cuh", "k_gemm_simt.cu"],
-    "gemm_bp": ["k_gemm_tc.cu", "tc_sm100.cuh", "k_gemm_simt.cu"],
-    "synth_fwd": ["k_gemm_tc.cu", "k_gemm_simt.cu"],
-    "synth_bp": ["k_gemm_tc.cu", "k_gemm_simt.cu"],
+    "gemm_fwd": ["k_gemm_tc.cu", "tc_sm100.cuh", "k_gemm_f32.cu"],
+    "gemm_bp": ["k_gemm_tc.cu", "tc_sm100.cuh", "k_gemm_f32.cu"],
+    "synth_fwd": ["k_gemm_tc.cu", "k_gemm_f32.cu"],
+    "synth_bp": ["k_gemm_tc.cu", "k_gemm_f32.cu"],
     "synth": ["k_gemm_tc.cu"],
 }
 
@@ -112,19 +109,20 @@ def algorithmic(kernel: str, N: int, X: int, precision: str):
         return 16.0 * NX + 16.0 * N * (N - 1), "byte", "hbm"
     planes = 2.0 if precision == "bf16x3" else 1.0   # split BF16 writes a lo plane per hi plane
     if kernel == "synth_fwd":
-        return (16.0 + (8.0 * planes if precision != "fp32" else 8.0)) * NX, "byte", "hbm"
+        # FP32: three BF16 parts of every real number
+        return (16.0 + (8.0 * planes if precision != "fp32" else 24.0)) * NX, "byte", "hbm"
     if kernel == "synth":
         # fused: tables in once; forward (4 planes) and back-projection (6 planes) BF16 out
         return (16.0 + 20.0 * planes) * NX, "byte", "hbm"
     if kernel == "synth_bp":
-        # tables in; FP32: angular density in, U and kappa out; BF16: 6 planes out (x2 when split)
-        out = {"fp32": 4.0 + 16.0, "bf16": 12.0, "bf16x3": 24.0}[precision]
+        # tables in; BF16: 6 planes out; split BF16: the two parts of u and conj(kappa) u; FP32: the
+        # 20 bytes counted are those of u, conj(kappa) u and the angular density held in FP32 (the
+        # three BF16 parts written are 24)
+        out = {"fp32": 4.0 + 16.0, "bf16": 12.0, "bf16x3": 16.0}[precision]
         return (16.0 + out) * NX, "byte", "hbm"
     if kernel == "tables":
-        # direct Green's function (exits in, N x N complex out); FP32 also forms the angular
-        # density array (tables in, one float out per entry)
-        green = 16.0 * N * (N - 1) + 8.0 * N * N
-        return green + ((16.0 + 4.0) * NX if precision == "fp32" else 0.0), "byte", "hbm"
+        # direct Green's function (exits in, N x N complex out)
+        return 16.0 * N * (N - 1) + 8.0 * N * N, "byte", "hbm"
     return None, None, None
 
 
@@ -275,8 +273,8 @@ def time_noalloc(job, rbx, torch, g, f: float, stream, reps: int = 5) -> dict:
         torch.cuda.synchronize()
         out[name + "_ms"] = e0.elapsed_time(e1) / reps
     out["scratch_split_cap"] = (1 << 20) // (N * N)    # 8 MiB of float2 partial sums / (N x N per split)
-    out["note"] = ("rbx_forward at the job's precision (synthesis pass + contraction); rbx_forward_noalloc FP32 SIMT "
-                   "with the Green's functions formed in the tile loads, unsplit at N = 1024")
+    out["note"] = ("rbx_forward at the job's precision (synthesis pass + contraction); rbx_forward_noalloc FP32-accurate "
+                   "on the tensor cores, the Green's functions formed inside the contraction")
     return out
 
 
@@ -711,7 +709,7 @@ def main():
                    "h2d_bytes_per_step": N * N * 8,
                    "d2h_bytes_per_step": g.nx * g.ny * 4}
         # the allocation-free Born forward (rbx_forward_noalloc: Green's functions formed inside an
-        # FP32 SIMT contraction, fixed scratch) beside rbx_forward on the same tables
+        # FP32-accurate tensor-core contraction, fixed scratch) beside rbx_forward on the same tables
         noalloc = None
         if not args.no_forms and world == 1 and N <= 1024:
             noalloc = time_noalloc(job, rbx, torch, g, float(w.freqs[fidx[0]]), stream)
@@ -739,7 +737,7 @@ def main():
     # per-kernel device time averaged over the timed steps; roofline of every kernel with an
     # algorithmic work figure, and of the dominant one
     kms = {k: float(np.mean([s["ms_kernel"][k] for s in stats])) for k in stats[0]["ms_kernel"]}
-    if args.precision != "fp32" and args.integration != "raw":
+    if args.precision == "bf16" and args.integration != "raw":
         # one pass over the tables writes both contractions' operands (timed as the forward's)
         kms["synth"] = kms.pop("synth_fwd") + kms.pop("synth_bp")
     dom = max(kms, key=kms.get)
@@ -753,21 +751,21 @@ def main():
         if bound == "hbm":
             achieved, peak, u = amount / dur / 1e9, pk["hbm_gbs"], "GB/s"
         elif bound == "tensor":
-            # the contractions run as ~2 ms bursts between SIMT kernels, below the power cap a
+            # the contractions run as ~2 ms bursts between other kernels, below the power cap a
             # seconds-long GEMM loop reaches: the burst peak is theirs (the sustained one beside it)
             achieved, peak, u = amount / dur / 1e12, pk["bf16_tflops"], "TFLOP/s"
         else:
-            achieved = amount / dur / 1e12
-            peak = SM_COUNT * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
-            u = "TFLOP/s"
+            # FP32-accurate contractions: six BF16 products each on the tensor cores
+            bound = "tensor"
+            achieved, peak, u = amount / dur / 1e12, pk["bf16_tflops"] / 6, "TFLOP/s"
         tr = NCU_TRAFFIC.get((args.workload, kernel))
         traffic = tr["bytes"] if tr and tr.get("src") == kernel_src_hash(kernel) else None
         r = {"kernel": kernel, "bound": bound, "achieved": achieved, "peak": peak, "unit": u,
              "frac": achieved / peak, "traffic": traffic, "algorithmic_per_launch": amount, "ms": kms[kernel],
-             "peak_source": ((pk["source"] + (" burst bf16" if bound == "tensor" else " copy bandwidth"))
-                             if bound != "alu" else "FP32 SIMT: 152 SMs x 128 lanes x 2 flop x 2070 MHz")}
+             "peak_source": pk["source"] + (" copy bandwidth" if bound == "hbm" else
+                                            " burst bf16" + (" / 6 products" if args.precision == "fp32" else ""))}
         if bound == "tensor":
-            r["frac_of_sustained"] = achieved / pk["bf16_tflops_sustained"]
+            r["frac_of_sustained"] = r["frac"] * pk["bf16_tflops"] / pk["bf16_tflops_sustained"]
         return r
 
     roof = roofline(dom)

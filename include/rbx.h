@@ -82,8 +82,8 @@ typedef struct {
 
 /* indices into rbx_stats.ms_kernel */
 #define RBX_K_TRACE 0       /* ray trace + ray-to-grid scatter */
-#define RBX_K_SYNTH_FWD 1   /* Green's function synthesis for the forward; in an update on the
-                               BF16 paths it also writes the back-projection's operands */
+#define RBX_K_SYNTH_FWD 1   /* Green's function synthesis for the forward; in an update in
+                               RBX_BF16 it also writes the back-projection's operands */
 #define RBX_K_GEMM_FWD 2    /* Born forward contraction */
 #define RBX_K_SYNTH_BP 3    /* reciprocal Green's function synthesis (about 0 where
                                RBX_K_SYNTH_FWD did it) */
@@ -366,7 +366,7 @@ const char *rbx_last_error(const rbx_job *job);
  * query. Mode 2: the heuristic split with the fused-synthesis forward (see
  * rbx_get_tuning_times). Returns the previous mode. The choice changes the forward's
  * summation order, so results differ between split counts by rounding (within the BF16
- * tolerance). */
+ * tolerance). RBX_FP32 and RBX_BF16X3 jobs take the split that fills the GPU once. */
 int rbx_autotune(int mode);
 
 /* The forward K split the job uses and the number of candidates it timed (0: reused or
