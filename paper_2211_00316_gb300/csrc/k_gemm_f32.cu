@@ -98,7 +98,7 @@ struct GemmArgs {
     const TabEntry *tab;            // back-projection: directions of stack 1
     const __nv_bfloat16 *planes;    // back-projection: parts of the weights, [plane][N][xld]
     size_t pstride;
-    int xld, X, x0, nx;             // back-projection: row length, nodes in all, first node and count of the slab
+    int xld, X;                     // back-projection: row length of the planes, nodes
     float2 *bpart;                  // back-projection: [stack][e tile][X] partial row-dots
     unsigned *err;
 };
@@ -286,8 +286,8 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
             // (loaded from global memory into registers, eight emitters at a time: 768 transducers,
             // 59,800 nodes, split: an update from tables 2.58 -> 2.35 ms; 256, 48,120 nodes, FP32:
             // an update 75 us less).
-            const int xl = min(ta * BM + row, g.nx - 1), e0 = tb * BN + half * 64, ne = min(64, N - e0);
-            const TabEntry *tab = g.tab + (size_t)e0 * g.X + g.x0 + xl;
+            const int xl = min(ta * BM + row, g.X - 1), e0 = tb * BN + half * 64, ne = min(64, N - e0);
+            const TabEntry *tab = g.tab + (size_t)e0 * g.X + xl;
             const uint8_t *wt = tiles + (size_t)((nc + half) % STAGES) * 2 * OPER + (row >> 6) * (OPER / 2);
             const uint32_t chunk = (uint32_t)(row & 63) >> 3, in_chunk = (uint32_t)(row & 7) * 2;
             float2 s[8];   // partial sums, of every eighth emitter
@@ -360,9 +360,9 @@ __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant_
             asm volatile("bar.sync 1, 256;" ::: "memory");   // the epilogue warps
             const int t = threadIdx.x - 64;
             const int xo = ta * BM + t;
-            if (t < BM && xo < g.nx) {
+            if (t < BM && xo < g.X) {
                 const float2 a = half_sum[t], b = half_sum[BM + t];
-                g.bpart[((size_t)stack * g.ntile + tb) * g.X + g.x0 + xo] = make_float2(a.x + b.x, a.y + b.y);
+                g.bpart[((size_t)stack * g.ntile + tb) * g.X + xo] = make_float2(a.x + b.x, a.y + b.y);
             }
         }
     }
@@ -400,7 +400,7 @@ __device__ __forceinline__ void put_parts(__nv_bfloat16 *planes, size_t pstride,
 }
 
 // Operands of the contractions from the tables, two nodes and `walk` transducers per thread, as
-// parts in [plane][N][xld] for the slab of nx nodes from x0 on.
+// parts in [plane][N][xld].
 //  KIND 0: first operand G_e[x] = (8 pi omega/c0)^(-1/2) a exp(i 2 pi (f T - K/4 + 1/8)) (Eq. 2D_greens)
 //  KIND 1: first G, second G v (the forward)
 //  KIND 2: first u_e[x] = dgamma / ((8 pi omega/c0)^(-1/2) a) exp(-i 2 pi (...)) (Eq.
@@ -412,13 +412,13 @@ __device__ __forceinline__ void put_parts(__nv_bfloat16 *planes, size_t pstride,
 // nodes, NP = 3: 0.98 GB in 147 us.
 template <int KIND, int NP>
 __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict__ tab, const float2 *__restrict__ v, int N,
-                                                     int X, int x0, int nx, int xld, size_t pstride, float fhi, float flo,
+                                                     int X, int xld, size_t pstride, float fhi, float flo,
                                                      float C, __nv_bfloat16 *__restrict__ planes, int walk)
 {
     const int xl = 2 * (blockIdx.x * blockDim.x + threadIdx.x), e0 = blockIdx.y * walk;
-    if (xl >= nx) return;
-    const bool two = xl + 1 < nx;
-    const TabEntry *t = tab + x0 + xl;
+    if (xl >= X) return;
+    const bool two = xl + 1 < X;
+    const TabEntry *t = tab + xl;
     TabEntry none;
     none.idk = kUncovered;
     none.T = none.a = none.gam = 0.f;
@@ -431,8 +431,8 @@ __global__ __launch_bounds__(128) void k_synth_parts(const TabEntry *__restrict_
     row(e0, cur);
     float2 w[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     if (KIND == 1) {
-        w[0] = v[x0 + xl];
-        if (two) w[1] = v[x0 + xl + 1];
+        w[0] = v[xl];
+        if (two) w[1] = v[xl + 1];
     }
     const int e1 = min(N, e0 + walk);
     for (int e = e0; e < e1; e++) {
@@ -527,21 +527,21 @@ bool make_map(CUtensorMap *m, void *base, size_t cols, size_t rows, size_t plane
 }
 
 template <int KIND>
-void synth(const F32Planes &p, const TabEntry *tab, const float2 *v, int x0, int nx, double f, double c0, cudaStream_t s)
+void synth(const F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
     float fhi, flo;
     fsplit(f, fhi, flo);
     // a walk of 8 once that still gives every SM a full set of blocks; short ones on small
     // problems, which a long walk leaves waiting on its chain of loads
-    const unsigned bx = (unsigned)((nx + 255) / 256);
+    const unsigned bx = (unsigned)((p.X + 255) / 256);
     const int walk = (size_t)bx * ((p.N + 7) / 8) >= 152 * 16 ? 8 : 2;
     const dim3 grd(bx, (unsigned)((p.N + walk - 1) / walk));
     __nv_bfloat16 *planes = static_cast<__nv_bfloat16 *>(p.planes);
     if (p.parts == 3)
-        k_synth_parts<KIND, 3><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo,
+        k_synth_parts<KIND, 3><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.xld, p.pstride, fhi, flo,
                                                    green_const(f, c0), planes, walk);
     else
-        k_synth_parts<KIND, 2><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, x0, nx, p.xld, p.pstride, fhi, flo,
+        k_synth_parts<KIND, 2><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.xld, p.pstride, fhi, flo,
                                                    green_const(f, c0), planes, walk);
 }
 
@@ -578,12 +578,9 @@ bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st
     p.N = N;
     p.X = X;
     p.parts = parts;
-    p.full = full;
-    const int x8 = (X + 7) / 8 * 8;
-    // all nodes' forward or back-projection operands (24 or 16 B an entry), or on a tensor-core job,
-    // whose plain adjoint alone comes here, 8 B an entry and the nodes in slabs
-    p.xs = full ? x8 : std::max(std::min(x8, 64), (int)((size_t)X * 2 / 3 / 8 * 8));
-    p.xld = p.xs;
+    // all nodes' forward or back-projection operands (24 or 16 B an entry), or on a BF16 or split
+    // BF16 job the plain adjoint's alone (12 B)
+    p.xld = (X + 7) / 8 * 8;
     p.pstride = (size_t)N * p.xld;
     p.rld = (N + 7) / 8 * 8;
     const size_t deep = 2 * parts, planes = full ? 2 * deep : deep;
@@ -595,9 +592,8 @@ bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st
         return false;
     if (cudaMallocAsync(reinterpret_cast<void **>(&p.err), sizeof(unsigned), st) != cudaSuccess) return false;
     cudaMemsetAsync(p.err, 0, sizeof(unsigned), st);
-    const size_t cols = std::min(p.xs, X);
-    return make_map(&p.fmap, p.planes, cols, N, planes, p.xld, BK, BM, deep) &&
-           make_map(&p.amap, p.planes, cols, N, planes, p.xld, 64, BK, deep) &&
+    return make_map(&p.fmap, p.planes, X, N, planes, p.xld, BK, BM, deep) &&
+           make_map(&p.amap, p.planes, X, N, planes, p.xld, 64, BK, deep) &&
            make_map(&p.rmap, p.rs, N, N, deep, p.rld, BK, BN, deep) && (parts == 3 ? allow_smem<3>() : allow_smem<2>());
 }
 
@@ -611,12 +607,12 @@ void f32_free(F32Planes &p, cudaStream_t st)
 
 void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
-    synth<1>(p, tab, v, 0, p.X, f, c0, s);
+    synth<1>(p, tab, v, f, c0, s);
 }
 
 void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s)
 {
-    synth<2>(p, tab, nullptr, 0, p.X, f, c0, s);
+    synth<2>(p, tab, nullptr, f, c0, s);
 }
 
 void launch_forward_f32(F32Planes &p, int splits, float2 *part, cudaStream_t s)
@@ -675,8 +671,7 @@ int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *R, b
         rs_parts<false>(p, R, s);
     else
         rs_parts<true>(p, R, s);
-    GemmArgs g = bp_args(p, tab, gpart);
-    g.nx = p.X;
+    const GemmArgs g = bp_args(p, tab, gpart);
     const dim3 grd((unsigned)ET * ((p.X + BM - 1) / BM), 2);
     if (p.parts == 3)
         k_cgemm_f32<3, true, false><<<grd, THREADS, Form<3>::SMEM, s>>>(g);
@@ -687,23 +682,18 @@ int launch_backproject_f32(F32Planes &p, const TabEntry *tab, const float2 *R, b
     return 3;
 }
 
-// The plain adjoint's sum_{e,r} conj(G_e G_r) R_s: synthesis and contraction, slab by slab.
+// The plain adjoint's sum_{e,r} conj(G_e G_r) R_s: synthesis and contraction, all nodes at once (BF16
+// job, 48 transducers, 2,828 nodes: 22.6 us, 37 in two slabs of nodes; 24.7 as FP32 multiply-adds).
 int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *R, double f, double c0, float2 *gpart,
                        cudaStream_t s)
 {
     const int ET = (p.N + BN - 1) / BN;
-    int n = 1;
     rs_parts<true>(p, R, s);
-    for (int x0 = 0; x0 < p.X; x0 += p.xs, n += 2) {
-        GemmArgs g = bp_args(p, tab, gpart);
-        g.x0 = x0;
-        g.nx = std::min(p.xs, p.X - x0);
-        synth<0>(p, tab, nullptr, x0, g.nx, f, c0, s);
-        k_cgemm_f32<3, true, true><<<(unsigned)ET * ((g.nx + BM - 1) / BM), THREADS, Form<3>::SMEM, s>>>(g);   // parts == 3
-    }
-    if (ET == 1) return n;
+    synth<0>(p, tab, nullptr, f, c0, s);
+    k_cgemm_f32<3, true, true><<<(unsigned)ET * ((p.X + BM - 1) / BM), THREADS, Form<3>::SMEM, s>>>(bp_args(p, tab, gpart));
+    if (ET == 1) return 3;
     k_bp_sum<<<dim3((p.X + 255) / 256, 1), 256, 0, s>>>(p.bpart, ET, p.X, gpart);
-    return n + 1;
+    return 4;
 }
 
 }  // namespace rbx

@@ -30,7 +30,6 @@ struct rbx_job {
     bool raw = false;          // integration on the non-smoothed map (rbx_set_integration)
     int link_iters = 0;        // secant ray linking of the direct term, new rays per pair (0: off)
     bool linked_valid = false; // w.linked holds the linked rays of the current tables
-    bool dg_valid = false;     // w.dg holds the angular density of the current tables
     double abs_y = 0.0;
     Workspace w;
     int *d_count = nullptr;
@@ -97,7 +96,7 @@ static cudaError_t dalloc(T *&p, size_t n, cudaStream_t s)
 
 static void free_ws(Workspace &w, cudaStream_t s)
 {
-    void *ps[] = {w.hist, w.node2x, w.idx, w.rows, w.c, w.ns, w.tmp, w.fields, w.ns64, w.tmp64, w.tab, w.dg, w.exits, w.v, w.gdir, w.D, w.R, w.Rs, w.part, w.gpart, w.data, w.red, w.counters, w.alpha0, w.as64,
+    void *ps[] = {w.hist, w.node2x, w.idx, w.rows, w.c, w.ns, w.tmp, w.fields, w.ns64, w.tmp64, w.tab, w.exits, w.v, w.gdir, w.D, w.R, w.Rs, w.part, w.gpart, w.data, w.red, w.counters, w.alpha0, w.as64,
                   w.dmacc, w.linked, w.beta};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, s);
@@ -268,7 +267,6 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.tmp64, nxy);
     ALLOC(w.fields, nxy * kFieldStride);
     ALLOC(w.tab, NX);
-    ALLOC(w.dg, NX);
     ALLOC(w.exits, N * (N - 1));
     // FP32 jobs: the operands of both contractions; the others: those of the plain adjoint
     if (!f32_setup(w.f32, w.N, X, 3, g.precision == RBX_FP32, j->stream) ||
@@ -446,17 +444,6 @@ static rbx_status direct_green(rbx_job *j, double f, float2 *out)
     return RBX_OK;
 }
 
-// The angular density array w.dg (step a4), formed when rbx_get_tables first asks for it after
-// the tables changed; the operand syntheses form the same values from the tables themselves.
-static rbx_status ensure_dgamma(rbx_job *j)
-{
-    if (j->dg_valid) return RBX_OK;
-    launch_dgamma(j->w.tab, j->w.dg, j->w.N, j->w.X, j->stream);
-    LAUNCHED(j, 1);
-    j->dg_valid = true;
-    return RBX_OK;
-}
-
 // The trace of step a2/a3 in three parts, so that the batched form can run the middle one
 // for all its jobs as one grouped launch: the fields and the cleared tables, the ray trace
 // with its rasteriser, and the tables' bookkeeping.
@@ -487,7 +474,7 @@ static rbx_status trace_launch(rbx_job *j)
 static rbx_status trace_end(rbx_job *j)
 {
     rbx_status st;
-    j->linked_valid = j->dg_valid = false;
+    j->linked_valid = false;
     if ((st = record(j, EV_TRACE))) return st;
     if ((st = record(j, EV_TABLES))) return st;
     j->has_tables = true;
@@ -514,7 +501,7 @@ rbx_status rbx_set_tables(rbx_job *j, const float *T, const float *a, const floa
     size_t n = (size_t)w.N * w.X;
     CUDA_TRY(j, cudaMemsetAsync(w.counters, 0, 4 * sizeof(unsigned long long), j->stream));
     launch_set_tables(T, a, gam, K, w.tab, n, w.counters, j->stream);
-    j->linked_valid = j->dg_valid = false;
+    j->linked_valid = false;
     CUDA_TRY(j, cudaMemcpyAsync(w.exits, exits, sizeof(float4) * (size_t)w.N * (w.N - 1), cudaMemcpyDeviceToDevice,
                                 j->stream));
     LAUNCHED(j, 1);
@@ -532,10 +519,9 @@ rbx_status rbx_get_tables(rbx_job *j, float *T, float *a, float *gam, uint8_t *K
         launch_get_tables(w.tab, T, a, gam, K, n, j->stream);
         LAUNCHED(j, 1);
     }
-    if (dg) {
-        rbx_status st = ensure_dgamma(j);
-        if (st) return st;
-        CUDA_TRY(j, cudaMemcpyAsync(dg, w.dg, sizeof(float) * n, cudaMemcpyDeviceToDevice, j->stream));
+    if (dg) {   // angular density (step a4); the operand syntheses form the same values
+        launch_dgamma(w.tab, dg, w.N, w.X, j->stream);
+        LAUNCHED(j, 1);
     }
     if (exits)
         CUDA_TRY(j, cudaMemcpyAsync(exits, w.exits, sizeof(float4) * (size_t)w.N * (w.N - 1), cudaMemcpyDeviceToDevice,
@@ -1258,9 +1244,9 @@ size_t job_bytes_estimate(const rbx_geometry &g, int nf)
     const double r = g.mask_radius / g.dx;
     const size_t X = (size_t)(3.14159265358979 * r * r + 6.3 * r + 16);
     const size_t N = (size_t)g.n_xducers, NX = N * X, nxy = (size_t)g.nx * g.ny, NN = N * N;
-    size_t b = NX * (16 + 4 + 8);                                 // tables, angular density, FP32 operand planes
+    size_t b = NX * (16 + 12);                                    // tables, the plain adjoint's planes
     if (g.precision == RBX_FP32 || g.precision == RBX_BF16X3) {
-        b += NX * 16;                                             // (24 B an entry in all; split BF16 8 + 16)
+        b += NX * 16;                                             // (FP32 24 B an entry in all; split BF16 12 + 16)
     } else {
         const size_t Np = (N + 127) / 128 * 128, Xk = (X + 63) / 64 * 64, Xm = (X + 127) / 128 * 128;
         b += (4 * Np * Xk + 6 * Xm * Np + 2 * Np * Np) * 2 + (Np / 128) * Xm * 8;

@@ -79,11 +79,10 @@ struct TcPlanes {
 // Operands of the FP32-accurate (or split BF16) contractions of one job: values as three (two) BF16
 // parts, their TMA descriptors and the back-projection partials (k_gemm_f32.cu).
 struct F32Planes {
-    int N = 0, X = 0, xs = 0, xld = 0, rld = 0;   // xs nodes per slab, rows of xld (operands) and rld (R_s)
+    int N = 0, X = 0, xld = 0, rld = 0;   // rows of xld (operands) and rld (R_s)
     int parts = 3;
-    bool full = false;         // both operand sets of all nodes ; else the plain adjoint's slab
     size_t pstride = 0;
-    void *planes = nullptr;    // [4 parts, or 2 parts of a slab][N][xld] bf16
+    void *planes = nullptr;    // [4 parts, or 2 parts (plain adjoint alone)][N][xld] bf16
     void *rs = nullptr;        // [2 parts][N][rld] bf16
     float2 *bpart = nullptr;   // [stacks][emitter tiles][X]; nullptr with one emitter tile
     unsigned *err = nullptr;   // bounded-wait timeouts
@@ -98,7 +97,6 @@ struct Workspace {
     float *c = nullptr, *ns = nullptr, *tmp = nullptr, *fields = nullptr;
     double *ns64 = nullptr, *tmp64 = nullptr;
     TabEntry *tab = nullptr;
-    float *dg = nullptr;
     float4 *exits = nullptr;
     float2 *v = nullptr;        // Born weight Upsilon_m dA (m - m_s) per mask node (complex when lossy)
     float *alpha0 = nullptr;    // absorption map alpha0 [ny][nx], Np (rad/s)^-y m^-1 (lossy jobs only)

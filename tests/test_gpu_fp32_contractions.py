@@ -1,6 +1,6 @@
 """The FP32 contractions (three BF16 parts per operand on the tensor cores) at the edges of their
 tiles: transducer counts around one and two 128-wide tiles and 32-wide K chunks, odd node counts,
-and the plain adjoint of a tensor-core job, which goes through the nodes in slabs; and the forward that
+and the plain adjoint of a BF16 job; and the forward that
 allocates nothing (its operands formed in the kernel, one CTA or a cluster per tile).
 
 Reference: the sums in complex128 on the same FP32 tables. Tolerance: an operand carries about six
