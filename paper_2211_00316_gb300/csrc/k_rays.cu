@@ -1046,12 +1046,19 @@ void launch_uniform_radius(const float *fields, const RayParams &p, unsigned lon
     k_uniform_radius<<<(n + 255) / 256, 256, 0, s>>>(reinterpret_cast<const float4 *>(fields), p, ru);
 }
 
-// Lanes per ray: the most (up to 8) whose warps the GPU still holds at once (152 SMs x 20). One lane,
-// and k_trace_raster, from about 215 transducers on.
-static int lanes_per_ray(int N, int nwarps)
+// Lanes per ray: the most (up to 8) whose warps the GPU still holds at once (152 SMs x 20) and whose
+// block keeps its queues and `rows_bytes` of mask rows in the 48 KB of shared memory that a launch
+// has without asking for more (eight lanes to 2,173 grid rows, four to 2,558). One lane, and
+// k_trace_raster, from about 215 transducers on.
+static int lanes_per_ray(int N, int nwarps, size_t rows_bytes)
 {
     int l = 1;
     while (l < 8 && (size_t)N * nwarps * 2 * l <= 3040) l *= 2;
+    auto fits = [&](int lanes) {
+        const size_t queues = lanes == 8 ? sizeof(WideShared<8>) : lanes == 4 ? sizeof(WideShared<4>) : sizeof(WideShared<2>);
+        return queues + rows_bytes <= 48 * 1024;
+    };
+    while (l > 1 && !fits(l)) l /= 2;
     return l;
 }
 
@@ -1064,7 +1071,7 @@ void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, f
     int nwarps = (p.N - 2 + 30) / 31;
     dim3 grd((p.N + kFansPerBlock - 1) / kFansPerBlock, nwarps);
     const size_t sm = (size_t)p.ny * sizeof(int4);
-    const int lpr = lanes_per_ray(p.N, nwarps);
+    const int lpr = lanes_per_ray(p.N, nwarps, sm);
     if (lpr > 1) {
         auto wide = [&](auto lp) {
             constexpr int L = decltype(lp)::value;
