@@ -1046,14 +1046,24 @@ void launch_uniform_radius(const float *fields, const RayParams &p, unsigned lon
     k_uniform_radius<<<(n + 255) / 256, 256, 0, s>>>(reinterpret_cast<const float4 *>(fields), p, ru);
 }
 
-// Lanes per ray: the most (up to 8) whose warps the GPU still holds at once (152 SMs x 20) and whose
-// block keeps its queues and `rows_bytes` of mask rows in the 48 KB of shared memory that a launch
+// Lanes per ray: the most (up to 8) with which the traces running together (load: their warps with one
+// lane per ray; own: this trace's) stay within 3,040 warps, or 1,520 beside other jobs. Every lane of a ray
+// integrates it, which costs nothing only while the GPU has issue slots to spare; beside other jobs
+// their contractions take some of those. The GPU holds 2,432 warps of k_trace_wide (16 per SM), 3,040
+// of k_trace_raster: that the line lies there is what was measured. ms of one trace alone with 1 / 2 / 4 / 8
+// lanes: 64 transducers on 102 x 102 0.507 / 0.484 / 0.406 / 0.378, 128 on 160 x 160 0.806 / 0.807 / 0.755 /
+// 1.069, 152 on 181 x 181 0.915 / 0.885 / 0.830 / 1.407, 217 on 240 x 240 1.356 / 1.333 / 1.931 / 3.349. Together:
+// four of 64 on 96 x 96 0.497 / 0.494 / 0.487 / 0.648, eight 0.561 / 0.604 / 0.735 / 1.229, 24 of 128 on
+// 160 x 160 4.0 with one lane and 11.2 with the four of a ring alone; a batch of three updates each, eight of
+// 64: 1.98 with one lane, 2.53 with two.
+// The block keeps its queues and `rows_bytes` of mask rows in the 48 KB of shared memory that a launch
 // has without asking for more (eight lanes to 2,173 grid rows, four to 2,558). One lane, and
 // k_trace_raster, from about 215 transducers on.
-static int lanes_per_ray(int N, int nwarps, size_t rows_bytes)
+static int lanes_per_ray(size_t load, size_t own, size_t rows_bytes)
 {
+    const size_t most = load > own ? 1520 : 3040;
     int l = 1;
-    while (l < 8 && (size_t)N * nwarps * 2 * l <= 3040) l *= 2;
+    while (l < 8 && load * 2 * l <= most) l *= 2;
     auto fits = [&](int lanes) {
         const size_t queues = lanes == 8 ? sizeof(WideShared<8>) : lanes == 4 ? sizeof(WideShared<4>) : sizeof(WideShared<2>);
         return queues + rows_bytes <= 48 * 1024;
@@ -1063,7 +1073,7 @@ static int lanes_per_ray(int N, int nwarps, size_t rows_bytes)
 }
 
 void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, float4 *exits, const RayParams &p,
-                         unsigned long long *counters, bool lossy, bool raw, cudaStream_t s)
+                         unsigned long long *counters, size_t load, bool lossy, bool raw, cudaStream_t s)
 {
     // the longest warps of every fan first: the blocks that start last, and those that share
     // an SM when the grid is a single wave, then differ least (1024 transducers on 512 x 512:
@@ -1071,7 +1081,7 @@ void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, f
     int nwarps = (p.N - 2 + 30) / 31;
     dim3 grd((p.N + kFansPerBlock - 1) / kFansPerBlock, nwarps);
     const size_t sm = (size_t)p.ny * sizeof(int4);
-    const int lpr = lanes_per_ray(p.N, nwarps, sm);
+    const int lpr = lanes_per_ray(load, (size_t)p.N * nwarps, sm);
     if (lpr > 1) {
         auto wide = [&](auto lp) {
             constexpr int L = decltype(lp)::value;
@@ -1109,6 +1119,8 @@ void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, f
     else
         go(std::integral_constant<int, 20>{});
 }
+
+size_t trace_warps(int N) { return (size_t)N * ((N - 2 + 30) / 31); }
 
 int trace_items(int N, int *nwarps)
 {

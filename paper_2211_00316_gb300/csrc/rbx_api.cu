@@ -3,6 +3,7 @@
 #include "rbx_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -43,6 +44,56 @@ struct rbx_job {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_in_free = nullptr, ev_in_ready = nullptr;
     long long launches = 0;
+    int load_dev = -1;         // device whose g_load counts this job's trace (set with the geometry)
+    bool waits = false;        // inside a call that traces and waits for the update (Waiting)
+};
+
+// Warps (one lane per ray) of the traces that may run together on a device: those of all jobs that
+// hold a geometry, and those of the jobs inside a call that returns when its update is done. A call of
+// the second kind shares the GPU with the others of its kind (other host threads); one that only
+// queues work may share it with every job. The choice of lanes per ray does not change a result.
+struct TraceLoad {
+    std::atomic<size_t> held{0}, waiting{0};
+};
+static TraceLoad g_load[64];
+
+static void hold_load(rbx_job *j)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+    j->load_dev = dev;
+    g_load[dev].held += trace_warps(j->g.n_xducers);
+}
+
+static void drop_load(rbx_job *j)
+{
+    if (j->load_dev >= 0) g_load[j->load_dev].held -= trace_warps(j->g.n_xducers);
+    j->load_dev = -1;
+}
+
+static size_t trace_load(const rbx_job *j)
+{
+    const size_t own = trace_warps(j->g.n_xducers);
+    if (j->load_dev < 0) return own;
+    const TraceLoad &l = g_load[j->load_dev];
+    return std::max(own, (j->waits ? l.waiting : l.held).load());
+}
+
+// Marks a job as waiting for the update it traces, from here to the end of the scope.
+struct Waiting {
+    rbx_job *j;
+    explicit Waiting(rbx_job *job) : j(job)
+    {
+        if (j->load_dev < 0) return;
+        g_load[j->load_dev].waiting += trace_warps(j->g.n_xducers);
+        j->waits = true;
+    }
+    ~Waiting()
+    {
+        if (!j->waits) return;
+        g_load[j->load_dev].waiting -= trace_warps(j->g.n_xducers);
+        j->waits = false;
+    }
 };
 
 static rbx_status fail(rbx_job *j, rbx_status st, const char *fmt, ...)
@@ -159,6 +210,7 @@ rbx_status rbx_destroy(rbx_job *j)
 {
     if (!j) return RBX_EINVAL;
     cudaStreamSynchronize(j->stream);
+    drop_load(j);
     free_ws(j->w, j->stream);
     if (j->d_count) cudaFreeAsync(j->d_count, j->stream);
     cudaStreamSynchronize(j->stream);
@@ -231,6 +283,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     }
 
     CUDA_TRY(j, cudaStreamSynchronize(j->stream));
+    drop_load(j);
     free_ws(j->w, j->stream);
     keep_pool_memory();
     j->has_geom = j->has_tables = j->ns_valid = j->lossy = j->raw = false;
@@ -313,6 +366,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     CUDA_TRY(j, cudaStreamSynchronize(j->stream));
     j->g = g;
     j->has_geom = true;
+    hold_load(j);
     return RBX_OK;
 }
 
@@ -466,7 +520,8 @@ static rbx_status trace_begin(rbx_job *j, double f)
 static rbx_status trace_launch(rbx_job *j)
 {
     Workspace &w = j->w;
-    launch_trace_raster(w.fields, w.rows, w.tab, w.exits, ray_params(j), w.counters, j->lossy, j->raw, j->stream);
+    launch_trace_raster(w.fields, w.rows, w.tab, w.exits, ray_params(j), w.counters, trace_load(j), j->lossy, j->raw,
+                        j->stream);
     LAUNCHED(j, 1);
     return RBX_OK;
 }
@@ -810,6 +865,7 @@ rbx_status rbx_update_frequency(rbx_job *j, double f, double df, const void *dat
     if (!j || !data_dev) return RBX_EINVAL;
     NEED(j, j->has_geom, RBX_ESTATE, "rbx_update_frequency before rbx_set_geometry");
     NEED(j, !bad_freq(f) && std::isfinite(df) && df > 0, RBX_EINVAL, "frequency and spacing must be finite and > 0");
+    Waiting waiting(j);
     long long l0 = j->launches;
     rbx_status st = rbx_trace_rays(j, f);
     if (st) return st;
@@ -852,6 +908,7 @@ rbx_status rbx_update_set(rbx_job *j, const double *freqs, int nf, double df, co
     NEED(j, std::isfinite(df) && df > 0, RBX_EINVAL, "frequency spacing must be finite and > 0");
     for (int k = 0; k < nf; k++) NEED(j, !bad_freq(freqs[k]), RBX_EINVAL, "frequencies must be finite and > 0");
     if (nf == 1) return rbx_update_frequency(j, freqs[0], df, data_dev, out);
+    Waiting waiting(j);
     Workspace &w = j->w;
     long long l0 = j->launches;
     if (!w.dmacc && dalloc(w.dmacc, (size_t)w.X, j->stream) != cudaSuccess) {
@@ -899,6 +956,7 @@ rbx_status rbx_update_frequency_host(rbx_job *j, double f, double df, const void
     CUDA_TRY(j, cudaStreamWaitEvent(j->copy_stream, j->ev_in_free, 0));
     CUDA_TRY(j, cudaMemcpyAsync(j->w.data, data_host, sizeof(float2) * nn, cudaMemcpyHostToDevice, j->copy_stream));
     CUDA_TRY(j, cudaEventRecord(j->ev_in_ready, j->copy_stream));
+    Waiting waiting(j);
     const long long l0 = j->launches;
     rbx_status st = rbx_trace_rays(j, f);
     if (st) {

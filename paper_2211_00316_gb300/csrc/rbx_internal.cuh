@@ -135,7 +135,9 @@ void launch_fill(float *p, float v, size_t n, cudaStream_t s);
 // k_rays.cu
 void launch_uniform_radius(const float *fields, const RayParams &p, unsigned long long *ru, cudaStream_t s);
 void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, float4 *exits, const RayParams &p,
-                         unsigned long long *counters, bool lossy, bool raw, cudaStream_t s);
+                         unsigned long long *counters, size_t load, bool lossy, bool raw, cudaStream_t s);
+// Warps of a ring's trace with one lane per ray
+size_t trace_warps(int N);
 // One job of a persistent grouped trace (the batched form): its buffers and ray parameters,
 // and the range of work items it owns, [item0, item0 + nwarps * ceil(N / 4)).
 struct TraceJob {
