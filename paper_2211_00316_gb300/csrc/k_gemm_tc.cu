@@ -542,6 +542,8 @@ __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_g
 constexpr int kSynE = 64, kSynThreads = 512;
 constexpr int kSynSlots = (kSynE + 2) * 32;   // slot s holds row (e0 - 1 + s) mod N, nodes x0 .. x0 + 31
 
+constexpr size_t SYN_SMEM = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * (kSynE + 2) * sizeof(__nv_bfloat16);
+
 // Queue the copies of tile t's table entries into buf (entries past the last node are not
 // copied; the consumer treats them as uncovered).
 __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab, int N, int X, int XT, int t,
@@ -724,6 +726,21 @@ bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, 
 
 // ---------------------------------------------------------------- API used by rbx_api.cu
 
+// Shared memory and persistent grid of k_synth_tc<FWD>, for the current device: the opt-in above 48 KB
+// belongs to a device's context, so every job makes it for the one it lives on.
+template <bool FWD>
+static bool synth_setup(TcPlanes &p)
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaFuncSetAttribute(k_synth_tc<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SYN_SMEM) != cudaSuccess ||
+        cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, kSynThreads, SYN_SMEM) != cudaSuccess)
+        return false;
+    p.syn_blocks[FWD] = sms * std::max(per_sm, 1);
+    return true;
+}
+
 bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t st)
 {
     p.N = N;
@@ -773,7 +790,8 @@ bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t st)
     ok = cudaFuncSetAttribute(k_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) == cudaSuccess &&
          cudaFuncSetAttribute(k_forward_tc_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) ==
              cudaSuccess &&
-         cudaFuncSetAttribute(k_backproject_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) == cudaSuccess;
+         cudaFuncSetAttribute(k_backproject_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) == cudaSuccess &&
+         synth_setup<false>(p) && synth_setup<true>(p);
     p.ready = ok;
     return ok;
 }
@@ -953,32 +971,13 @@ int launch_forward_tc(TcPlanes &p, float2 *part, cudaStream_t s)
     return p.fwd_splits;
 }
 
-// Shared memory and persistent grid of k_synth_tc<FWD> (set up once per instance).
-template <bool FWD>
-static int synth_grid(size_t &smem)
-{
-    smem = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * (kSynE + 2) * sizeof(__nv_bfloat16);
-    static int blocks = 0;
-    if (blocks == 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_synth_tc<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, kSynThreads, smem);
-        blocks = sms * (per_sm > 0 ? per_sm : 1);
-    }
-    return blocks;
-}
-
 template <bool FWD>
 static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
     const float fhi = (float)f, flo = (float)(f - (double)fhi);
     const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + kSynE - 1) / kSynE);
-    size_t smem = 0;
-    int grd = synth_grid<FWD>(smem);
-    if (grd > ntiles) grd = ntiles;
-    k_synth_tc<FWD><<<grd, kSynThreads, smem, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
+    const int grd = std::min(p.syn_blocks[FWD], ntiles);
+    k_synth_tc<FWD><<<grd, kSynThreads, SYN_SMEM, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
                                                   static_cast<__nv_bfloat16 *>(p.bplanes), v, FWD ? p.Xpad : 0,
                                                   FWD ? p.fwd_pstride : 0,
                                                   FWD ? static_cast<__nv_bfloat16 *>(p.fplanes) : nullptr, XT, ntiles);

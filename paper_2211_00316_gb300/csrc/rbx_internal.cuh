@@ -64,6 +64,7 @@ struct TcPlanes {
     int fwd_splits = 1, fwd_kper = 1;
     int fwd_max_splits = 1;    // largest K split the autotuner may pick (sizes the partials)
     int tuned = 0;             // candidates timed for this job (0: heuristic or cached choice)
+    int syn_blocks[2] = {1, 1};   // persistent grid of the back-projection's synthesis, and of both contractions'
     bool fwd_fused = false;    // the forward forms its operands from the tables (k_forward_tc_fused)
     float tune_ms[4] = {0.f, 0.f, 0.f, 0.f};   // tuner's times: both synthesis passes, forward GEMM,
                                                // back-projection synthesis alone, fused forward
