@@ -288,7 +288,8 @@ rbx_status rbx_reconstruct(rbx_job *job, const double *freqs_hz, int nf, const v
  * rbx_forward. The first call on each
  * device looks up that array's device address (it may load the module): make it before any
  * stream capture. All calls share the array; calls that overlap on the GPU race and must be
- * serialised by the caller. Work is queued on cuda_stream (NULL: legacy default stream).
+ * serialised by the caller. A bounded wait that gives up leaves D_dev not a number (the call has
+ * returned by then). Work is queued on cuda_stream (NULL: legacy default stream).
  * err (errlen bytes, may be NULL) receives a message, "" on success. */
 rbx_status rbx_forward_noalloc(const float *T_dev, const float *a_dev, const uint8_t *K_dev, const float *v_dev,
                                int n_xducers, int n_nodes, double freq_hz, double c0, void *D_dev, void *cuda_stream,
@@ -392,15 +393,22 @@ rbx_status rbx_pool_usage(size_t *used, size_t *reserved, int trim);
 
 /* Diagnostic of the failure handling (the paper has no counterpart). Every wait of the
  * tensor-core kernels on a barrier or a copy is bounded: after one second of wall time
- * the kernel records a timeout, stops and frees what it holds, and the call returns
- * RBX_ETIMEOUT. This runs one kernel on the current device whose single thread waits, with
+ * the kernel records a timeout, stops and frees what it holds. An update then returns
+ * RBX_ETIMEOUT and leaves the model as it was. rbx_forward, rbx_predict and rbx_adjoint, which
+ * only queue work, write results that are not a number, and so do the job's later ones until
+ * rbx_synchronize or an update has returned RBX_ETIMEOUT. This runs one kernel on the current device whose single thread waits, with
  * that same bound, on a barrier that nothing ever signals. *timed_out = 1 when the wait gave
  * up as it should (the expected result), 0 if the barrier completed. The call allocates and
  * frees 4 bytes of device memory, synchronises the device, takes about one second and leaves
  * the CUDA context usable. */
 rbx_status rbx_selftest_bounded_wait(int *timed_out);
 
-/* Wait for all work queued on the job's stream. */
+/* The same wait on the job's stream, recorded where the job's contractions record theirs: what
+ * follows behaves as if one of them had given up. Returns at once (the kernel takes about a second). */
+rbx_status rbx_selftest_job_timeout(rbx_job *job);
+
+/* Wait for all work queued on the job's stream. RBX_ETIMEOUT when a wait of a forward, predict or
+ * adjoint call since the last report gave up (its results are not a number); reported once. */
 rbx_status rbx_synchronize(rbx_job *job);
 
 /* Wait for the job's stream, then free the job's device memory. */

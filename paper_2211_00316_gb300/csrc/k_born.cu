@@ -63,8 +63,10 @@ void launch_born_weights_dm(const float *dm, const float *c, const int *idx, int
     k_born_dm<<<(X + 255) / 256, 256, 0, s>>>(dm, c, idx, X, w, dA, ab.alpha0, wy, tn, v);
 }
 
-// D[e,r] = D[r,e] = sum over splits (fixed order) of the upper-triangle partials.
-__global__ void k_forward_reduce(const float2 *__restrict__ part, int N, int splits, float2 *__restrict__ D)
+// D[e,r] = D[r,e] = sum over splits (fixed order) of the upper-triangle partials; not a number when a wait
+// of the contraction gave up (*err), so that a call whose status is not waited for shows it.
+__global__ void k_forward_reduce(const float2 *__restrict__ part, int N, int splits, const unsigned *__restrict__ err,
+                                 float2 *__restrict__ D)
 {
     size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= (size_t)N * N) return;
@@ -77,13 +79,15 @@ __global__ void k_forward_reduce(const float2 *__restrict__ part, int N, int spl
         acc.x += p.x;
         acc.y += p.y;
     }
+    if (err && *err) acc.x = acc.y = __int_as_float(0x7fffffff);
     D[(size_t)e * N + r] = acc;
     D[(size_t)r * N + e] = acc;
 }
 
 // The same with four lanes per entry, each summing every fourth split: a small D with many splits
 // is one chain of loads otherwise (64 transducers, 54 splits: 15 -> 7 us).
-__global__ void k_forward_reduce4(const float2 *__restrict__ part, int N, int splits, float2 *__restrict__ D)
+__global__ void k_forward_reduce4(const float2 *__restrict__ part, int N, int splits, const unsigned *__restrict__ err,
+                                  float2 *__restrict__ D)
 {
     const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, i = t >> 2;
     const int e = (int)(i / N), r = (int)(i % N);
@@ -102,18 +106,19 @@ __global__ void k_forward_reduce4(const float2 *__restrict__ part, int N, int sp
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
     }
     if ((t & 3) == 0 && i < (size_t)N * N && e <= r) {
+        if (err && *err) acc.x = acc.y = __int_as_float(0x7fffffff);
         D[(size_t)e * N + r] = acc;
         D[(size_t)r * N + e] = acc;
     }
 }
 
-void launch_forward_reduce(const float2 *part, int N, int splits, float2 *D, cudaStream_t s)
+void launch_forward_reduce(const float2 *part, int N, int splits, const unsigned *err, float2 *D, cudaStream_t s)
 {
     size_t n = (size_t)N * N;
     if (splits > 16 && n <= 65536)   // beyond, one lane per entry fills the GPU by itself
-        k_forward_reduce4<<<(unsigned)((4 * n + 255) / 256), 256, 0, s>>>(part, N, splits, D);
+        k_forward_reduce4<<<(unsigned)((4 * n + 255) / 256), 256, 0, s>>>(part, N, splits, err, D);
     else
-        k_forward_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, N, splits, D);
+        k_forward_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, N, splits, err, D);
 }
 
 }  // namespace rbx

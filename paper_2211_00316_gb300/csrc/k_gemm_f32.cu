@@ -573,8 +573,9 @@ static bool allow_smem()
                                  (int)Form<3>::SMEM) == cudaSuccess);
 }
 
-bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st)
+bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, unsigned *err, cudaStream_t st)
 {
+    p.err = err;
     p.N = N;
     p.X = X;
     p.parts = parts;
@@ -590,8 +591,6 @@ bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st
     if (ET > 1 &&   // with one emitter tile the partial row-dots are the result
         cudaMallocAsync(reinterpret_cast<void **>(&p.bpart), (full ? 2 : 1) * ET * X * sizeof(float2), st) != cudaSuccess)
         return false;
-    if (cudaMallocAsync(reinterpret_cast<void **>(&p.err), sizeof(unsigned), st) != cudaSuccess) return false;
-    cudaMemsetAsync(p.err, 0, sizeof(unsigned), st);
     return make_map(&p.fmap, p.planes, X, N, planes, p.xld, BK, BM, deep) &&
            make_map(&p.amap, p.planes, X, N, planes, p.xld, 64, BK, deep) &&
            make_map(&p.rmap, p.rs, N, N, deep, p.rld, BK, BN, deep) && (parts == 3 ? allow_smem<3>() : allow_smem<2>());
@@ -599,7 +598,7 @@ bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t st
 
 void f32_free(F32Planes &p, cudaStream_t st)
 {
-    void *ps[] = {p.planes, p.rs, p.bpart, p.err};
+    void *ps[] = {p.planes, p.rs, p.bpart};
     for (void *q : ps)
         if (q) cudaFreeAsync(q, st);
     p = F32Planes{};

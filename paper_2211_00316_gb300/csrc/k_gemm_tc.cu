@@ -741,8 +741,9 @@ static bool synth_setup(TcPlanes &p)
     return true;
 }
 
-bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t st)
+bool tc_setup(TcPlanes &p, int N, int X, unsigned *err, cudaStream_t st)
 {
+    p.err = err;
     p.N = N;
     p.X = X;
     p.Npad = (N + BM - 1) / BM * BM;
@@ -773,11 +774,9 @@ bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t st)
     if (cudaMallocAsync(reinterpret_cast<void **>(&p.bpart), (size_t)(p.Npad / BN) * p.Xp * sizeof(float2), st) !=
         cudaSuccess)
         return false;
-    if (cudaMallocAsync(reinterpret_cast<void **>(&p.err), sizeof(unsigned), st) != cudaSuccess) return false;
     cudaMemsetAsync(p.fplanes, 0, fbytes, st);
     cudaMemsetAsync(p.bplanes, 0, bbytes, st);
     cudaMemsetAsync(p.rsplanes, 0, rbytes, st);
-    cudaMemsetAsync(p.err, 0, sizeof(unsigned), st);
     const __nv_bfloat16 *f = static_cast<const __nv_bfloat16 *>(p.fplanes);
     const __nv_bfloat16 *b = static_cast<const __nv_bfloat16 *>(p.bplanes);
     const __nv_bfloat16 *r = static_cast<const __nv_bfloat16 *>(p.rsplanes);
@@ -934,7 +933,7 @@ bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream
 
 void tc_free(TcPlanes &p, cudaStream_t st)
 {
-    void *ps[] = {p.fplanes, p.bplanes, p.rsplanes, p.bpart, p.err};
+    void *ps[] = {p.fplanes, p.bplanes, p.rsplanes, p.bpart};
     for (void *q : ps)
         if (q) cudaFreeAsync(q, st);
     p = TcPlanes{};
@@ -994,14 +993,14 @@ void launch_synth_both_tc(TcPlanes &p, const TabEntry *tab, const float2 *v, dou
 }
 
 // One thread waits, with the bound every tensor-core kernel uses, on an mbarrier that nothing
-// signals: flag = 1 when the wait gave up.
+// signals: flag |= 1 when the wait gave up.
 __global__ void k_wait_selftest(unsigned *flag)
 {
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         fence_mbar_init();
-        *flag = mbar_wait(&bar, 0) ? 0u : 1u;
+        if (!mbar_wait(&bar, 0)) atomicOr(flag, 1u);
     }
 }
 

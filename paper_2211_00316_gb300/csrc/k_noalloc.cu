@@ -391,7 +391,7 @@ extern "C" rbx_status rbx_forward_noalloc(const float *T_dev, const float *a_dev
         seterr(err, errlen, buf);
         return RBX_ECUDA;
     }
-    launch_forward_reduce(scratch, N, splits, static_cast<float2 *>(D_dev), s);
+    launch_forward_reduce(scratch, N, splits, nullptr, static_cast<float2 *>(D_dev), s);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         char buf[256];

@@ -103,8 +103,9 @@ void launch_symmetrize(const float2 *R, int N, float2 *Rs, cudaStream_t s)
 
 // out[x] = scale * (g0 + s g1) (mode 0, s = -1 or +1 by weight_mode, scale = 2)
 //        = scale * g0          (mode 1, scale = omega^2 dA)
+// Not a number when a wait of the contraction gave up (*err), as in k_forward_reduce.
 __global__ void k_combine(const float2 *__restrict__ gpart, int X, int mode, float sgn, double scale,
-                          float2 *__restrict__ out)
+                          const unsigned *__restrict__ err, float2 *__restrict__ out)
 {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= X) return;
@@ -115,35 +116,37 @@ __global__ void k_combine(const float2 *__restrict__ gpart, int X, int mode, flo
         re += sgn * (double)g1.x;
         im += sgn * (double)g1.y;
     }
+    if (*err) re = im = nan("");
     out[x] = make_float2((float)(scale * re), (float)(scale * im));
 }
 
-void launch_combine_adjoint(const float2 *gpart, int X, int mode, int weight_mode, double scale, float2 *out,
-                            cudaStream_t s)
+void launch_combine_adjoint(const float2 *gpart, int X, int mode, int weight_mode, double scale, const unsigned *err,
+                            float2 *out, cudaStream_t s)
 {
-    k_combine<<<(X + 255) / 256, 256, 0, s>>>(gpart, X, mode, weight_mode == 0 ? -1.f : 1.f, scale, out);
+    k_combine<<<(X + 255) / 256, 256, 0, s>>>(gpart, X, mode, weight_mode == 0 ? -1.f : 1.f, scale, err, out);
 }
 
 // plain adjoint on a lossy medium: out[x] = dA conj(Upsilon_m) g0[x], Upsilon_m = omega c k~
 __global__ void k_combine_lossy(const float2 *__restrict__ gpart, const float *__restrict__ c,
                                 const float *__restrict__ alpha0, const int *__restrict__ idx, int X, double w,
-                                double wy, double tn, double dA, float2 *__restrict__ out)
+                                double wy, double tn, double dA, const unsigned *__restrict__ err,
+                                float2 *__restrict__ out)
 {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= X) return;
     const int k = idx[x];
     const double cc = c[k], al = wy * (double)alpha0[k];
     const double ur = w * w + w * cc * al * tn, ui = -w * cc * al;       // conj(Upsilon_m)
-    const double gr = gpart[x].x, gi = gpart[x].y;
+    const double gr = *err ? nan("") : (double)gpart[x].x, gi = gpart[x].y;
     out[x] = make_float2((float)(dA * (ur * gr - ui * gi)), (float)(dA * (ur * gi + ui * gr)));
 }
 
 void launch_combine_adjoint_lossy(const float2 *gpart, const float *c, const int *idx, int X, double f, double dA,
-                                  const Lossy &ab, float2 *out, cudaStream_t s)
+                                  const Lossy &ab, const unsigned *err, float2 *out, cudaStream_t s)
 {
     const double PI = 3.14159265358979323846, w = 2 * PI * f;
     k_combine_lossy<<<(X + 255) / 256, 256, 0, s>>>(gpart, c, ab.alpha0, idx, X, w, pow(w, ab.y),
-                                                    tan(PI * ab.y / 2), dA, out);
+                                                    tan(PI * ab.y / 2), dA, err, out);
 }
 
 // red layout (nb = update blocks): [0,nb) sum dc^2, [nb,2nb) max |dc|, [2nb,3nb) sum dm^2,
@@ -157,12 +160,12 @@ __global__ __launch_bounds__(RB) void k_update(const float2 *__restrict__ gpart,
                                                float *__restrict__ c, double *__restrict__ red,
                                                unsigned long long *counters, const float *__restrict__ alpha0,
                                                double w, double y, double wy, double tn, double *__restrict__ acc,
-                                               int mode)
+                                               int mode, const unsigned *__restrict__ err)
 {
     __shared__ double sh[RB];
     int k = blockIdx.x * RB + threadIdx.x;
     double dc2 = 0, dcm = 0, dm2 = 0;
-    if (k < nxy) {
+    if (k < nxy && !*err) {   // where a wait of a contraction gave up, the model stays
         int xi = node2x[k];
         if (xi < 0) {
             c[k] = c0;
@@ -234,7 +237,7 @@ __global__ __launch_bounds__(RB) void k_final_update(const double *__restrict__ 
 
 void launch_update(const float2 *gpart, const int *node2x, int nx, int ny, int X, int weight_mode, double f,
                    double df, double tau, double c0, float *c, double *red, unsigned long long *counters,
-                   const Lossy &ab, double *acc, int mode, cudaStream_t s)
+                   const Lossy &ab, double *acc, int mode, const unsigned *err, cudaStream_t s)
 {
     const double PI = 3.14159265358979323846;
     double w = 2 * PI * f, dw = 2 * PI * df;
@@ -242,7 +245,7 @@ void launch_update(const float2 *gpart, const int *node2x, int nx, int ny, int X
     int nb = update_blocks(nx, ny);
     const double wy = ab.alpha0 ? pow(w, ab.y) : 0.0, tn = ab.alpha0 ? tan(PI * ab.y / 2) : 0.0;
     k_update<<<nb, RB, 0, s>>>(gpart, node2x, X, nx * ny, weight_mode == 0 ? -1.f : 1.f, pref / w, tau, (float)c0, c,
-                               red, counters, ab.alpha0, w, ab.y, wy, tn, acc, mode);
+                               red, counters, ab.alpha0, w, ab.y, wy, tn, acc, mode, err);
     k_final_update<<<1, RB, 0, s>>>(red, nb, red + 3 * nb);
 }
 
@@ -270,9 +273,9 @@ void launch_add_offdiag(const float2 *a, const float2 *b, int N, float2 *out, cu
 namespace rbx {
 
 // slot = (|R|^2, sum dc^2, max |dc|, sum dm^2, uncovered, clamped, bad rays, CAS bound,
-//         non-positive m, bad model, tensor-core timeout, 0)
-__global__ void k_snapshot(const double *r2, const double *upd3, const unsigned long long *counters,
-                           const unsigned *tc_err, unsigned long long n_entries, double *slot)
+//         non-positive m, bad model, tensor-core timeout, 0); the timeout is then reported and cleared
+__global__ void k_snapshot(const double *r2, const double *upd3, const unsigned long long *counters, unsigned *err,
+                           unsigned long long n_entries, double *slot)
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     slot[0] = *r2;
@@ -281,14 +284,15 @@ __global__ void k_snapshot(const double *r2, const double *upd3, const unsigned 
     slot[3] = upd3[2];
     slot[4] = (double)(n_entries - counters[0]);   // counters[0] holds the covered entries
     for (int k = 1; k < 6; k++) slot[4 + k] = (double)counters[k];
-    slot[10] = tc_err ? (double)*tc_err : 0.0;
+    slot[10] = (double)*err;
+    *err = 0u;
     slot[11] = 0.0;
 }
 
-void launch_snapshot(const double *r2, const double *upd3, const unsigned long long *counters, const unsigned *tc_err,
+void launch_snapshot(const double *r2, const double *upd3, const unsigned long long *counters, unsigned *err,
                      unsigned long long n_entries, double *slot, cudaStream_t s)
 {
-    k_snapshot<<<1, 32, 0, s>>>(r2, upd3, counters, tc_err, n_entries, slot);
+    k_snapshot<<<1, 32, 0, s>>>(r2, upd3, counters, err, n_entries, slot);
 }
 
 // dst = (first ? 0 : dst) + src: the residual norm summed over a frequency set

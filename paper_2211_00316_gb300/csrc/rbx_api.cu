@@ -44,6 +44,7 @@ struct rbx_job {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_in_free = nullptr, ev_in_ready = nullptr;
     long long launches = 0;
+    bool unread = false;       // a call without a status of its own may have set w.err (rbx_synchronize reads it)
     int load_dev = -1;         // device whose g_load counts this job's trace (set with the geometry)
     bool waits = false;        // inside a call that traces and waits for the update (Waiting)
 };
@@ -148,7 +149,7 @@ static cudaError_t dalloc(T *&p, size_t n, cudaStream_t s)
 static void free_ws(Workspace &w, cudaStream_t s)
 {
     void *ps[] = {w.hist, w.node2x, w.idx, w.rows, w.c, w.ns, w.tmp, w.fields, w.ns64, w.tmp64, w.tab, w.exits, w.v, w.gdir, w.D, w.R, w.Rs, w.part, w.gpart, w.data, w.red, w.counters, w.alpha0, w.as64,
-                  w.dmacc, w.linked, w.beta};
+                  w.dmacc, w.linked, w.beta, w.err};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, s);
     tc_free(w.tc, s);
@@ -236,7 +237,26 @@ const char *rbx_last_error(const rbx_job *j) { return j ? j->err.c_str() : "null
 rbx_status rbx_synchronize(rbx_job *j)
 {
     if (!j) return RBX_EINVAL;
+    if (!j->unread) {
+        CUDA_TRY(j, cudaStreamSynchronize(j->stream));
+        return RBX_OK;
+    }
+    unsigned e = 0;
+    CUDA_TRY(j, cudaMemcpyAsync(&e, j->w.err, sizeof e, cudaMemcpyDeviceToHost, j->stream));
     CUDA_TRY(j, cudaStreamSynchronize(j->stream));
+    j->unread = false;
+    if (e == 0) return RBX_OK;
+    CUDA_TRY(j, cudaMemsetAsync(j->w.err, 0, sizeof e, j->stream));
+    return fail(j, RBX_ETIMEOUT, "a tensor-core kernel's bounded wait gave up");
+}
+
+rbx_status rbx_selftest_job_timeout(rbx_job *j)
+{
+    if (!j) return RBX_EINVAL;
+    NEED(j, j->has_geom, RBX_ESTATE, "rbx_selftest_job_timeout before rbx_set_geometry");
+    launch_wait_selftest(j->w.err, j->stream);
+    LAUNCHED(j, 1);
+    j->unread = true;
     return RBX_OK;
 }
 
@@ -286,7 +306,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     drop_load(j);
     free_ws(j->w, j->stream);
     keep_pool_memory();
-    j->has_geom = j->has_tables = j->ns_valid = j->lossy = j->raw = false;
+    j->has_geom = j->has_tables = j->ns_valid = j->lossy = j->raw = j->unread = false;
     j->link_iters = 0;
     Workspace &w = j->w;
     w.N = g.n_xducers;
@@ -321,9 +341,11 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.fields, nxy * kFieldStride);
     ALLOC(w.tab, NX);
     ALLOC(w.exits, N * (N - 1));
+    ALLOC(w.err, 1);
+    CUDA_TRY(j, cudaMemsetAsync(w.err, 0, sizeof(unsigned), j->stream));
     // FP32 jobs: the operands of both contractions; the others: those of the plain adjoint
-    if (!f32_setup(w.f32, w.N, X, 3, g.precision == RBX_FP32, j->stream) ||
-        (g.precision == RBX_BF16X3 && !f32_setup(w.split, w.N, X, 2, true, j->stream))) {
+    if (!f32_setup(w.f32, w.N, X, 3, g.precision == RBX_FP32, w.err, j->stream) ||
+        (g.precision == RBX_BF16X3 && !f32_setup(w.split, w.N, X, 2, true, w.err, j->stream))) {
         cudaGetLastError();
         free_ws(w, j->stream);
         return fail(j, RBX_ENOMEM, "operand set-up failed (allocation or TMA descriptor)");
@@ -335,7 +357,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     ALLOC(w.Rs, N * N);
     ALLOC(w.data, N * N);
     if (g.precision == RBX_BF16) {
-        if (!tc_setup(w.tc, w.N, X, j->stream)) {
+        if (!tc_setup(w.tc, w.N, X, w.err, j->stream)) {
             cudaGetLastError();
             free_ws(w, j->stream);
             return fail(j, RBX_ENOMEM, "tensor-core operand set-up failed (allocation or TMA descriptor)");
@@ -615,7 +637,7 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
         }
         if (timed && (st = record(j, EV_SYNTH_F))) return st;
         int splits = launch_forward_tc_fused(w.tc, w.tab, w.v, f, j->g.c0, w.part, j->stream);
-        launch_forward_reduce(w.part, w.N, splits, w.D, j->stream);
+        launch_forward_reduce(w.part, w.N, splits, w.err, w.D, j->stream);
         LAUNCHED(j, 2);
     } else if (j->g.precision == RBX_BF16) {
         if (both)
@@ -625,14 +647,14 @@ static rbx_status forward_core(rbx_job *j, double f, bool timed, bool both = fal
         LAUNCHED(j, 1);
         if (timed && (st = record(j, EV_SYNTH_F))) return st;
         int splits = launch_forward_tc(w.tc, w.part, j->stream);
-        launch_forward_reduce(w.part, w.N, splits, w.D, j->stream);
+        launch_forward_reduce(w.part, w.N, splits, w.err, w.D, j->stream);
         LAUNCHED(j, 2);
     } else {
         launch_synth_fwd(parts_of(j), w.tab, w.v, f, j->g.c0, j->stream);
         LAUNCHED(j, 1);
         if (timed && (st = record(j, EV_SYNTH_F))) return st;
         launch_forward_f32(parts_of(j), w.fwd_splits, w.part, j->stream);
-        launch_forward_reduce(w.part, w.N, w.fwd_splits, w.D, j->stream);
+        launch_forward_reduce(w.part, w.N, w.fwd_splits, w.err, w.D, j->stream);
         LAUNCHED(j, 2);
     }
     if (timed && (st = record(j, EV_GEMM_F))) return st;
@@ -647,6 +669,7 @@ rbx_status rbx_forward(rbx_job *j, double f, const float *dm_dev, void *D_dev)
     Workspace &w = j->w;
     launch_born_weights_dm(dm_dev, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j), w.v, j->stream);
     LAUNCHED(j, 1);
+    j->unread = true;
     rbx_status st = forward_core(j, f, false);
     if (st) return st;
     CUDA_TRY(j, cudaMemcpyAsync(D_dev, w.D, sizeof(float2) * (size_t)w.N * w.N, cudaMemcpyDeviceToDevice, j->stream));
@@ -668,6 +691,7 @@ rbx_status rbx_predict(rbx_job *j, double f, void *g_dev)
     } else {
         launch_born_weights_rough(w.c, w.ns64, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j), w.v, j->stream);
         LAUNCHED(j, 1);
+        j->unread = true;
         if ((st = forward_core(j, f, false))) return st;
     }
     launch_add_offdiag(w.gdir, w.D, w.N, static_cast<float2 *>(g_dev), j->stream);
@@ -682,24 +706,25 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
     NEED(j, !bad_freq(f), RBX_EINVAL, "frequency must be finite and > 0");
     Workspace &w = j->w;
     const float2 *R = static_cast<const float2 *>(R_dev);
+    j->unread = true;
     if (preconditioned && j->g.precision == RBX_BF16) {
         launch_symmetrize(R, w.N, w.Rs, j->stream);
         launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);
         launch_backproject_tc(w.tc, w.Rs, j->g.weight_mode, w.gpart, j->stream);
-        launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
+        launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, w.err, static_cast<float2 *>(out_dev), j->stream);
         LAUNCHED(j, 5);
     } else if (preconditioned) {
         launch_synth_bp(parts_of(j), w.tab, f, j->g.c0, j->stream);
         LAUNCHED(j, launch_backproject_f32(parts_of(j), w.tab, R, false, w.gpart, j->stream));
-        launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, static_cast<float2 *>(out_dev), j->stream);
+        launch_combine_adjoint(w.gpart, w.X, 0, j->g.weight_mode, 2.0, w.err, static_cast<float2 *>(out_dev), j->stream);
     } else {
         double om = 2 * 3.14159265358979323846 * f;
         LAUNCHED(j, launch_adjoint_f32(w.f32, w.tab, R, f, j->g.c0, w.gpart, j->stream));
         if (j->lossy)
-            launch_combine_adjoint_lossy(w.gpart, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j),
+            launch_combine_adjoint_lossy(w.gpart, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j), w.err,
                                          static_cast<float2 *>(out_dev), j->stream);
         else
-            launch_combine_adjoint(w.gpart, w.X, 1, j->g.weight_mode, om * om * j->g.dx * j->g.dx,
+            launch_combine_adjoint(w.gpart, w.X, 1, j->g.weight_mode, om * om * j->g.dx * j->g.dx, w.err,
                                    static_cast<float2 *>(out_dev), j->stream);
     }
     LAUNCHED(j, 1);
@@ -746,15 +771,9 @@ static rbx_status enqueue_freq(rbx_job *j, double f, double df, const float2 *da
     if ((st = record(j, EV_GEMM_B))) return st;
     const int roff = residual_blocks(w.N) + 8;
     launch_update(w.gpart, w.node2x, w.nx, w.ny, w.X, j->g.weight_mode, f, df, j->g.tau, j->g.c0, w.c, w.red + roff,
-                  w.counters, lossy_of(j), w.dmacc, mode, j->stream);
+                  w.counters, lossy_of(j), w.dmacc, mode, w.err, j->stream);
     LAUNCHED(j, 2);
     return RBX_OK;
-}
-
-// Where the kernels of an update's contractions record a bounded wait that gave up.
-static const unsigned *contraction_err(const rbx_job *j)
-{
-    return j->g.precision == RBX_BF16 ? j->w.tc.err : (j->g.precision == RBX_FP32 ? j->w.f32 : j->w.split).err;
 }
 
 static rbx_status enqueue_update(rbx_job *j, double f, double df, const float2 *data, bool traced, int slot)
@@ -768,7 +787,7 @@ static rbx_status enqueue_update(rbx_job *j, double f, double df, const float2 *
     if ((st = enqueue_freq(j, f, df, data, 0))) return st;
     const int roff = residual_blocks(w.N) + 8;
     launch_snapshot(w.red + residual_blocks(w.N), w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters,
-                    contraction_err(j), (unsigned long long)w.N * w.X, w.hist + (size_t)slot * kHistStride, j->stream);
+                    w.err, (unsigned long long)w.N * w.X, w.hist + (size_t)slot * kHistStride, j->stream);
     LAUNCHED(j, 1);
     if ((st = record(j, EV_UPDATE))) return st;
     j->ns_valid = false;   // the model changed
@@ -928,7 +947,7 @@ rbx_status rbx_update_set(rbx_job *j, const double *freqs, int nf, double df, co
         launch_acc_scalar(w.red + nb, w.red + nb + 4, k == 0, j->stream);
         LAUNCHED(j, 1);
     }
-    launch_snapshot(w.red + nb + 4, w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters, contraction_err(j),
+    launch_snapshot(w.red + nb + 4, w.red + roff + 3 * update_blocks(w.nx, w.ny), w.counters, w.err,
                     (unsigned long long)w.N * w.X, w.hist, j->stream);
     LAUNCHED(j, 1);
     if ((st = record(j, EV_UPDATE))) return st;

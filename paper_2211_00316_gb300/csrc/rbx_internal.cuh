@@ -72,7 +72,7 @@ struct TcPlanes {
     void *bplanes = nullptr;   // [6][Xp][Npad] bf16: u, conj(kappa) u, kappa u (re, im)
     void *rsplanes = nullptr;  // [2][Npad][Npad] bf16: R_s re, im
     float2 *bpart = nullptr;   // [Npad/128][Xp] partial back-projection
-    unsigned *err = nullptr;   // bounded-wait timeouts of the tensor-core kernels
+    unsigned *err = nullptr;   // the job's timeout word (Workspace::err)
     CUtensorMap fmaps[4], bmaps[6];
     bool ready = false;
 };
@@ -86,7 +86,7 @@ struct F32Planes {
     void *planes = nullptr;    // [4 parts, or 2 parts (plain adjoint alone)][N][xld] bf16
     void *rs = nullptr;        // [2 parts][N][rld] bf16
     float2 *bpart = nullptr;   // [stacks][emitter tiles][X]; nullptr with one emitter tile
-    unsigned *err = nullptr;   // bounded-wait timeouts
+    unsigned *err = nullptr;   // the job's timeout word (Workspace::err)
     CUtensorMap fmap, amap, rmap;   // K-major and M-major boxes of planes, K-major boxes of rs
 };
 
@@ -110,6 +110,9 @@ struct Workspace {
     double *red = nullptr;           // reduction scratch
     double *hist = nullptr;          // [kHistSlots][kHistStride] per-update scalars
     unsigned long long *counters = nullptr;   // [0] covered entries [1] clamped [2] bad rays [3] CAS bound [4] m <= 0 [5] bad model [6] mask count [7] uniform radius (float bits)
+    // Bits of the bounded waits of the contractions that gave up. Set, it makes what they feed not a
+    // number until it is reported, by an update's status or rbx_synchronize, and cleared.
+    unsigned *err = nullptr;
     int fwd_splits = 1;
     TcPlanes tc;
     F32Planes f32;              // FP32 jobs; the plain adjoint of the others
@@ -184,11 +187,11 @@ void launch_born_weights_rough(const float *c, const double *ns64, const int *id
                                const Lossy &ab, float2 *v, cudaStream_t s);
 void launch_born_weights_dm(const float *dm, const float *c, const int *idx, int X, double f, double dA,
                             const Lossy &ab, float2 *v, cudaStream_t s);
-void launch_forward_reduce(const float2 *part, int N, int splits, float2 *D, cudaStream_t s);
+void launch_forward_reduce(const float2 *part, int N, int splits, const unsigned *err, float2 *D, cudaStream_t s);
 
 // k_gemm_f32.cu (FP32 accuracy on the tensor cores)
 int forward_splits(int N, int X);
-bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, cudaStream_t s);
+bool f32_setup(F32Planes &p, int N, int X, int parts, bool full, unsigned *err, cudaStream_t s);
 void f32_free(F32Planes &p, cudaStream_t s);
 void launch_synth_fwd(F32Planes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s);
 void launch_synth_bp(F32Planes &p, const TabEntry *tab, double f, double c0, cudaStream_t s);
@@ -203,7 +206,7 @@ int launch_adjoint_f32(F32Planes &p, const TabEntry *tab, const float2 *R, doubl
 // k_gemm_tc.cu (BF16 tensor cores)
 bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
                   const cuuint32_t *box, const cuuint32_t *estr, CUtensorMapSwizzle swizzle);
-bool tc_setup(TcPlanes &p, int N, int X, cudaStream_t s);
+bool tc_setup(TcPlanes &p, int N, int X, unsigned *err, cudaStream_t s);
 // Choose the forward K split by timing the candidates on this job's planes (once per shape
 // and process; later jobs of the shape reuse the choice). part holds fwd_max_splits partials.
 bool tc_autotune(TcPlanes &p, float2 *part, TabEntry *tab, float2 *v, cudaStream_t s);
@@ -215,7 +218,7 @@ int launch_forward_tc(TcPlanes &p, float2 *part, cudaStream_t s);
 int launch_forward_tc_fused(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, float2 *part,
                             cudaStream_t s);
 void launch_synth_bp_tc(TcPlanes &p, const TabEntry *tab, double f, double c0, cudaStream_t s);
-// a bounded wait on a barrier nothing signals (flag = 1 when it gave up)
+// a bounded wait on a barrier nothing signals (flag |= 1 when it gave up)
 void launch_wait_selftest(unsigned *flag, cudaStream_t s);
 // both operand sets of an update in one pass over the tables (forward planes with weights v)
 void launch_synth_both_tc(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s);
@@ -225,16 +228,16 @@ void launch_backproject_tc(TcPlanes &p, const float2 *Rs, int weight_mode, float
 void launch_residual(const float2 *gdir, const float2 *D, const float2 *data, int N, float2 *R, float2 *Rs,
                      double *red, cudaStream_t s);
 void launch_symmetrize(const float2 *R, int N, float2 *Rs, cudaStream_t s);
-void launch_combine_adjoint(const float2 *gpart, int X, int mode, int weight_mode, double scale, float2 *out,
-                            cudaStream_t s);
+void launch_combine_adjoint(const float2 *gpart, int X, int mode, int weight_mode, double scale, const unsigned *err,
+                            float2 *out, cudaStream_t s);
 // plain adjoint of a lossy job: out[x] = dA conj(Upsilon_m[x]) gpart[x]
 void launch_combine_adjoint_lossy(const float2 *gpart, const float *c, const int *idx, int X, double f, double dA,
-                                  const Lossy &ab, float2 *out, cudaStream_t s);
+                                  const Lossy &ab, const unsigned *err, float2 *out, cudaStream_t s);
 void launch_acc_scalar(const double *src, double *dst, bool first, cudaStream_t s);
 void launch_update(const float2 *gpart, const int *node2x, int nx, int ny, int X, int weight_mode, double f,
                    double df, double tau, double c0, float *c, double *red, unsigned long long *counters,
-                   const Lossy &ab, double *acc, int mode, cudaStream_t s);
-void launch_snapshot(const double *r2, const double *upd3, const unsigned long long *counters, const unsigned *tc_err,
+                   const Lossy &ab, double *acc, int mode, const unsigned *err, cudaStream_t s);
+void launch_snapshot(const double *r2, const double *upd3, const unsigned long long *counters, unsigned *err,
                      unsigned long long n_entries, double *slot, cudaStream_t s);
 int residual_blocks(int N);
 int update_blocks(int nx, int ny);

@@ -89,6 +89,7 @@ _SIGS = {
     "rbx_get_tuning_times": [_P, C.POINTER(C.c_float), C.POINTER(C.c_int)],
     "rbx_set_slot_timing": [_J, C.c_int],
     "rbx_selftest_bounded_wait": [C.POINTER(C.c_int)],
+    "rbx_selftest_job_timeout": [_J],
     "rbx_pool_usage": [C.POINTER(C.c_size_t), C.POINTER(C.c_size_t), C.c_int],
     "rbx_server_times": [_P, C.c_longlong, C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)],
     "rbx_server_info": [_P, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_size_t)],
@@ -334,7 +335,12 @@ class Job:
         return dict(fwd_splits=sp.value, candidates_timed=nc.value, fused_forward=bool(fu.value),
                     ms_synth_both=ms[0], ms_forward_gemm=ms[1], ms_synth_bp=ms[2], ms_forward_fused=ms[3])
 
+    def selftest_timeout(self):
+        """Let a bounded wait run out on the job's stream (rbx_selftest_job_timeout)."""
+        self._check(self.L.rbx_selftest_job_timeout(self.h))
+
     def sync(self):
+        """Wait for the job's work; raises RBX_ETIMEOUT once if a bounded wait of it gave up."""
         self._check(self.L.rbx_synchronize(self.h))
 
 
