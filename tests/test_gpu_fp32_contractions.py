@@ -105,3 +105,60 @@ def test_more_than_65535_node_tiles():
         assert bool(torch.isfinite(torch.view_as_real(out)).all()) and float(out[0].abs()) > 0
         assert bool((out == out[0]).all())
     job.close()
+
+
+# (12, 2), (10, 4), (25, 2), (3, 4), (2, 4), (1, 4): partial sums and CTAs of a cluster per tile pair, by
+# noalloc_shape on 152 SMs; all with a ragged last tile, with node counts that are no multiple of 4 or
+# of a chunk, and all but the fifth with CTAs that get fewer chunks or none
+@pytest.mark.parametrize("n,x", [(257, 2337), (250, 4001), (150, 4827), (500, 1203), (600, 1251), (1000, 1299)])
+def test_noalloc_clusters(n, x):
+    rng = np.random.default_rng(n)
+    T = rng.uniform(1e-6, 1e-4, (n, x)).astype(np.float32)
+    a = rng.uniform(2.0, 30.0, (n, x)).astype(np.float32)
+    a[rng.random(a.shape) < 0.02] = 0.0
+    K = rng.integers(0, 3, a.shape).astype(np.uint8)
+    v = rng.standard_normal(x).astype(np.float32)
+    G = (8 * math.pi * 2 * math.pi * F / C0) ** -0.5 * a.astype(np.float64) * np.exp(
+        2j * np.pi * (F * T.astype(np.float64) - K / 4 + 0.125))
+    dev = [torch.tensor(t, device="cuda") for t in (T, a, K, v)]
+    D = torch.empty((n, n), dtype=torch.complex64, device="cuda")
+    err = ctypes.create_string_buffer(256)
+    assert rbx.load().rbx_forward_noalloc(*[t.data_ptr() for t in dev], n, x, F, C0, D.data_ptr(),
+                                          torch.cuda.current_stream().cuda_stream or None, err, 256) == 0
+    D = D.cpu().numpy()
+    assert rel(D, (G * v.astype(np.float64)) @ G.T) <= 1e-6
+    assert np.array_equal(D, D.T)
+
+
+@pytest.mark.parametrize("n", [3, 16, 17, 31, 32, 33, 64, 65, 95, 97, 127, 128, 129, 144, 257])
+@pytest.mark.parametrize("nx,ny", [(24, 24), (41, 37)])
+def test_split_against_complex128(n, nx, ny):
+    """Split BF16 at the same edges, and with fewer chunks than stages. Two parts leave 2^-18 of an operand, and lo lo
+    2^-18 of a product: 3 x 2^-18 = 1.2e-5 of every product; 2e-5 leaves the FP32 roundings room, the
+    preconditioned operands' dgamma on top."""
+    g = P.Geometry(nx=nx, ny=ny, dx=1e-3, n_xducers=n, ring_radius=(min(nx, ny) - 1) * 0.5e-3 - 1.5e-3)
+    T, a, gam, K = tables(g, n)
+    rng = np.random.default_rng(8)
+    cov = a > 0
+    w = 2 * math.pi * F
+    G = np.where(cov, (8 * math.pi * w / C0) ** -0.5 * a.astype(np.float64) *
+                 np.exp(2j * np.pi * (F * T.astype(np.float64) - K / 4 + 0.125)), 0)
+    gd = gam.astype(np.float64)
+    d = np.roll(gd, -1, 0) - np.roll(gd, 1, 0)
+    d = 0.5 * np.abs(np.mod(d + np.pi, 2 * np.pi) - np.pi)
+    d[~(np.roll(cov, -1, 0) & np.roll(cov, 1, 0))] = 0
+    U = np.where(cov, d / np.where(cov, G, 1), 0)
+    kap = np.exp(1j * gd)
+    dm = (1e-9 * rng.standard_normal((ny, nx))).astype(np.float32)
+    v = w * w * g.dx ** 2 * dm[g.mask()].astype(np.float64)
+    R = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    Rs = 0.5 * (R + R.T).astype(np.complex128)
+    job = rbx.Job()
+    job.set_geometry(g, precision=rbx.RBX_BF16X3)
+    job.set_tables(*[torch.tensor(t, device="cuda") for t in (T, a, gam, K)], torch.zeros((n, n - 1, 4), device="cuda"))
+    Rd = torch.tensor(R, device="cuda")
+    assert rel(job.forward(F, torch.tensor(dm, device="cuda")).cpu().numpy(), (G * v) @ G.T) <= 2e-5
+    assert rel(job.adjoint(F, Rd, True).cpu().numpy(),
+               2 * ((U * (Rs @ U)).sum(0) - (kap * U * (Rs @ (kap.conj() * U))).sum(0))) <= 2e-5 + n * 2.0 ** -24
+    assert rel(job.adjoint(F, Rd, False).cpu().numpy(), w * w * g.dx ** 2 * (G.conj() * (Rs @ G.conj())).sum(0)) <= 1e-6
+    job.close()
