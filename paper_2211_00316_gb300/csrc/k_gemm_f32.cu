@@ -12,7 +12,9 @@
 //  i.e. a complex GEMM with the two stacks as rows and a fused row-dot epilogue.
 //
 // An FP32 operand is held as three BF16 parts, v = hi + mid + lo, which together carry its 24
-// bits exactly; the six products hi hi, hi mid, mid hi, mid mid, hi lo, lo hi leave out terms of
+// bits exactly while its size lies between 2^-110 (1e-33; below, the last part would be less than BF16's
+// smallest number, and the lowest bits go) and BF16's largest, 3.39e38 (a larger one, an infinity and not a number
+// all give not a number). The six products hi hi, hi mid, mid hi, mid mid, hi lo, lo hi leave out terms of
 // 2^-26 of the product. tcgen05 adds to its FP32 accumulators in tensor memory without rounding
 // to nearest, so a long sum there drifts; here a sum in tensor memory covers 32 terms of K (one
 // pipeline stage, the five small products before hi hi so that only four additions meet the
@@ -26,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace rbx {
 using namespace tc;
@@ -96,9 +99,7 @@ struct GemmArgs {
     int N, ntile, nk, kper;         // tiles of transducers, K chunks; forward: chunks per split
     float2 *part;                   // forward: [split][N][N] partial D
     const TabEntry *tab;            // back-projection: directions of stack 1
-    const __nv_bfloat16 *planes;    // back-projection: parts of the weights, [plane][N][xld]
-    size_t pstride;
-    int xld, X;                     // back-projection: row length of the planes, nodes
+    int X;                          // back-projection: nodes
     float2 *bpart;                  // back-projection: [stack][e tile][X] partial row-dots
     unsigned *err;
 };
@@ -118,9 +119,10 @@ struct GemmArgs {
 // Against FP32 multiply-adds on the CUDA cores (64 x 64 tiles, 0.5 of their peak), ncu: 256
 // transducers, 48,120 nodes: forward 437 -> 89 us, back-projection 1297 -> 321 us (its row-dot as it
 // is now takes another 75 us off the update); 768 transducers, 19,760 nodes: plain adjoint 2915 -> 384
-// us, 364 now. Error against 64 bits no larger at any
-// size from 48 transducers on (N = 1024, 20,000 nodes: forward 6.0e-7 -> 2.2e-7, plain adjoint
-// 6.1e-7 -> 1.7e-7).
+// us, 364 now. Error against 64 bits smaller at
+// every size from 5 transducers on (N = 1024, 20,000 nodes: forward 6.0e-7 -> 2.2e-7, plain adjoint
+// 6.1e-7 -> 1.7e-7; N = 8, mean of six tables: forward 2.7e-7 -> 1.2e-7, plain 1.42e-7 -> 1.36e-7,
+// preconditioned 1.9e-7 -> 1.7e-7); with 3 transducers the plain adjoint's is 1.30e-7 -> 1.37e-7.
 template <int NP, bool BP, bool CONJ>
 __global__ __launch_bounds__(THREADS, 1) void k_cgemm_f32(const __grid_constant__ GemmArgs g)
 {
@@ -537,12 +539,14 @@ void synth(const F32Planes &p, const TabEntry *tab, const float2 *v, double f, d
     const int walk = (size_t)bx * ((p.N + 7) / 8) >= 152 * 16 ? 8 : 2;
     const dim3 grd(bx, (unsigned)((p.N + walk - 1) / walk));
     __nv_bfloat16 *planes = static_cast<__nv_bfloat16 *>(p.planes);
-    if (p.parts == 3)
-        k_synth_parts<KIND, 3><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.xld, p.pstride, fhi, flo,
-                                                   green_const(f, c0), planes, walk);
-    else
-        k_synth_parts<KIND, 2><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.xld, p.pstride, fhi, flo,
-                                                   green_const(f, c0), planes, walk);
+    auto go = [&](auto parts) {
+        k_synth_parts<KIND, decltype(parts)::value><<<grd, 128, 0, s>>>(tab, v, p.N, p.X, p.xld, p.pstride, fhi, flo,
+                                                                        green_const(f, c0), planes, walk);
+    };
+    if constexpr (KIND != 0) {   // the plain adjoint always takes three parts
+        if (p.parts == 2) return go(std::integral_constant<int, 2>{});
+    }
+    go(std::integral_constant<int, 3>{});
 }
 
 }  // namespace
@@ -641,9 +645,6 @@ static GemmArgs bp_args(F32Planes &p, const TabEntry *tab, float2 *gpart)
     g.ntile = (p.N + BN - 1) / BN;
     g.nk = (p.N + BK - 1) / BK;
     g.tab = tab;
-    g.planes = static_cast<const __nv_bfloat16 *>(p.planes);
-    g.pstride = p.pstride;
-    g.xld = p.xld;
     g.X = p.X;
     g.bpart = p.bpart ? p.bpart : gpart;
     g.err = p.err;
