@@ -71,7 +71,9 @@ __device__ __forceinline__ int clampi(int i, int lo, int hi) { return i < lo ? l
 
 // a / b correctly rounded from r, the correctly rounded 1 / b: the quotient's first approximation
 // and one correction with the exact remainder (P. W. Markstein, Computation of elementary
-// functions on the IBM RISC System/6000 processor, IBM J. Res. Dev. 34, 1990). FP64 division is
+// functions on the IBM RISC System/6000 processor, IBM J. Res. Dev. 34, 1990). The theorem there asks for a
+// first approximation within one ulp, and a r may be 1.5 off: correct rounding is what was found (none of
+// 2e8 random quotients by the divisors used here differs from a / b). FP64 division is
 // the bulk of these kernels otherwise (k_fields, 288 x 288: 25.6 -> 11.6 us).
 __device__ __forceinline__ double quotient(double a, double b, double r)
 {

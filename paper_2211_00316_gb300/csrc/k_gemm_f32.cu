@@ -114,7 +114,9 @@ struct GemmArgs {
 //
 // Bound: shared-memory bandwidth of the tensor cores. A 128 x 128 x 16 MMA reads 8 KB in the 64
 // clocks it takes at the peak rate (128 B per clock, all an SM has), the tile loads write 31 B
-// per clock besides, so 0.7-0.8 of the BF16 peak over the six products is what the form allows.
+// per clock besides, so 0.7-0.8 of the BF16 peak over the six products is what the form allows (tensor
+// pipes busy, ncu: plain adjoint of 768 transducers 65 % of the launch; of 256, forward 53 %, back-projection 49 %:
+// there the start of each CTA, its last drain and the row-dot weigh more).
 // K chunks of 32 because a 64-term stage of both operands' parts (192 KB) leaves no second one.
 // Against FP32 multiply-adds on the CUDA cores (64 x 64 tiles, 0.5 of their peak), ncu: 256
 // transducers, 48,120 nodes: forward 437 -> 89 us, back-projection 1297 -> 321 us (its row-dot as it

@@ -696,8 +696,10 @@ __global__ __launch_bounds__(32 * kFansPerBlock, WARPS / kFansPerBlock) void k_t
 // the candidate nodes of its tube (most of a step's time there). The rays' samples go to their
 // neighbours through shared memory, one barrier per step. Same arithmetic, ray groups and
 // table as k_trace_raster.
-// Against one lane per ray: 64 transducers (96 x 96), eight lanes: 0.485 -> 0.333 ms; 128 (160 x 160),
-// four: 0.75 -> 0.66; 192 (200 x 200), two: 0.95 -> 0.90.
+// Against one lane per ray (rbx_trace_rays): 64 transducers (96 x 96), eight lanes: 0.453 -> 0.351 ms; 128
+// (160 x 160), four: 0.805 -> 0.755; 192 (217 x 217), two: 1.139 -> 1.112 (200 x 200: 0.99, 1.00). Bound: a ray's
+// chain of steps and the barrier between them (64 transducers: issue port busy 27 % of the cycles of
+// the SMs at work, a third of the stalled time at the barrier).
 template <int LPR>
 struct WideShared {
     uint4 v[LPR][64];
@@ -1050,7 +1052,7 @@ void launch_uniform_radius(const float *fields, const RayParams &p, unsigned lon
 // lane per ray; own: this trace's) stay within 3,040 warps, or 1,520 beside other jobs. Every lane of a ray
 // integrates it, which costs nothing only while the GPU has issue slots to spare; beside other jobs
 // their contractions take some of those. The GPU holds 2,432 warps of k_trace_wide (16 per SM), 3,040
-// of k_trace_raster: that the line lies there is what was measured. ms of one trace alone with 1 / 2 / 4 / 8
+// of k_trace_raster: that the line lies there is what was measured. ms of one rbx_trace_rays alone with 1 / 2 / 4 / 8
 // lanes: 64 transducers on 102 x 102 0.507 / 0.484 / 0.406 / 0.378, 128 on 160 x 160 0.806 / 0.807 / 0.755 /
 // 1.069, 152 on 181 x 181 0.915 / 0.885 / 0.830 / 1.407, 217 on 240 x 240 1.356 / 1.333 / 1.931 / 3.349. Together:
 // four of 64 on 96 x 96 0.497 / 0.494 / 0.487 / 0.648, eight 0.561 / 0.604 / 0.735 / 1.229, 24 of 128 on
