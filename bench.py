@@ -93,8 +93,8 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none
     #     -k regex:k_trace_raster -s 3 -c 1 --csv   (k_synth_tc: -k regex:k_synth_tc -s 6 -c 1)
     #     python bench.py --steps 2 --warmup 1 --no-cpu-baseline --no-e2e --no-forms   (1 pass)
-    ("precision_ring1024", "trace"): {"bytes": 2.803052800e9 + 2.557826048e9, "src": "c223f0c990fb"},
-    ("precision_ring1024", "synth"): {"bytes": 2.494422016e9 + 3.067075584e9, "src": "30658383676f"},
+    ("precision_ring1024", "trace"): {"bytes": 2.802625536e9 + 2.558109184e9, "src": "b26b36ffc609"},
+    ("precision_ring1024", "synth"): {"bytes": 2.495077888e9 + 3.067216640e9, "src": "78a90e9170f4"},
 }
 
 
@@ -116,8 +116,8 @@ def algorithmic(kernel: str, N: int, X: int, precision: str):
         return (16.0 + 20.0 * planes) * NX, "byte", "hbm"
     if kernel == "synth_bp":
         # tables in; BF16: 6 planes out; split BF16: the two parts of u and conj(kappa) u; FP32: the
-        # 20 bytes counted are those of u, conj(kappa) u and the angular density held in FP32 (the
-        # three BF16 parts written are 24)
+        # same two as FP32 (16) and four bytes more (a lower bound: the three BF16 parts of each, 24
+        # bytes, are what is written)
         out = {"fp32": 4.0 + 16.0, "bf16": 12.0, "bf16x3": 16.0}[precision]
         return (16.0 + out) * NX, "byte", "hbm"
     if kernel == "tables":
