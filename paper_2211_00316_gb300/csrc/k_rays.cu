@@ -1049,21 +1049,28 @@ void launch_uniform_radius(const float *fields, const RayParams &p, unsigned lon
 }
 
 // Lanes per ray: the most (up to 8) with which the traces running together (load: their warps with one
-// lane per ray; own: this trace's) stay within 3,040 warps, or 1,520 beside other jobs. Every lane of a ray
-// integrates it, which costs nothing only while the GPU has issue slots to spare; beside other jobs
-// their contractions take some of those. The GPU holds 2,432 warps of k_trace_wide (16 per SM), 3,040
-// of k_trace_raster: that the line lies there is what was measured. ms of one rbx_trace_rays alone with 1 / 2 / 4 / 8
-// lanes: 64 transducers on 102 x 102 0.507 / 0.484 / 0.406 / 0.378, 128 on 160 x 160 0.806 / 0.807 / 0.755 /
-// 1.069, 152 on 181 x 181 0.915 / 0.885 / 0.830 / 1.407, 217 on 240 x 240 1.356 / 1.333 / 1.931 / 3.349. Together:
-// four of 64 on 96 x 96 0.497 / 0.494 / 0.487 / 0.648, eight 0.561 / 0.604 / 0.735 / 1.229, 24 of 128 on
-// 160 x 160 4.0 with one lane and 11.2 with the four of a ring alone; a batch of three updates each, eight of
-// 64: 1.98 with one lane, 2.53 with two.
+// lane per ray, this one's included) stay within a number of warps. Every lane of a ray integrates it, which
+// costs nothing only while the GPU has issue slots to spare, and gives nothing where a ray's tube holds
+// no node to share out. So the number is 3,040 for a trace alone, 1,216 (8 per SM) where the tubes are thin
+// (2 R ds / (dx dx N), to a factor the nodes that a quad of the fan holds on average, below 1/2), and half of
+// that beside other jobs, whose contractions take some of the slots. The GPU holds 2,432 warps of k_trace_wide (16 per SM) and
+// 3,040 of k_trace_raster; that the line lies there is what was measured (rbx_trace_rays alone, ms, lanes 1 / 2 /
+// 4 / 8, ds = dx / 2):
+//   thick, N on nodes: 64 on 96 0.464 / 0.442 / 0.383 / 0.358, 128 on 160 0.865 / 0.842 / 0.789 / 1.088, 152 on 160
+//     0.810 / 0.787 / 0.734 / 1.250, 215 on 224 1.299 / 1.290 / 1.829 / 3.094
+//   thin: 64 on 48 0.173 / 0.171 / 0.165 / 0.169, 96 on 64 0.225 / 0.229 / 0.239 / 0.251, 128 on 80 0.284 / 0.306 /
+//     0.335 / 0.502, 215 on 80 0.263 / 0.370 / 0.585 / 1.048 (the two lanes of 3,040 warps took longer than the
+//     0.327 of the kernel before the present one)
+//   together: four of 64 on 96 0.497 / 0.494 / 0.487 / 0.648, eight 0.561 / 0.604 / 0.735 / 1.229; 24 of 128 on 160 4.0
+//     with one lane, 11.2 with the four of a ring alone; a batch of three updates each, eight of 64: 1.98 with one
+//     lane, 2.53 with two
 // The block keeps its queues and `rows_bytes` of mask rows in the 48 KB of shared memory that a launch
 // has without asking for more (eight lanes to 2,173 grid rows, four to 2,558). One lane, and
 // k_trace_raster, from about 215 transducers on.
-static int lanes_per_ray(size_t load, size_t own, size_t rows_bytes)
+static int lanes_per_ray(const RayParams &p, size_t load, size_t rows_bytes)
 {
-    const size_t most = load > own ? 1520 : 3040;
+    const bool thin = 2.f * p.R * p.ds < 0.5f * p.dx * p.dx * (float)p.N;
+    const size_t most = (thin ? 1216 : 3040) / (load > trace_warps(p.N) ? 2 : 1);
     int l = 1;
     while (l < 8 && load * 2 * l <= most) l *= 2;
     auto fits = [&](int lanes) {
@@ -1083,7 +1090,7 @@ void launch_trace_raster(const float *fields, const int4 *rows, TabEntry *tab, f
     int nwarps = (p.N - 2 + 30) / 31;
     dim3 grd((p.N + kFansPerBlock - 1) / kFansPerBlock, nwarps);
     const size_t sm = (size_t)p.ny * sizeof(int4);
-    const int lpr = lanes_per_ray(load, (size_t)p.N * nwarps, sm);
+    const int lpr = lanes_per_ray(p, load, sm);
     if (lpr > 1) {
         auto wide = [&](auto lp) {
             constexpr int L = decltype(lp)::value;
