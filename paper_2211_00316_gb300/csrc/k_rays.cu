@@ -1196,24 +1196,6 @@ void launch_mask_rows(const int *node2x, int nx, int ny, int4 *rows, cudaStream_
 
 // ---------------------------------------------------------------- a4
 
-// Angular density of every entry (the back-projection's tensor-core operand synthesis forms
-// the same values itself, from the same expression, and does not need this array).
-__global__ void k_dgamma(const TabEntry *__restrict__ tab, float *__restrict__ dg, int N, int X)
-{
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= (size_t)N * X) return;
-    int e = (int)(i / X), k = (int)(i % X);
-    const TabEntry &tp = tab[(size_t)((e + 1) % N) * X + k];
-    const TabEntry &tm = tab[(size_t)((e + N - 1) % N) * X + k];
-    dg[i] = (tp.idk == kUncovered || tm.idk == kUncovered) ? 0.f : dgamma_of(tp.gam, tm.gam);
-}
-
-void launch_dgamma(const TabEntry *tab, float *dg, int N, int X, cudaStream_t s)
-{
-    size_t n = (size_t)N * X;
-    k_dgamma<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tab, dg, N, X);
-}
-
 // ---------------------------------------------------------------- a5
 
 // Phase in cycles: f T - K/4 + 1/8, with f = fhi + flo and the product f T formed
@@ -1694,21 +1676,38 @@ void launch_set_tables(const float *T, const float *a, const float *gam, const u
     k_set_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(T, a, gam, K, tab, n, counters);
 }
 
-__global__ void k_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, size_t n)
+// dg: the angular density (step a4), the values that the operand syntheses form, from the direction angles of
+// the neighbouring transducers. A thread walks eight transducers of a node, so the tables are read 1.25 times
+// for all arrays.
+constexpr int kGetWalk = 8;
+
+__global__ void k_get_tables(const TabEntry *__restrict__ tab, float *T, float *a, float *gam, uint8_t *K, float *dg, int N,
+                             int X)
 {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    TabEntry t = tab[i];
-    bool cov = t.idk != kUncovered;
-    if (T) T[i] = cov ? t.T : 0.f;
-    if (a) a[i] = cov ? t.a : 0.f;
-    if (gam) gam[i] = cov ? t.gam : 0.f;
-    if (K) K[i] = cov ? (uint8_t)(t.idk & 0xffu) : 0;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, e0 = blockIdx.y * kGetWalk, e1 = min(N, e0 + kGetWalk);
+    if (x >= X) return;
+    auto row = [&](int e) { return tab[(size_t)e * X + x]; };
+    TabEntry prev{}, t = row(e0), next{};
+    if (dg) prev = row(e0 > 0 ? e0 - 1 : N - 1);
+    for (int e = e0; e < e1; e++) {
+        if (dg || e + 1 < e1) next = row(e + 1 < N ? e + 1 : 0);
+        const size_t i = (size_t)e * X + x;
+        const bool cov = t.idk != kUncovered;
+        if (T) T[i] = cov ? t.T : 0.f;
+        if (a) a[i] = cov ? t.a : 0.f;
+        if (gam) gam[i] = cov ? t.gam : 0.f;
+        if (K) K[i] = cov ? (uint8_t)(t.idk & 0xffu) : 0;
+        if (dg) dg[i] = (next.idk == kUncovered || prev.idk == kUncovered) ? 0.f : dgamma_of(next.gam, prev.gam);
+        prev = t;
+        t = next;
+    }
 }
 
-void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, size_t n, cudaStream_t s)
+void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, float *dg, int N, int X,
+                       cudaStream_t s)
 {
-    k_get_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tab, T, a, gam, K, n);
+    const dim3 grd((X + 255) / 256, (N + kGetWalk - 1) / kGetWalk);
+    k_get_tables<<<grd, 256, 0, s>>>(tab, T, a, gam, K, dg, N, X);
 }
 
 }  // namespace rbx

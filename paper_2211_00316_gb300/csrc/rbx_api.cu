@@ -591,13 +591,8 @@ rbx_status rbx_get_tables(rbx_job *j, float *T, float *a, float *gam, uint8_t *K
     if (!j) return RBX_EINVAL;
     NEED(j, j->has_tables, RBX_ESTATE, "rbx_get_tables before rbx_trace_rays or rbx_set_tables");
     Workspace &w = j->w;
-    size_t n = (size_t)w.N * w.X;
-    if (T || a || gam || K) {
-        launch_get_tables(w.tab, T, a, gam, K, n, j->stream);
-        LAUNCHED(j, 1);
-    }
-    if (dg) {   // angular density (step a4); the operand syntheses form the same values
-        launch_dgamma(w.tab, dg, w.N, w.X, j->stream);
+    if (T || a || gam || K || dg) {
+        launch_get_tables(w.tab, T, a, gam, K, dg, w.N, w.X, j->stream);
         LAUNCHED(j, 1);
     }
     if (exits)

@@ -172,13 +172,13 @@ void launch_mask_rows(const int *node2x, int nx, int ny, int4 *rows, cudaStream_
 void launch_link_rays(const float *fields, const RayParams &p, const float4 *exits, int maxit, float4 *linked,
                       unsigned long long *counters, bool lossy, bool raw, cudaStream_t s);
 void launch_green_linked(const float4 *linked, int N, double f, double c0, float2 *g, cudaStream_t s);
-void launch_dgamma(const TabEntry *tab, float *dg, int N, int X, cudaStream_t s);
 void launch_direct_green(const float4 *exits, int N, const double *beta, double f, double c0, float2 *g,
                          unsigned long long *counters,
                          cudaStream_t s);
 void launch_set_tables(const float *T, const float *a, const float *gam, const uint8_t *K, TabEntry *tab, size_t n,
                        unsigned long long *counters, cudaStream_t s);
-void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, size_t n, cudaStream_t s);
+void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, float *dg, int N, int X,
+                       cudaStream_t s);
 
 // k_born.cu
 // Born weights v[x] = Upsilon_m dA (m - m_s) (rough part) or Upsilon_m dA dm[x], with
