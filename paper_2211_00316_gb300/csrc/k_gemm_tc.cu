@@ -538,19 +538,33 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// One synthesis tile: 32 nodes x 64 transducers, with a halo row of transducers on each side.
-constexpr int kSynE = 64, kSynThreads = 512;
-constexpr int kSynSlots = (kSynE + 2) * 32;   // slot s holds row (e0 - 1 + s) mod N, nodes x0 .. x0 + 31
+// One synthesis tile: 32 nodes x E transducers (32 or 64), with a halo row of transducers on each side.
+template <int E>
+struct SynTile {
+    static constexpr int THREADS = 8 * E, ROWS = E / 4;   // four transducers a thread
+    static constexpr int SLOTS = (E + 2) * 32;            // slot s holds row (e0 - 1 + s) mod N, nodes x0 .. x0 + 31
+    static constexpr size_t SMEM = 2 * SLOTS * sizeof(TabEntry) + 6 * 32 * (E + 2) * sizeof(__nv_bfloat16);
+};
 
-constexpr size_t SYN_SMEM = 2 * kSynSlots * sizeof(TabEntry) + 6 * 32 * (kSynE + 2) * sizeof(__nv_bfloat16);
+// Transducers of a tile. 64 write a row of a back-projection plane in 128-byte pieces (1024 transducers, 200 x 200,
+// preconditioned adjoint: 435 -> 424 us), but a ragged last tile takes as long as a whole one, so they stay within 6 %
+// of the padding of 32 (80 transducers, 250 x 250: 52.9 us with 32, 59.7 with 64; 215: 118 and 123; 450, 200 x
+// 200, 7 %: 171 and 172; 513, 6 %: 227 and 225); one tile of at most 64 gains nothing (64 transducers, 200 x 200:
+// 37.0 and 37.8).
+int synth_tile(int N)
+{
+    const int p32 = (N + 31) / 32 * 32, p64 = (N + 63) / 64 * 64;
+    return N > 64 && 100 * p64 <= 106 * p32 ? 64 : 32;
+}
 
 // Queue the copies of tile t's table entries into buf (entries past the last node are not
 // copied; the consumer treats them as uncovered).
+template <int E>
 __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab, int N, int X, int XT, int t,
                                                 TabEntry *buf)
 {
-    const int ET = (N + kSynE - 1) / kSynE, x0 = (t / ET) * 32, e0 = (t % ET) * kSynE;
-    for (int idx = threadIdx.x; idx < kSynSlots; idx += kSynThreads) {
+    const int ET = (N + E - 1) / E, x0 = (t / ET) * 32, e0 = (t % ET) * E;
+    for (int idx = threadIdx.x; idx < SynTile<E>::SLOTS; idx += SynTile<E>::THREADS) {
         const int slot = idx >> 5, x = x0 + (idx & 31);
         if (x < X) {
             const int e = (e0 - 1 + slot + N) % N;
@@ -562,9 +576,8 @@ __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab
 // planes [6][Xp][Npad] at [x][e]: u, conj(kappa) u, kappa u (re, im each);
 // u_e[x] = dgamma / (C a) exp(-i 2 pi (f T - K/4 + 1/8)), kappa = exp(i gamma).
 // The angular density dgamma (step a4) is formed here from the direction angles of the
-// neighbouring transducers: a 64-transducer tile reads one halo row on each side (rows wrap
-// around the ring), so the tables are read once more by 1/32 instead of a separate pass, and a
-// row of a back-projection plane is written in 128-byte pieces.
+// neighbouring transducers: a tile reads one halo row on each side (rows wrap around the ring), so
+// the tables are read once more by 1/32 (1/16 in tiles of 32) instead of a separate pass.
 // With FWD the same pass also writes the forward's planes (those of k_synth_fwd_tc, from the
 // same phase): an update reads its tables once for both contractions' operands.
 // Persistent: each block walks the tiles t = blockIdx.x, + gridDim.x, ... (transducer blocks
@@ -572,36 +585,37 @@ __device__ __forceinline__ void synth_tile_load(const TabEntry *__restrict__ tab
 // back-projection planes, 8 % faster than nodes fastest) with
 // two shared-memory buffers, the next tile's entries copied in while the current one is
 // formed and stored, so that table reads stay in flight between the blocks' barriers.
-template <bool FWD>
-__global__ __launch_bounds__(kSynThreads, 2) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
+template <bool FWD, int E>
+__global__ __launch_bounds__(SynTile<E>::THREADS, E == 64 ? 2 : 4) void k_synth_tc(const TabEntry *__restrict__ tab, int N, int X, int Npad,
                                                      size_t pstride, float fhi, float flo, float C,
                                                      __nv_bfloat16 *__restrict__ planes, const float2 *__restrict__ bw,
                                                      int Xpad, size_t fpstride, __nv_bfloat16 *__restrict__ fplanes,
                                                      int XT, int ntiles)
 {
     constexpr int NPL = 6;                                   // back-projection planes
+    constexpr int SLOTS = SynTile<E>::SLOTS, ROWS = SynTile<E>::ROWS;
     extern __shared__ __align__(16) unsigned char syn_smem[];
-    TabEntry *buf = reinterpret_cast<TabEntry *>(syn_smem);  // [2][kSynSlots]
-    // [plane][x][e]: rows of 33 words, the tile transposed and rounded to BF16
-    __nv_bfloat16(*sv)[32][kSynE + 2] = reinterpret_cast<__nv_bfloat16(*)[32][kSynE + 2]>(syn_smem + 2 * kSynSlots * sizeof(TabEntry));
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 16
+    TabEntry *buf = reinterpret_cast<TabEntry *>(syn_smem);  // [2][SLOTS]
+    // [plane][x][e]: rows of E / 2 + 1 words, the tile transposed and rounded to BF16
+    __nv_bfloat16(*sv)[32][E + 2] = reinterpret_cast<__nv_bfloat16(*)[32][E + 2]>(syn_smem + 2 * SLOTS * sizeof(TabEntry));
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x ROWS
     int t = blockIdx.x, b = 0;
-    if (t < ntiles) synth_tile_load(tab, N, X, XT, t, buf);
+    if (t < ntiles) synth_tile_load<E>(tab, N, X, XT, t, buf);
     cp_async_commit();
     for (; t < ntiles; t += gridDim.x, b ^= 1) {
-        if (t + (int)gridDim.x < ntiles) synth_tile_load(tab, N, X, XT, t + gridDim.x, buf + (b ^ 1) * kSynSlots);
+        if (t + (int)gridDim.x < ntiles) synth_tile_load<E>(tab, N, X, XT, t + gridDim.x, buf + (b ^ 1) * SLOTS);
         cp_async_commit();
         cp_async_wait1();   // this thread's copies of tile t have landed
         __syncthreads();    // and every thread's
-        const TabEntry *B = buf + b * kSynSlots;
-        const int ET = (N + kSynE - 1) / kSynE, x0 = (t / ET) * 32, e0 = (t % ET) * kSynE;
+        const TabEntry *B = buf + b * SLOTS;
+        const int ET = (N + E - 1) / E, x0 = (t / ET) * 32, e0 = (t % ET) * E;
         const int x = x0 + tx;
         const bool xin = x < X;
         float2 vv = make_float2(0.f, 0.f);
         if (FWD && xin) vv = bw[x];   // Born weights of node x
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const int q = ty + 16 * k;
+            const int q = ty + ROWS * k;
             float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             float gr = 0.f, gi = 0.f;
             const TabEntry r = B[(q + 1) * 32 + tx];   // row e0 + q
@@ -642,12 +656,12 @@ __global__ __launch_bounds__(kSynThreads, 2) void k_synth_tc(const TabEntry *__r
         const uint32_t *sw = reinterpret_cast<const uint32_t *>(&sv[0][0][0]);
 #pragma unroll
         for (int j = 0; j < 2; j++) {
-            const int item = threadIdx.x + kSynThreads * j, xr = item >> 5, pr = item & 31;
+            const int item = threadIdx.x + SynTile<E>::THREADS * j, xr = item / (E / 2), pr = item % (E / 2);
             if (x0 + xr < X) {
                 const size_t o = (size_t)(x0 + xr) * Npad + e0 + 2 * pr;
 #pragma unroll
                 for (int m = 0; m < NPL; m++)
-                    *reinterpret_cast<uint32_t *>(planes + m * pstride + o) = sw[(m * 32 + xr) * (kSynE / 2 + 1) + pr];
+                    *reinterpret_cast<uint32_t *>(planes + m * pstride + o) = sw[(m * 32 + xr) * (E / 2 + 1) + pr];
             }
         }
     }
@@ -726,16 +740,17 @@ bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, 
 
 // ---------------------------------------------------------------- API used by rbx_api.cu
 
-// Shared memory and persistent grid of k_synth_tc<FWD>, for the current device: the opt-in above 48 KB
+// Shared memory and persistent grid of k_synth_tc<FWD, E>, for the current device: the opt-in above 48 KB
 // belongs to a device's context, so every job makes it for the one it lives on.
-template <bool FWD>
+template <bool FWD, int E>
 static bool synth_setup(TcPlanes &p)
 {
+    constexpr size_t SMEM = SynTile<E>::SMEM;
     int dev = 0, sms = 0, per_sm = 0;
-    if (cudaFuncSetAttribute(k_synth_tc<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SYN_SMEM) != cudaSuccess ||
+    if (cudaFuncSetAttribute(k_synth_tc<FWD, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM) != cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD>, kSynThreads, SYN_SMEM) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_tc<FWD, E>, SynTile<E>::THREADS, SMEM) != cudaSuccess)
         return false;
     p.syn_blocks[FWD] = sms * std::max(per_sm, 1);
     return true;
@@ -790,7 +805,8 @@ bool tc_setup(TcPlanes &p, int N, int X, unsigned *err, cudaStream_t st)
          cudaFuncSetAttribute(k_forward_tc_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) ==
              cudaSuccess &&
          cudaFuncSetAttribute(k_backproject_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B_SMEM) == cudaSuccess &&
-         synth_setup<false>(p) && synth_setup<true>(p);
+         (synth_tile(N) == 64 ? synth_setup<false, 64>(p) && synth_setup<true, 64>(p)
+                              : synth_setup<false, 32>(p) && synth_setup<true, 32>(p));
     p.ready = ok;
     return ok;
 }
@@ -970,13 +986,13 @@ int launch_forward_tc(TcPlanes &p, float2 *part, cudaStream_t s)
     return p.fwd_splits;
 }
 
-template <bool FWD>
+template <bool FWD, int E>
 static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
     const float fhi = (float)f, flo = (float)(f - (double)fhi);
-    const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + kSynE - 1) / kSynE);
+    const int XT = (p.X + 31) / 32, ntiles = XT * ((p.N + E - 1) / E);
     const int grd = std::min(p.syn_blocks[FWD], ntiles);
-    k_synth_tc<FWD><<<grd, kSynThreads, SYN_SMEM, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
+    k_synth_tc<FWD, E><<<grd, SynTile<E>::THREADS, SynTile<E>::SMEM, s>>>(tab, p.N, p.X, p.Npad, p.bp_pstride, fhi, flo, green_const_tc(f, c0),
                                                   static_cast<__nv_bfloat16 *>(p.bplanes), v, FWD ? p.Xpad : 0,
                                                   FWD ? p.fwd_pstride : 0,
                                                   FWD ? static_cast<__nv_bfloat16 *>(p.fplanes) : nullptr, XT, ntiles);
@@ -984,12 +1000,18 @@ static void synth_launch(TcPlanes &p, const TabEntry *tab, const float2 *v, doub
 
 void launch_synth_bp_tc(TcPlanes &p, const TabEntry *tab, double f, double c0, cudaStream_t s)
 {
-    synth_launch<false>(p, tab, nullptr, f, c0, s);
+    if (synth_tile(p.N) == 64)
+        synth_launch<false, 64>(p, tab, nullptr, f, c0, s);
+    else
+        synth_launch<false, 32>(p, tab, nullptr, f, c0, s);
 }
 
 void launch_synth_both_tc(TcPlanes &p, const TabEntry *tab, const float2 *v, double f, double c0, cudaStream_t s)
 {
-    synth_launch<true>(p, tab, v, f, c0, s);
+    if (synth_tile(p.N) == 64)
+        synth_launch<true, 64>(p, tab, v, f, c0, s);
+    else
+        synth_launch<true, 32>(p, tab, v, f, c0, s);
 }
 
 // One thread waits, with the bound every tensor-core kernel uses, on an mbarrier that nothing
