@@ -175,6 +175,8 @@ void launch_green_linked(const float4 *linked, int N, double f, double c0, float
 void launch_direct_green(const float4 *exits, int N, const double *beta, double f, double c0, float2 *g,
                          unsigned long long *counters,
                          cudaStream_t s);
+
+// k_tables.cu
 void launch_set_tables(const float *T, const float *a, const float *gam, const uint8_t *K, TabEntry *tab, size_t n,
                        unsigned long long *counters, cudaStream_t s);
 void launch_get_tables(const TabEntry *tab, float *T, float *a, float *gam, uint8_t *K, float *dg, int N, int X,
