@@ -45,6 +45,7 @@ struct rbx_job {
     cudaEvent_t ev_in_free = nullptr, ev_in_ready = nullptr;
     long long launches = 0;
     bool unread = false;       // a call without a status of its own may have set w.err (rbx_synchronize reads it)
+    bool captured = false;     // such a call may run again at any time, from a graph of the caller's
     int load_dev = -1;         // device whose g_load counts this job's trace (set with the geometry)
     bool waits = false;        // inside a call that traces and waits for the update (Waiting)
 };
@@ -237,7 +238,7 @@ const char *rbx_last_error(const rbx_job *j) { return j ? j->err.c_str() : "null
 rbx_status rbx_synchronize(rbx_job *j)
 {
     if (!j) return RBX_EINVAL;
-    if (!j->unread) {
+    if (!j->unread && !j->captured) {
         CUDA_TRY(j, cudaStreamSynchronize(j->stream));
         return RBX_OK;
     }
@@ -256,7 +257,6 @@ rbx_status rbx_selftest_job_timeout(rbx_job *j)
     NEED(j, j->has_geom, RBX_ESTATE, "rbx_selftest_job_timeout before rbx_set_geometry");
     launch_wait_selftest(j->w.err, j->stream);
     LAUNCHED(j, 1);
-    j->unread = true;
     return RBX_OK;
 }
 
@@ -306,7 +306,7 @@ rbx_status rbx_set_geometry(rbx_job *j, const rbx_geometry *geom, const double *
     drop_load(j);
     free_ws(j->w, j->stream);
     keep_pool_memory();
-    j->has_geom = j->has_tables = j->ns_valid = j->lossy = j->raw = j->unread = false;
+    j->has_geom = j->has_tables = j->ns_valid = j->lossy = j->raw = j->unread = j->captured = false;
     j->link_iters = 0;
     Workspace &w = j->w;
     w.N = g.n_xducers;
@@ -613,6 +613,15 @@ rbx_status rbx_direct_green(rbx_job *j, double f, void *g_dev)
     return direct_green(j, f, static_cast<float2 *>(g_dev));
 }
 
+// Marks a call that has no status of its own to report a time-out with.
+static void mark_unread(rbx_job *j)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    j->unread = true;
+    if (cudaStreamIsCapturing(j->stream, &st) != cudaSuccess) cudaGetLastError();   // the legacy stream during a capture
+    if (st != cudaStreamCaptureStatusNone) j->captured = true;
+}
+
 // The operands of an FP32 or split BF16 job's contractions.
 static F32Planes &parts_of(rbx_job *j) { return j->g.precision == RBX_FP32 ? j->w.f32 : j->w.split; }
 
@@ -664,7 +673,7 @@ rbx_status rbx_forward(rbx_job *j, double f, const float *dm_dev, void *D_dev)
     Workspace &w = j->w;
     launch_born_weights_dm(dm_dev, w.c, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j), w.v, j->stream);
     LAUNCHED(j, 1);
-    j->unread = true;
+    mark_unread(j);
     rbx_status st = forward_core(j, f, false);
     if (st) return st;
     CUDA_TRY(j, cudaMemcpyAsync(D_dev, w.D, sizeof(float2) * (size_t)w.N * w.N, cudaMemcpyDeviceToDevice, j->stream));
@@ -686,7 +695,7 @@ rbx_status rbx_predict(rbx_job *j, double f, void *g_dev)
     } else {
         launch_born_weights_rough(w.c, w.ns64, w.idx, w.X, f, j->g.dx * j->g.dx, lossy_of(j), w.v, j->stream);
         LAUNCHED(j, 1);
-        j->unread = true;
+        mark_unread(j);
         if ((st = forward_core(j, f, false))) return st;
     }
     launch_add_offdiag(w.gdir, w.D, w.N, static_cast<float2 *>(g_dev), j->stream);
@@ -701,7 +710,7 @@ rbx_status rbx_adjoint(rbx_job *j, double f, const void *R_dev, void *out_dev, i
     NEED(j, !bad_freq(f), RBX_EINVAL, "frequency must be finite and > 0");
     Workspace &w = j->w;
     const float2 *R = static_cast<const float2 *>(R_dev);
-    j->unread = true;
+    mark_unread(j);
     if (preconditioned && j->g.precision == RBX_BF16) {
         launch_symmetrize(R, w.N, w.Rs, j->stream);
         launch_synth_bp_tc(w.tc, w.tab, f, j->g.c0, j->stream);

@@ -65,6 +65,7 @@ int cudaMemcpyAsync(void *to, const void *from, size_t n, int kind, void *s)
 }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int t, size_t m, unsigned fl) { *n = 2; return 0; }
 int cudaStreamSynchronize(void *s) { return 0; }
+int cudaStreamIsCapturing(void *s, int *status) { *status = 0; return 0; }
 int cudaEventCreate(void **e) { *e = (void *)16; return 0; }
 int cudaEventDestroy(void *e) { return 0; }
 int cudaEventRecord(void *e, void *s) { return 0; }

@@ -62,3 +62,32 @@ def test_reported_once(precision, n, lossy):
     job.update_frequency_async(F, DF, R, 3)
     job.get_stats(3)
     job.close()
+
+
+def test_reported_from_a_graph():
+    """A forward captured into the caller's graph runs again without a call of the library."""
+    n = 48
+    w = P.custom(n, 64, 1e-3, 28e-3, kind="discs", freqs=(F,))
+    dm = torch.full((64, 64), 1e-9, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        job = rbx.Job(stream)
+        job.set_geometry(w.geom, precision=rbx.RBX_FP32)
+        job.set_model(torch.tensor(w.c_init, dtype=torch.float32, device="cuda"))
+        job.trace_rays(F)
+        want = job.forward(F, dm).clone()
+        job.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            out = job.forward(F, dm)
+        job.sync()
+        job.selftest_timeout()
+        graph.replay()
+        assert reported(job.sync)
+        assert bool(torch.isnan(torch.view_as_real(out)).any(-1).all())
+        graph.replay()
+        job.sync()
+        assert bool((out == want).all())
+        del graph
+        job.close()
