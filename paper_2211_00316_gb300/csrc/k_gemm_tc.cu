@@ -741,7 +741,7 @@ bool encode_tiled(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims, 
 // ---------------------------------------------------------------- API used by rbx_api.cu
 
 // Shared memory and persistent grid of k_synth_tc<FWD, E>, for the current device: the opt-in above 48 KB
-// belongs to a device's context, so every job makes it for the one it lives on.
+// belongs to a device, so every job makes it for the one it lives on.
 template <bool FWD, int E>
 static bool synth_setup(TcPlanes &p)
 {
