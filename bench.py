@@ -93,8 +93,8 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none
     #     -k regex:k_trace_raster -s 3 -c 1 --csv   (k_synth_tc: -k regex:k_synth_tc -s 6 -c 1)
     #     python bench.py --steps 2 --warmup 1 --no-cpu-baseline --no-e2e --no-forms   (1 pass)
-    ("precision_ring1024", "trace"): {"bytes": 2.804101120e9 + 2.557893632e9, "src": "ac7daf1ce0a9"},
-    ("precision_ring1024", "synth"): {"bytes": 2.494324992e9 + 3.066876416e9, "src": "7354497b5d3a"},
+    ("precision_ring1024", "trace"): {"bytes": 2.802663424e9 + 2.558331392e9, "src": "6f1b0f640848"},
+    ("precision_ring1024", "synth"): {"bytes": 2.494389504e9 + 3.066620416e9, "src": "5ba71c3f4af4"},
 }
 
 
