@@ -93,8 +93,8 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none
     #     -k regex:k_trace_raster -s 3 -c 1 --csv   (k_synth_tc: -k regex:k_synth_tc -s 6 -c 1)
     #     python bench.py --steps 2 --warmup 1 --no-cpu-baseline --no-e2e --no-forms   (1 pass)
-    ("precision_ring1024", "trace"): {"bytes": 2.802663424e9 + 2.558331392e9, "src": "6f1b0f640848"},
-    ("precision_ring1024", "synth"): {"bytes": 2.494389504e9 + 3.066620416e9, "src": "5ba71c3f4af4"},
+    ("precision_ring1024", "trace"): {"bytes": 2.802563840e9 + 2.557772032e9, "src": "6f1b0f640848"},
+    ("precision_ring1024", "synth"): {"bytes": 2.494356480e9 + 3.066587392e9, "src": "98a2d783a166"},
 }
 
 
